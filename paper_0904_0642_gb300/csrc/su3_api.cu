@@ -415,6 +415,9 @@ static void fill_desc(Chain &ch, int tile) {
 
   d.beta_f = (float)c.beta;
   d.beta_d = c.beta;
+  int e = 1 << 20;
+  d.inv_beta_m = (int64_t)std::ldexp(c.beta > 0.0 && std::isfinite(1.5 / c.beta) ? std::frexp(1.5 / c.beta, &e) : 0.5, 60);
+  d.inv_beta_e = e;
   const double b1 = c.beta1 >= 0.0 ? c.beta1 : c.beta;
   d.weighted = (d.nlayers == 2 && b1 != c.beta) ? 1 : 0;
   d.beta1_f = (float)b1;
@@ -440,6 +443,17 @@ struct Engine {
   // the tick kernel's torus form: 0 none, 1 the torus form, 2 its form for several chains
   int torus_form() const { return torus_all ? (chains.size() > 1 ? 2 : 1) : 0; }
   int torus_form_built = 0;   // the form the captured graph launches
+  bool coop = false;          // FP64, too few links to fill the GPU: eight lanes per link
+  int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
+  int kernel_variant() const { return coop ? 1 : variant; }
+  // The links of one update phase of an FP64 chain that may take eight lanes
+  // per link (others: more than any limit).
+  long long coop_sites(const Chain &ch) const {
+    if (storage != SU3_FP64_18) return 1ll << 40;
+    long long n = ch.cfg.boundary == SU3_DLT ? 2 : 1;
+    for (int i = 0; i < ch.cfg.D; ++i) n *= ch.cfg.dims[i];
+    return n / 2;
+  }
   cudaStream_t stream = nullptr;
   std::vector<Chain> chains;
   // device mirrors
@@ -648,10 +662,13 @@ struct Engine {
       ch.own_links = true;
       ch.bytes_total += ch.link_bytes;
     }
-    fill_desc(ch, 32);  // partials sized for the narrowest tile
+    // partials and action slots sized for the narrowest tile
+    const bool coop = coop_sites(ch) <= kCoopSites;
+    const int narrow = coop ? 32 / kCoopLanes : 32;
+    fill_desc(ch, narrow);
     size_t ntiles = (size_t)ch.desc.nlayers * ch.desc.tiles_per_layer;
     if (ch.sub) {
-      fill_plain(ch, 32);
+      fill_plain(ch, narrow);
       ntiles = std::max(ntiles, (size_t)ch.pdesc.nlayers * ch.pdesc.tiles_per_layer);
     }
     const size_t npart = ntiles * kPartVals;
@@ -664,7 +681,7 @@ struct Engine {
       return fail(SU3_ENOMEM, "scratch allocation failed");
     }
     ch.bytes_total += npart * sizeof(double) + nres * sizeof(double) + 16;
-    ch.n_action_slots = ch.desc.nlayers * ch.desc.nb * ((ch.desc.Vn + 31) / 32);
+    ch.n_action_slots = ch.desc.nlayers * ch.desc.nb * ((ch.desc.Vn + narrow - 1) / narrow);
     if (cudaMalloc(&ch.action_slots, (size_t)ch.n_action_slots * sizeof(double)) != cudaSuccess) {
       free_chain(ch);
       return fail(SU3_ENOMEM, "action bookkeeping allocation failed");
@@ -715,8 +732,18 @@ struct Engine {
   su3_status rebuild() {
     const int old_tiles = total_tiles;
     int tiles = 0;
+    long long sites = 0;
+    bool weighted = false;
     for (auto &ch : chains) {
       fill_desc(ch, block);
+      sites += coop_sites(ch);
+      weighted = weighted || ch.desc.weighted;
+    }
+    const bool cp = sites <= kCoopSites && !weighted;
+    if (cp != coop) drop_graph();
+    coop = cp;
+    for (auto &ch : chains) {
+      fill_desc(ch, tile());
       ch.desc.tile_base = tiles;
       tiles += ch.desc.nlayers * ch.desc.tiles_per_layer;
     }
@@ -727,7 +754,7 @@ struct Engine {
       w = w || ch.desc.weighted;
       sb = sb || ch.sub;
       if (ch.sub) {
-        fill_plain(ch, block);
+        fill_plain(ch, tile());
         CU(cudaMemcpyAsync(ch.d_pdesc, &ch.pdesc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
       }
     }
@@ -773,7 +800,7 @@ struct Engine {
     EngineHeader h{};
     h.nchains = (int32_t)chains.size();
     h.total_tiles = tiles;
-    h.tile = block;
+    h.tile = tile();
     h.parity = 0;
     h.done = 0;
     h.n_meas = 0;
@@ -848,12 +875,12 @@ struct Engine {
 
   // One tick, and for a divided chain the halo refresh of what it changed.
   su3_status one_tick(int grid) {
-    cudaError_t e = launch_tick(storage, variant, weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
+    cudaError_t e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
     if (e != cudaSuccess && pdl) {  // not offered here: plain launches from now on
       cudaGetLastError();
       pdl = false;
       drop_graph();
-      e = launch_tick(storage, variant, weighted_any, sub_any, torus_form(), args(), grid, block, stream, false);
+      e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, false);
     }
     CU(e);
     if (sub_any) CU(halo_refresh(d_desc, d_state, 0));
@@ -912,7 +939,7 @@ struct Engine {
     cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     for (int i = 0; i < kGraphTicks && e == cudaSuccess; ++i) {
-      e = launch_tick(storage, variant, weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
+      e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
       if (e == cudaSuccess && sub_any) e = halo_refresh(d_desc, d_state, 0);
     }
     cudaError_t e2 = cudaStreamEndCapture(stream, &g);
@@ -1522,7 +1549,7 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     for (int t : cand_t) {
       if (t > tick_max_threads(e.storage, v)) continue;
       int occ = 0;
-      if (tick_occupancy(e.storage, v, e.weighted_any, e.sub_any, e.torus_form(), t, &occ) != cudaSuccess || occ < 1) continue;
+      if (tick_occupancy(e.storage, e.coop ? 1 : v, e.weighted_any, e.sub_any, e.torus_form(), t, &occ) != cudaSuccess || occ < 1) continue;
       // 0 = one CTA per tile, then persistent grids of 1, 2, 4, ..., occ CTAs per SM
       for (int c = 0; c <= occ && st == SU3_OK; c = (c == 0) ? 1 : ((c < occ && 2 * c > occ) ? occ : 2 * c)) {
         if ((st = e.set_launch(v, t, c)) != SU3_OK) break;

@@ -38,6 +38,14 @@ constexpr float kAlphaFp64 = 32.0f;
 // would be divided by alpha).
 constexpr float kAlphaAccurateLog = 2.0f;
 
+// FP64 chains of one coupling with at most kCoopSites links per update phase
+// take eight lanes per link (update_site_coop): a tile then holds an eighth
+// of a CTA's threads.  One thread per link takes 35 us per phase for any
+// lattice below one wave (38912 links at 8 warps per SM); eight lanes take
+// 15 us per wave of 4864 links, so the line lies at two waves, rounded down.
+constexpr int kCoopLanes = 8;
+constexpr int kCoopSites = 8192;
+
 // Results per measurement slot: [total, space, time, poly_re, poly_im].
 constexpr int kMeasVals = 5;
 // Partial sums per tile in a measurement: [space, time, poly_re, poly_im].
@@ -94,6 +102,10 @@ struct ChainDesc {
   int32_t weighted;
   float beta1_f;
   double beta1_d;
+  // 3 / (2 beta) = inv_beta_m 2^-60 2^inv_beta_e, the mantissa in [1/2, 1)
+  // (beta = 0: an exponent beyond any acceptance): the fixed-point draw
+  int64_t inv_beta_m;
+  int32_t inv_beta_e;
   double action_factor;      // booked dS per unit change of Re Tr(U A): -beta/3, or -1/3 when weighted
 };
 

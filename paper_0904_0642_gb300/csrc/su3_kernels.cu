@@ -17,6 +17,7 @@
 #include <cuda.h>  // CUcontext / CUresult for the two driver calls reached through the runtime
 
 #include "su3_device.cuh"
+#include "su3_fixed.cuh"
 #include "su3_launch.h"
 
 namespace su3g {
@@ -371,6 +372,422 @@ __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, 
   S::store(pu, Vh, ju, U);
 }
 
+
+// ------------------------------------------------------------------ FP64 link update in fixed point
+// The one-coupling FP64 update with its linear algebra (staples, projections,
+// rotations) in the integers of su3_fixed.cuh.
+
+// Row `row` of a stored FP64 link in fixed point.
+__device__ __forceinline__ void load_row_f(const StoreF64x18::Vec *plane, int Vh, int jj, int row, Fc (&r)[3],
+                                           FxRange &rg) {
+  if (!in_bounds(jj, Vh, kBoundsIndex)) {
+    r[0] = r[1] = r[2] = Fc{{0, 0}, {0, 0}};
+    return;
+  }
+  const double2 *p = plane + jj + 3 * row * Vh;
+  const double2 q0 = __ldg(p), q1 = __ldg(p + Vh), q2 = __ldg(p + 2 * Vh);
+  r[0] = fc_of(q0.x, q0.y, rg);
+  r[1] = fc_of(q1.x, q1.y, rg);
+  r[2] = fc_of(q2.x, q2.y, rg);
+}
+
+__device__ __forceinline__ void load_f(const StoreF64x18::Vec *plane, int Vh, int jj, FM3 &m, FxRange &rg) {
+#pragma unroll
+  for (int i = 0; i < 3; ++i) load_row_f(plane, Vh, jj, i, m.e[i], rg);
+}
+
+// The draw of one subgroup in double, out of line: proposals with too few
+// digits in fixed point only (propose_fx).
+struct DrawD {
+  double x[4];
+  uint32_t nprop;
+  bool accepted;
+};
+__device__ __noinline__ DrawD su2_draw_general(double alpha, int hits, uint2 key, uint32_t c0, uint32_t c1,
+                                               uint32_t tag) {
+  DrawD r;
+  r.nprop = 0;
+  r.accepted = su2_draw_d(alpha, hits, key, c0, c1, tag, r.x, r.nprop);
+  return r;
+}
+
+// The three links of one staple (staple_f): rows 0, 1 of X, all of Y and G.
+// t counts the 2 (D - 1) staples: the upper ones of the other directions in
+// order, then the lower ones.
+template <bool SUB>
+__device__ __forceinline__ void staple_fixed(const ChainDesc &d, const SiteGeo &g, int colour, int mu, int t, int sp,
+                                             int lp, FSum &A, FxRange &rg) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh, oc = colour ^ 1, layer = g.layer;
+  const bool up = t < d.D - 1;
+  int nu = up ? t : t - (d.D - 1);
+  nu += nu >= mu ? 1 : 0;
+  int offn, fln, offm, flm;
+  const int xnu = sel(g.x, nu);
+  step_fwd(d, xnu, nu, offn, fln);
+  step_bwd(d, xnu, nu, offm, flm);
+  const int sn = g.s + offn, ln = lflip<SUB>(d, layer, fln);  // x + nu
+  const int sm = g.s + offm, lm = lflip<SUB>(d, layer, flm);  // x - nu
+  const int spm = sp + offm, lpm = lflip<SUB>(d, lp, flm);    // x + mu - nu
+  const S::Vec *py = up ? plane_ptr<S>(d, ln, oc, mu) : plane_ptr<S>(d, lpm, colour, nu);
+  const S::Vec *px = up ? plane_ptr<S>(d, layer, colour, nu) : plane_ptr<S>(d, lm, oc, mu);
+  const S::Vec *pg = up ? plane_ptr<S>(d, lp, oc, nu) : plane_ptr<S>(d, lm, oc, nu);
+  const int jy = (up ? sn : spm) >> 1, jx = (up ? g.s : sm) >> 1, jg = (up ? sp : sm) >> 1;
+  FM3 Y, G;
+  Fc X[2][3];
+  load_f(py, Vh, jy, Y, rg);
+  load_row_f(px, Vh, jx, 0, X[0], rg);
+  load_row_f(px, Vh, jx, 1, X[1], rg);
+  load_f(pg, Vh, jg, G, rg);
+  staple_f(A, X, Y, G, up, rg);
+}
+
+__device__ __forceinline__ Direction direction_of(uint2 w) {
+  Direction r;
+  int64_t c, s;
+  trig_fx(w.y, 1, c, s);
+  r.st = sin_theta_fx(w.x);
+  r.ct = cos_theta_fx(w.x);
+  r.cphi = fx_split(c);
+  r.sphi = fx_split(s);
+  return r;
+}
+
+// The proposals h, h + 1, ... of a subgroup until one is not rejected.
+__device__ __forceinline__ ProposalStatus propose_until(int &h, int hits, uint2 key, uint32_t c0, uint32_t c1,
+                                                        uint32_t tag, const FxNorm &n, const InvBeta &ib,
+                                                        Proposal &p) {
+  ProposalStatus st = kRejected;
+#pragma unroll 1
+  for (; h < hits && st == kRejected; ++h) {
+    const uint4 w = philox4x32_10(make_uint4(c0, c1, tag | (uint32_t)h, kPurposeHeatbath), key);
+    int64_t cs, sn;
+    trig_fx(2u * w.y + 1u, 0, cs, sn);
+    st = propose_fx(radius_fx(neg_log_fx(w.x), neg_log_fx(w.z), cs), square_fx(w.w), n, ib, p);
+  }
+  return st;
+}
+
+__device__ __forceinline__ void swap_rows(Fc (&a)[3], Fc (&b)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const Fc t = a[k];
+    a[k] = b[k];
+    b[k] = t;
+  }
+}
+
+// cm_update with U in units 2^-60 and the staple sum in units 2^-56, all in
+// fixed point.  The loop over the subgroups stays a loop (its body once in
+// the instruction cache): the rows of U and the columns of A of the current
+// subgroup are swapped into places 0 and 1.
+// dretr2: the change of Re Tr(U A) / 2 in units 2^-57.
+__device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, const FM3 &A, uint32_t c0, uint32_t c1,
+                                                int colour, int mu, uint32_t &nprop, uint32_t &nacc,
+                                                int64_t &dretr2) {
+  const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
+  const InvBeta ib = {d.inv_beta_m, d.inv_beta_e};
+  const int hits = d.hits;
+  Fc(&u0)[3] = U.e[0], (&u1)[3] = U.e[1], (&u2)[3] = U.e[2];
+  Fc a0[3], a1[3], a2[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    a0[k] = A.e[k][0];
+    a1[k] = A.e[k][1];
+    a2[k] = A.e[k][2];
+  }
+  dretr2 = 0;
+#pragma unroll 1
+  for (int sg = 0; sg < 3; ++sg) {
+    const uint32_t tag = heatbath_tag(colour, mu, sg);
+    FxAcc s[4] = {{0, kHalf60}, {0, kHalf60}, {0, kHalf60}, {0, kHalf60}};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) project_k_f(s, u0[k], u1[k], a0[k], a1[k]);
+    const int64_t a[4] = {fold60(s[0]), fold60(s[1]), fold60(s[2]), fold60(s[3])};  // 2^-56, and the factor 1/2
+    FxNorm n;
+    if (norm_fx(a, n)) {
+      Proposal p;
+      int h = 0;
+      const ProposalStatus st = propose_until(h, hits, key, c0, c1, tag, n, ib, p);
+      Fx x[4];
+      bool accepted = st == kAccepted;
+      if (accepted) {
+        direction_fx(p, direction_of(direction_words(key, c0, c1, tag)), x);
+      } else if (st == kInDouble) {
+        const DrawD r = su2_draw_general(2.0 * d.beta_d / 3.0 * dbl_of(n.kappa, 57 + n.s), hits, key, c0, c1, tag);
+        h = (int)r.nprop;
+        accepted = r.accepted;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = fx_of(r.x[q]);
+      }
+      nprop += (uint32_t)h;
+      if (accepted) {
+        ++nacc;
+        // k x0 - a0 with k = kappa 2^(3 - s)
+        dretr2 += (fx_mul(fx_split(n.kappa), x[0]) >> n.s) - a[0];
+        Fx r[4], rn[4];
+        quat_fx(x, n.v, r);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rn[q] = fx_neg(r[q]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) rotate_col_f(u0[k], u1[k], r, rn);
+      }
+    }
+    // subgroups (0,1), (0,2), (1,2)
+    if (sg == 0) {
+      swap_rows(u1, u2);
+      swap_rows(a1, a2);
+    } else if (sg == 1) {  // places hold rows 0, 2, 1
+      swap_rows(u0, u2);   // 1, 2, 0
+      swap_rows(a0, a2);
+    }
+  }
+}
+
+// The counts and the action change of one update.
+struct UpdateCount {
+  uint32_t nprop, nacc;
+  double dretr;
+};
+
+// The double-precision update of one site, out of line: links outside the
+// fixed-point range only.
+template <bool SUB>
+__device__ __noinline__ UpdateCount update_site_f64_general(const ChainDesc *d, uint32_t sweep, int colour, int mu,
+                                                            int layer, int jj) {
+  UpdateCount u = {0, 0, 0.0};
+  if constexpr (SUB)
+    update_site<StoreF64x18, false, false, true>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
+  else
+    update_site_lean<StoreF64x18, false>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
+  return u;
+}
+
+// The change of Re Tr(U A) of one update: in units 2^-49 (sums over a warp are
+// exact), and in double where the double-precision form ran.
+struct ActionChange {
+  int64_t v;
+  double general;
+};
+
+// One thread per link.
+template <bool SUB>
+__device__ __forceinline__ void update_site_fixed(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
+                                                  int jj, uint32_t &nprop, uint32_t &nacc, ActionChange &dr) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh;
+  const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
+  const int js = g.s >> 1;
+  int offp, flp;
+  step_fwd(d, sel(g.x, mu), mu, offp, flp);
+  const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
+  FSum A = {};
+  FxRange rg;
+  // one staple at a time: its instructions once, not six times, in the
+  // instruction cache
+#pragma unroll 1
+  for (int t = 0; t < 2 * (d.D - 1); ++t) staple_fixed<SUB>(d, g, colour, mu, t, sp, lp, A, rg);
+  S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
+  FM3 U;
+  load_f(pu, Vh, js, U, rg);
+  if (!rg.ok()) {
+    const UpdateCount u = update_site_f64_general<SUB>(&d, sweep, colour, mu, layer, jj);
+    nprop += u.nprop;
+    nacc += u.nacc;
+    dr.general = u.dretr;
+    return;
+  }
+  const uint32_t before = nacc;
+  int64_t half;
+  cm_update_fixed(d, U, factor56(A), site_key<SUB>(d, g), sweep, colour, mu, nprop, nacc, half);
+  dr.v = half >> 7;
+  // a link none of whose subgroups accepted keeps its bits
+  if (nacc != before && in_bounds(js, Vh, kBoundsIndex)) {
+    // the rows lie in the order 1, 2, 0 after the last subgroup
+    S::Vec *p = pu + js;
+#pragma unroll
+    for (int q = 0; q < 9; ++q) {
+      const Fc e = U.e[(q / 3 + 2) % 3][q % 3];
+      p[q * Vh] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
+    }
+  }
+}
+
+__device__ __forceinline__ Fx shfl_fx(const Fx &a, int src) {
+  return {__shfl_sync(0xffffffffu, a.h, src), __shfl_sync(0xffffffffu, a.l, src)};
+}
+__device__ __forceinline__ int64_t shfl_ll(int64_t a, int src) { return __shfl_sync(0xffffffffu, (long long)a, src); }
+__device__ __forceinline__ int64_t shfl_xor_ll(int64_t a, int m) {
+  return __shfl_xor_sync(0xffffffffu, (long long)a, m);
+}
+
+// Eight lanes per link, for lattices that do not fill the GPU with one
+// thread per link (an update is then one thread's chain of ~20000 dependent
+// instructions): each lane forms one staple (integer sums: the same total in
+// any order), the logarithms, angles and directions of the three subgroups'
+// first proposals take one pass over the lanes, and lanes 0..2 hold one
+// column of U each in the projections and rotations.  Results are bitwise
+// those of update_site_fixed.  Called by whole warps; lanes without a link
+// (valid false) run along on a repeated one.
+template <bool SUB>
+__device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
+                                                 int jj, bool valid, uint32_t &nprop, uint32_t &nacc,
+                                                 ActionChange &dr) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh;
+  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
+  const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
+  const int js = g.s >> 1;
+  int offp, flp;
+  step_fwd(d, sel(g.x, mu), mu, offp, flp);
+  const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
+  const uint32_t c0 = site_key<SUB>(d, g);
+  const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
+  const InvBeta ib = {d.inv_beta_m, d.inv_beta_e};
+  const int hits = d.hits;
+
+  // The first proposals and directions: a block of random words per lane
+  // (lanes 0..2: the proposals, 3 and 4: the direction blocks of subgroups 0,
+  // 1 and of subgroup 2), then lanes 0..2 take ln u1 and the proposal's angle,
+  // lanes 3..5 ln u3 and the direction.
+  const int sub = l8 < 3 ? l8 : (l8 < 6 ? l8 - 3 : 0);
+  const uint32_t btag = heatbath_tag(colour, mu, l8 < 3 ? l8 : (l8 == 4 ? 2 : 0)) | (l8 < 3 ? 0u : kHitDirection);
+  const uint4 w = philox4x32_10(make_uint4(c0, sweep, btag, kPurposeHeatbath), key);
+  const int dl = base + (sub == 2 ? 4 : 3);
+  const uint32_t d0 = __shfl_sync(0xffffffffu, w.x, dl), d1 = __shfl_sync(0xffffffffu, w.y, dl);
+  const uint32_t d2 = __shfl_sync(0xffffffffu, w.z, dl), d3 = __shfl_sync(0xffffffffu, w.w, dl);
+  const uint32_t w3rd = __shfl_sync(0xffffffffu, w.z, base + sub);
+  const uint32_t wth = sub == 1 ? d2 : d0, wphi = sub == 1 ? d3 : d1;
+  const bool prop = l8 < 3;
+  int64_t cs, sn;
+  trig_fx(prop ? 2u * w.y + 1u : wphi, prop ? 0 : 1, cs, sn);
+  const int64_t nl = neg_log_fx(prop ? w.x : w3rd);
+  const int64_t L1 = radius_fx(nl, shfl_ll(nl, base + (l8 + 3 & 7)), cs), u41 = square_fx(w.w);
+  const Fx st1 = sin_theta_fx(wth), ct1 = cos_theta_fx(wth), cp1 = fx_split(cs), sp1 = fx_split(sn);
+
+  // staples
+  FSum A = {};
+  FxRange rg;
+  const int ns = 2 * (d.D - 1);
+  staple_fixed<SUB>(d, g, colour, mu, l8 < ns ? l8 : 0, sp, lp, A, rg);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      int64_t re = l8 < ns ? A.re[i][j] : 0, im = l8 < ns ? A.im[i][j] : 0;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        re += shfl_xor_ll(re, o);
+        im += shfl_xor_ll(im, o);
+      }
+      A.re[i][j] = re;
+      A.im[i][j] = im;
+    }
+  // column c of U, row c of A
+  const int c = l8 & 3, cc = c < 3 ? c : 0;
+  S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
+  Fc u[3], a[3];
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    double2 q = make_double2(0.0, 0.0);
+    if (in_bounds(js, Vh, kBoundsIndex)) q = __ldg(pu + js + (3 * r + cc) * Vh);
+    u[r] = fc_of(q.x, q.y, rg);
+    const int64_t re = cc == 0 ? A.re[0][r] : (cc == 1 ? A.re[1][r] : A.re[2][r]);
+    const int64_t im = cc == 0 ? A.im[0][r] : (cc == 1 ? A.im[1][r] : A.im[2][r]);
+    a[r] = {fx_split((re + 8) >> 4), fx_split((im + 8) >> 4)};
+    if (c == 3) u[r] = a[r] = Fc{{0, 0}, {0, 0}};
+  }
+  const bool bad = (__ballot_sync(0xffffffffu, !rg.ok()) >> base & 0xffu) != 0;
+
+  uint32_t np = 0, na = 0;
+  int64_t half = 0;
+#pragma unroll 1
+  for (int sg = 0; sg < 3; ++sg) {
+    // the projection: this lane's k, then the sum over the lanes (the rounding
+    // constant enters once)
+    const int64_t round = c == 0 ? kHalf60 : 0;
+    FxAcc s[4] = {{0, round}, {0, round}, {0, round}, {0, round}};
+    project_k_f(s, u[0], u[1], a[0], a[1]);
+    int64_t pa[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+#pragma unroll
+      for (int o = 1; o < 4; o <<= 1) {
+        s[q].hh += shfl_xor_ll(s[q].hh, o);
+        s[q].x += shfl_xor_ll(s[q].x, o);
+      }
+      pa[q] = fold60(s[q]);
+    }
+    const int64_t L = shfl_ll(L1, base + sg), u4 = shfl_ll(u41, base + sg);
+    Direction dir;
+    dir.st = shfl_fx(st1, base + 3 + sg);
+    dir.ct = shfl_fx(ct1, base + 3 + sg);
+    dir.cphi = shfl_fx(cp1, base + 3 + sg);
+    dir.sphi = shfl_fx(sp1, base + 3 + sg);
+    FxNorm n;
+    if (norm_fx(pa, n)) {
+      const uint32_t tag = heatbath_tag(colour, mu, sg);
+      Proposal p;
+      int h = 1;
+      ProposalStatus st = propose_fx(L, u4, n, ib, p);
+      if (st == kRejected) st = propose_until(h, hits, key, c0, sweep, tag, n, ib, p);
+      Fx x[4];
+      bool accepted = st == kAccepted;
+      if (accepted) {
+        direction_fx(p, dir, x);
+      } else if (st == kInDouble) {
+        const DrawD r = su2_draw_general(2.0 * d.beta_d / 3.0 * dbl_of(n.kappa, 57 + n.s), hits, key, c0, sweep, tag);
+        h = (int)r.nprop;
+        accepted = r.accepted;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = fx_of(r.x[q]);
+      }
+      np += (uint32_t)h;
+      if (accepted) {
+        ++na;
+        half += (fx_mul(fx_split(n.kappa), x[0]) >> n.s) - pa[0];
+        Fx r[4], rn[4];
+        quat_fx(x, n.v, r);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) rn[q] = fx_neg(r[q]);
+        rotate_col_f(u[0], u[1], r, rn);
+      }
+    }
+    __syncwarp();
+    // subgroups (0,1), (0,2), (1,2): as cm_update_fixed
+    const int keep = sg == 0 ? 0 : 1;
+    const Fc tu = u[2], ta = a[2];
+    u[2] = fc_sel(keep == 0, u[1], u[0]);
+    a[2] = fc_sel(keep == 0, a[1], a[0]);
+    u[0] = fc_sel(keep == 0, u[0], tu);
+    a[0] = fc_sel(keep == 0, a[0], ta);
+    u[1] = fc_sel(keep == 0, tu, u[1]);
+    a[1] = fc_sel(keep == 0, ta, a[1]);
+  }
+  if (!valid) return;
+  if (bad) {
+    if (l8 == 0) {
+      const UpdateCount uc = update_site_f64_general<SUB>(&d, sweep, colour, mu, layer, jj);
+      nprop += uc.nprop;
+      nacc += uc.nacc;
+      dr.general = uc.dretr;
+    }
+    return;
+  }
+  if (l8 == 0) {
+    nprop += np;
+    nacc += na;
+    dr.v = half >> 7;
+  }
+  // after the last swap the rows lie in the order 0, 2, 1
+  if (l8 < 3 && na && in_bounds(js, Vh, kBoundsIndex)) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const Fc e = u[r == 0 ? 0 : 3 - r];
+      pu[js + (3 * r + c) * Vh] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
+    }
+  }
+}
 
 // ------------------------------------------------------------------ re-unitarisation
 
@@ -832,12 +1249,14 @@ __device__ __forceinline__ void finish_single_chain(const EngineArgs &ea, const 
 // measuring: a split into a staple kernel and a heatbath kernel (30 %
 // slower), an L1 prefetch of the next staple direction's links (8 %).
 template <int V> struct TickBounds;
+constexpr int kCoopVariant = 11;
 template <> struct TickBounds<0> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };   // FP32, 128 regs
 template <> struct TickBounds<1> { static constexpr int kThreads = 128, kMinBlocks = 5; static constexpr bool kRolled = false; };   // FP32, 96 regs
 template <> struct TickBounds<2> { static constexpr int kThreads = 128, kMinBlocks = 5; static constexpr bool kRolled = true; };    // FP32, rolled, 96 regs
 template <> struct TickBounds<3> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = true; };    // FP32, rolled, 128 regs
 template <> struct TickBounds<4> { static constexpr int kThreads = 256, kMinBlocks = 3; static constexpr bool kRolled = true; };    // FP32, rolled, 85 regs
 template <> struct TickBounds<10> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64
+template <> struct TickBounds<kCoopVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64, eight lanes per link
 
 // WT: compiled for engines holding a two-coupling DLT chain (any chain with
 // beta1 != beta); unweighted chains compute identically in both forms.
@@ -868,6 +1287,9 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
   // be scheduled.  Both are no-ops for an ordinary launch.
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // the one-coupling FP64 update runs in fixed point, with kLanes lanes per link
+  constexpr bool kFixed = std::is_same<S, StoreF64x18>::value && !WT;
+  constexpr int kLanes = V == kCoopVariant ? kCoopLanes : 1;
   const int total = ea.hdr->total_tiles;
   const int nchains = ea.hdr->nchains;
   int cur = -1;
@@ -903,29 +1325,57 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
     if (!ss.active) continue;
     const int lt = t - sd.tile_base;
     const int layer = lt / sd.tiles_per_vl;  // a layer, or a sublattice box of one
-    const int jj = (lt - layer * sd.tiles_per_vl) * blockDim.x + threadIdx.x;
-    const bool valid = jj < sd.Vn;
+    const int tile = (int)blockDim.x / kLanes, j0 = (lt - layer * sd.tiles_per_vl) * tile;
+    const int jj = j0 + threadIdx.x;
+    const bool valid = (int)threadIdx.x < tile && jj < sd.Vn;
     if (ss.stage < 2 * sd.D) {
       const int colour = ss.stage / sd.D, mu = ss.stage - colour * sd.D;
-      typename S::R dr = 0;  // change of Re Tr(U A), in the kernel's precision
-      if (valid) {
-        if constexpr (TOR)
-          update_site_lean<S, false, 4>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
-        else if constexpr (!TickBounds<V>::kRolled && !SUB)
-          update_site_lean<S, WT>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
-        else
-          update_site<S, TickBounds<V>::kRolled, WT, SUB>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
-      }
-      // book the action change S = sum_p beta_p (1 - Re Tr U_p / 3): each warp
-      // owns the slot of its 32 sites, so the one fire-and-forget add per warp
-      // meets no other add in this launch and the order of adds is fixed
+      if constexpr (kFixed) {
+        ActionChange dr = {0, 0.0};
+        const int jw = j0 + (int)(threadIdx.x & ~31u) / kLanes;  // the first link of the warp
+        if constexpr (kLanes > 1) {
+          const int ju = j0 + (int)threadIdx.x / kLanes;
+          if (jw < sd.Vn)
+            update_site_coop<SUB>(sd, ss.sweep, colour, mu, layer, min(ju, sd.Vn - 1), ju < sd.Vn, np, na, dr);
+        } else {
+          if (valid) update_site_fixed<SUB>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
+        }
+        // the action change, as below: one slot per warp, the sum in integers
+        __syncwarp();
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
-      // (a warp of the ragged last tile with no valid site has no slot)
-      if ((threadIdx.x & 31) == 0 && valid && sd.action_slots) {
-        const int slot = layer * ((sd.Vn + 31) >> 5) + (jj >> 5);
-        if (in_bounds(slot, sd.n_action_slots, kBoundsSlot))
-          atomicAdd(sd.action_slots + slot, sd.action_factor * (double)dr);
+        for (int o = 16; o > 0; o >>= 1) dr.v += __shfl_down_sync(0xffffffffu, (long long)dr.v, o);
+        double sum = dbl_of(dr.v, 49);
+        if (__any_sync(0xffffffffu, dr.general != 0.0)) {
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) dr.general += __shfl_down_sync(0xffffffffu, dr.general, o);
+          sum += dr.general;
+        }
+        if ((threadIdx.x & 31) == 0 && jw < sd.Vn && sd.action_slots) {
+          constexpr int kPerWarp = 32 / kLanes;
+          const int slot = layer * ((sd.Vn + kPerWarp - 1) / kPerWarp) + jw / kPerWarp;
+          if (in_bounds(slot, sd.n_action_slots, kBoundsSlot)) atomicAdd(sd.action_slots + slot, sd.action_factor * sum);
+        }
+      } else {
+        typename S::R dr = 0;  // change of Re Tr(U A), in the kernel's precision
+        if (valid) {
+          if constexpr (TOR)
+            update_site_lean<S, false, 4>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
+          else if constexpr (!TickBounds<V>::kRolled && !SUB)
+            update_site_lean<S, WT>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
+          else
+            update_site<S, TickBounds<V>::kRolled, WT, SUB>(sd, ss.sweep, colour, mu, layer, jj, np, na, dr);
+        }
+        // book the action change S = sum_p beta_p (1 - Re Tr U_p / 3): each warp
+        // owns the slot of its 32 sites, so the one fire-and-forget add per warp
+        // meets no other add in this launch and the order of adds is fixed
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
+        // (a warp of the ragged last tile with no valid site has no slot)
+        if ((threadIdx.x & 31) == 0 && valid && sd.action_slots) {
+          const int slot = layer * ((sd.Vn + 31) >> 5) + (jj >> 5);
+          if (in_bounds(slot, sd.n_action_slots, kBoundsSlot))
+            atomicAdd(sd.action_slots + slot, sd.action_factor * (double)dr);
+        }
       }
     } else if (ss.stage == kStageReunit) {
       if (valid) reunit_site<S, SUB>(sd, layer, jj);
@@ -1480,7 +1930,8 @@ cudaError_t launch_bounds_selftest() {
 
 // ------------------------------------------------------------------ launchers
 // Tick kernel forms: FP32 12-real has variants 0..4 (TickBounds), FP32
-// 18-real variant 0 only, FP64 its one form (10).  A chain divided into
+// 18-real variant 0 only, FP64 one form (10) and, as the launcher's variant 1
+// (not a choice of the caller), eight lanes per link.  A chain divided into
 // sublattice boxes runs one form: FP32 the rolled 128-register variant (3).
 
 constexpr int kSubVariant = 3;
@@ -1534,6 +1985,9 @@ int tick_max_threads(int storage, int variant) {
 template <template <class, int, bool, bool, bool, bool> class OP, bool WT, class... A>
 static cudaError_t tick_dispatch(int storage, int variant, bool sub, int torus, A... a) {
   const bool tor = torus != 0 && !sub && !WT, mc = tor && torus == 2;
+  if (storage == 0 && variant == 1 && !WT)
+    return sub ? OP<StoreF64x18, kCoopVariant, false, true, false, false>::run(a...)
+               : OP<StoreF64x18, kCoopVariant, false, false, false, false>::run(a...);
   if (storage == 0) return sub ? OP<StoreF64x18, 10, WT, true, false, false>::run(a...) : OP<StoreF64x18, 10, WT, false, false, false>::run(a...);
   if (storage == 2) {
     if (sub) return OP<StoreF32x18, kSubVariant, WT, true, false, false>::run(a...);
@@ -1565,7 +2019,7 @@ struct TickOccupancy {
 
 cudaError_t launch_tick(int storage, int variant, bool weighted, bool sub, int torus, const EngineArgs &ea, int grid,
                         int block, cudaStream_t st, bool pdl) {
-  if (sub) variant = storage == 0 ? 0 : kSubVariant;
+  if (sub && storage != 0) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaErrorInvalidConfiguration;
   const EngineArgs *pa = &ea;
   return weighted ? tick_dispatch<TickLaunch, true>(storage, variant, sub, torus, pa, grid, block, st, pdl)
@@ -1632,7 +2086,7 @@ cudaError_t launch_convert(int storage, ChainDesc *desc_dev, size_t nlinks, doub
 
 cudaError_t tick_occupancy(int storage, int variant, bool weighted, bool sub, int torus, int block, int *ctas_per_sm) {
   *ctas_per_sm = 0;
-  if (sub) variant = storage == 0 ? 0 : kSubVariant;
+  if (sub && storage != 0) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaSuccess;
   return weighted ? tick_dispatch<TickOccupancy, true>(storage, variant, sub, torus, block, ctas_per_sm)
                   : tick_dispatch<TickOccupancy, false>(storage, variant, sub, torus, block, ctas_per_sm);
