@@ -116,6 +116,7 @@ static su3_status bounds_status() {
   if (!debug_bounds_build()) return SU3_OK;
   unsigned long long r[3];
   CU(bounds_record(r));
+  if (!r[0]) CU(bounds_record_update(r));
   if (r[0])
     return fail(SU3_ECUDA, "device bounds check: %s %lld outside [0, %lld)", bounds_site_name(r[0]), (long long)r[1],
                 (long long)r[2]);
@@ -124,7 +125,10 @@ static su3_status bounds_status() {
 
 extern "C" su3_status su3_bounds_status(uint64_t *site, int64_t *index, int64_t *extent) {
   unsigned long long r[3] = {0, 0, 0};
-  if (debug_bounds_build()) CU(bounds_record(r));
+  if (debug_bounds_build()) {
+    CU(bounds_record(r));
+    if (!r[0]) CU(bounds_record_update(r));
+  }
   if (site) *site = r[0];
   if (index) *index = (int64_t)r[1];
   if (extent) *extent = (int64_t)r[2];
@@ -253,6 +257,8 @@ extern "C" size_t su3_link_bytes(const su3_config *c) {
 // ------------------------------------------------------------------ chains and the engine
 
 static int g_nsm = 0;
+
+constexpr size_t kCounterBytes = 2 * kCounterSlots * sizeof(unsigned long long);
 
 static su3_status device_sm_count(int *nsm) {
   if (!g_nsm) {
@@ -437,12 +443,13 @@ static void fill_plain(Chain &ch, int tile) {
 
 struct Engine {
   int storage = SU3_FP64_18;
-  bool weighted_any = false;  // some chain has two couplings: the tick kernel's weighted form
+  // One chain whose stages the host knows (lattices, ensembles of one): every
+  // stage is launched as a kernel of its own (run_schedule).  Otherwise the
+  // chains' stage machines live on the device (run_ticks).
+  bool fixed = false;
+  bool weighted_any = false;  // some chain has two couplings: the update's weighted form
   bool sub_any = false;       // the (only) chain is divided into sublattice boxes
   bool torus_all = false;     // every chain is an undivided periodic 4-D torus, one coupling, default key
-  // the tick kernel's torus form: 0 none, 1 the torus form, 2 its form for several chains
-  int torus_form() const { return torus_all ? (chains.size() > 1 ? 2 : 1) : 0; }
-  int torus_form_built = 0;   // the form the captured graph launches
   bool coop = false;          // FP64, too few links to fill the GPU: eight lanes per link
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
   int kernel_variant() const { return coop ? 1 : variant; }
@@ -454,12 +461,14 @@ struct Engine {
     for (int i = 0; i < ch.cfg.D; ++i) n *= ch.cfg.dims[i];
     return n / 2;
   }
+  static constexpr int kMaxChunk = 4;  // sweeps of one graph
   cudaStream_t stream = nullptr;
   std::vector<Chain> chains;
   // device mirrors
   ChainDesc *d_desc = nullptr;
   ChainState *d_state = nullptr;  // [chain][2]: the slot EngineHeader::parity is current
   EngineHeader *d_hdr = nullptr;
+  ChainCtl *d_ctl = nullptr;
   int32_t *d_tile_chain = nullptr;
   int32_t *d_meas_list = nullptr;  // [chain_cap] the chains a launch measures
   size_t tile_cap = 0, chain_cap = 0;
@@ -475,6 +484,8 @@ struct Engine {
   bool pdl = true;
   cudaGraphExec_t graph = nullptr;
   int graph_ticks = 0;
+  // fixed schedule: one graph per kind of chunk (chunk_kind)
+  cudaGraphExec_t chunk_graph[4 * (kMaxChunk + 1)] = {};
   bool tiles_dirty = true;
   // kernel timing (su3_set_profiling)
   bool profiling = false;
@@ -496,7 +507,22 @@ struct Engine {
     prof_pending.clear();
   }
 
-  // Ticks one by one, each between two events, classified by chain 0's stage.
+  // A launch between two events, of kind 0 (update), 1 (re-unitarisation) or
+  // 2 (measurement).
+  template <class F>
+  su3_status profiled(int kind, F &&launch) {
+    EvPair p;
+    p.kind = kind;
+    CU(cudaEventCreate(&p.a));
+    CU(cudaEventCreate(&p.b));
+    CU(cudaEventRecord(p.a, stream));
+    TRY(launch());
+    CU(cudaEventRecord(p.b, stream));
+    prof_pending.push_back(p);
+    return SU3_OK;
+  }
+
+  // Ticks one by one, classified by chain 0's stage.
   su3_status profiled_ticks(long long n) {
     if (tiles_dirty) TRY(rebuild());
     int grid = 0;
@@ -504,14 +530,7 @@ struct Engine {
     ChainState s = chains[0].state;
     const ChainDesc &d = chains[0].desc;
     for (long long t = 0; t < n; ++t) {
-      EvPair p;
-      p.kind = s.stage < 2 * d.D ? 0 : (s.stage == kStageReunit ? 1 : 2);
-      CU(cudaEventCreate(&p.a));
-      CU(cudaEventCreate(&p.b));
-      CU(cudaEventRecord(p.a, stream));
-      TRY(one_tick(grid));
-      CU(cudaEventRecord(p.b, stream));
-      prof_pending.push_back(p);
+      TRY(profiled(s.stage < 2 * d.D ? 0 : (s.stage == kStageReunit ? 1 : 2), [&] { return one_tick(grid); }));
       if (s.active) {
         if (s.stage == kStageMeasure) s.n_meas += 1;
         host_advance_stage(d, s);
@@ -564,13 +583,14 @@ struct Engine {
     drop_events();
     if (wait_event) cudaEventDestroy(wait_event);
     wait_event = nullptr;
-    if (graph) cudaGraphExecDestroy(graph);
-    graph = nullptr;
+    drop_graph();
     for (auto &ch : chains) free_chain(ch);
     chains.clear();
     cudaFree(d_desc);
     cudaFree(d_state);
     cudaFree(d_hdr);
+    cudaFree(d_ctl);
+    d_ctl = nullptr;
     cudaFree(d_tile_chain);
     cudaFree(d_meas_list);
     cudaFree(d_meas_out);
@@ -618,6 +638,8 @@ struct Engine {
     }
     CU(cudaMalloc(&d_hdr, sizeof(EngineHeader)));
     CU(cudaMemsetAsync(d_hdr, 0, sizeof(EngineHeader), stream));
+    CU(cudaMalloc(&d_ctl, sizeof(ChainCtl)));
+    CU(cudaMemsetAsync(d_ctl, 0, sizeof(ChainCtl), stream));
     CU(cudaMallocHost(&h_pinned, 4096));
     return SU3_OK;
   }
@@ -671,16 +693,16 @@ struct Engine {
       fill_plain(ch, narrow);
       ntiles = std::max(ntiles, (size_t)ch.pdesc.nlayers * ch.pdesc.tiles_per_layer);
     }
-    const size_t npart = ntiles * kPartVals;
+    const size_t npart = std::max(ntiles, (size_t)ch.desc.nlayers * kMeasureCtas) * kPartVals;
     const size_t nres = (size_t)ch.desc.result_cap * (ch.desc.nlayers + 1) * kMeasVals;
     cudaError_t e1 = cudaMalloc(&ch.partials, npart * sizeof(double));
     cudaError_t e2 = cudaMalloc(&ch.results, nres * sizeof(double));
-    cudaError_t e3 = cudaMalloc(&ch.counters, 2 * sizeof(unsigned long long));
+    cudaError_t e3 = cudaMalloc(&ch.counters, kCounterBytes);
     if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
       free_chain(ch);
       return fail(SU3_ENOMEM, "scratch allocation failed");
     }
-    ch.bytes_total += npart * sizeof(double) + nres * sizeof(double) + 16;
+    ch.bytes_total += npart * sizeof(double) + nres * sizeof(double) + kCounterBytes;
     ch.n_action_slots = ch.desc.nlayers * ch.desc.nb * ((ch.desc.Vn + narrow - 1) / narrow);
     if (cudaMalloc(&ch.action_slots, (size_t)ch.n_action_slots * sizeof(double)) != cudaSuccess) {
       free_chain(ch);
@@ -693,7 +715,7 @@ struct Engine {
       return fail(SU3_ENOMEM, "action reference allocation failed");
     }
     CU(cudaMemsetAsync(ch.ref_meas, 0, 3 * kMeasVals * sizeof(double), stream));
-    CU(cudaMemsetAsync(ch.counters, 0, 2 * sizeof(unsigned long long), stream));
+    CU(cudaMemsetAsync(ch.counters, 0, kCounterBytes, stream));
     CU(cudaMemsetAsync(ch.results, 0, nres * sizeof(double), stream));
     fill_desc(ch, block);
     if (ch.sub) fill_plain(ch, block);
@@ -715,11 +737,7 @@ struct Engine {
       CU(cudaMemcpyAsync(ch.d_pdesc, &ch.pdesc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
       CU(launch_start(storage, ch.d_pdesc, nlinks, ch.cfg.start == SU3_START_HOT, stream));
       CU(launch_sub_copy(storage, dd, ch.d_pdesc, nlinks, 1, stream));
-      ChainState *ds = nullptr;
-      CU(cudaMallocAsync(&ds, sizeof(ChainState), stream));
-      CU(cudaMemsetAsync(ds, 0, sizeof(ChainState), stream));
-      CU(launch_halo(storage, dd, ds, nullptr, 1, ch.desc.nlayers * ch.desc.nb, ch.halo_n[0] + ch.halo_n[1], stream));
-      CU(cudaFreeAsync(ds, stream));
+      CU(launch_halo(storage, ch.desc, -1, ch.halo_n[0] + ch.halo_n[1], stream));
     } else {
       CU(launch_start(storage, dd, nlinks, ch.cfg.start == SU3_START_HOT, stream));
     }
@@ -748,7 +766,7 @@ struct Engine {
       tiles += ch.desc.nlayers * ch.desc.tiles_per_layer;
     }
     total_tiles = tiles;
-    if (ctas_per_sm <= 0 && tiles != old_tiles) drop_graph();  // the grid follows the tile count
+    if (fixed || (ctas_per_sm <= 0 && tiles != old_tiles)) drop_graph();  // the grid follows the tile count
     bool w = false, sb = false;
     for (auto &ch : chains) {
       w = w || ch.desc.weighted;
@@ -765,10 +783,6 @@ struct Engine {
       weighted_any = w;
       sub_any = sb;
       torus_all = tor;
-      drop_graph();
-    }
-    if (torus_form() != torus_form_built) {  // one chain <-> several: the torus form changes too
-      torus_form_built = torus_form();
       drop_graph();
     }
     if (chains.size() > chain_cap) {
@@ -811,14 +825,23 @@ struct Engine {
       CU(cudaMemcpyAsync(d_state, states.data(), states.size() * sizeof(ChainState), cudaMemcpyHostToDevice, stream));
     }
     CU(cudaMemcpyAsync(d_hdr, &h, sizeof h, cudaMemcpyHostToDevice, stream));
+    if (fixed) TRY(upload_ctl());
     CU(cudaStreamSynchronize(stream));
     tiles_dirty = false;
+    return SU3_OK;
+  }
+
+  // The host mirror's counters of a fixed schedule, in stream order.
+  su3_status upload_ctl() {
+    const ChainState &s = chains[0].state;
+    CU(launch_set_ctl(d_ctl, s.sweep, s.n_meas, s.anchor, stream));
     return SU3_OK;
   }
 
   // Both state slots of every chain get the host mirror's state, so the
   // parity does not matter.
   su3_status upload_states() {
+    if (fixed) return upload_ctl();
     std::vector<ChainState> states(2 * chains.size());
     for (size_t c = 0; c < chains.size(); ++c) states[2 * c] = states[2 * c + 1] = chains[c].state;
     if (!states.empty())
@@ -850,6 +873,10 @@ struct Engine {
     if (graph) cudaGraphExecDestroy(graph);
     graph = nullptr;
     graph_ticks = 0;
+    for (auto &g : chunk_graph) {
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
   }
 
   // ctas_per_sm = 0: one CTA per tile (the hardware balances the tail);
@@ -867,23 +894,21 @@ struct Engine {
 
   EngineArgs args() const { return EngineArgs{d_desc, d_state, d_hdr, d_tile_chain, d_meas_list}; }
 
-  // Halo refresh of the (only) chain of an engine with a divided chain.
-  cudaError_t halo_refresh(ChainDesc *dd, ChainState *ds, int all) const {
+  // Halo refresh of a divided chain (stage -1: all links).
+  cudaError_t halo_refresh(int stage, bool programmatic) const {
     const Chain &ch = chains[0];
-    return launch_halo(storage, dd, ds, d_hdr, all, ch.desc.nlayers * ch.desc.nb, ch.halo_n[0] + ch.halo_n[1], stream);
+    return launch_halo(storage, ch.desc, stage, ch.halo_n[0] + ch.halo_n[1], stream, programmatic);
   }
 
-  // One tick, and for a divided chain the halo refresh of what it changed.
   su3_status one_tick(int grid) {
-    cudaError_t e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
+    cudaError_t e = launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, pdl);
     if (e != cudaSuccess && pdl) {  // not offered here: plain launches from now on
       cudaGetLastError();
       pdl = false;
       drop_graph();
-      e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, false);
+      e = launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, false);
     }
     CU(e);
-    if (sub_any) CU(halo_refresh(d_desc, d_state, 0));
     return SU3_OK;
   }
 
@@ -893,7 +918,7 @@ struct Engine {
     Chain &ch = chains[c];
     const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
     CU(launch_sub_copy(storage, d_desc + c, ch.d_pdesc, nlinks, to_sub, stream));
-    if (to_sub) CU(halo_refresh(d_desc + c, d_state + 2 * c, 1));
+    if (to_sub) CU(halo_refresh(-1, false));
     return SU3_OK;
   }
 
@@ -939,8 +964,7 @@ struct Engine {
     cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
     for (int i = 0; i < kGraphTicks && e == cudaSuccess; ++i) {
-      e = launch_tick(storage, kernel_variant(), weighted_any, sub_any, torus_form(), args(), grid, block, stream, pdl);
-      if (e == cudaSuccess && sub_any) e = halo_refresh(d_desc, d_state, 0);
+      e = launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, pdl);
     }
     cudaError_t e2 = cudaStreamEndCapture(stream, &g);
     if (e == cudaSuccess) e = e2;
@@ -963,6 +987,129 @@ struct Engine {
       }
     }
     return tick_direct((int)n);
+  }
+
+  // ---- fixed schedule (one chain)
+  // A chunk: m sweeps, then a re-unitarisation and a measurement if due.
+  struct Chunk {
+    int m;
+    bool reunit, measure;
+    int kind() const { return 4 * m + 2 * (reunit ? 1 : 0) + (measure ? 1 : 0); }
+  };
+
+  // The next chunk of a chain with n sweeps to go: up to the next stage that
+  // is due, kMaxChunk sweeps at most.
+  Chunk next_chunk(int n) const {
+    const Chain &ch = chains[0];
+    Chunk c{0, false, false};
+    while (c.m < n && c.m < kMaxChunk && !c.reunit && !c.measure) {
+      ++c.m;
+      const uint32_t s = ch.state.sweep + (uint32_t)c.m;
+      c.reunit = ch.desc.reunit_every > 0 && s % (uint32_t)ch.desc.reunit_every == 0;
+      c.measure = ch.desc.measure_every > 0 && s % (uint32_t)ch.desc.measure_every == 0;
+    }
+    return c;
+  }
+
+  cudaError_t measure_recorded() {
+    return launch_measure(storage, sub_any, chains[0].desc, nullptr, d_ctl, stream, pdl);
+  }
+  cudaError_t reunit_all() {
+    cudaError_t e = launch_reunit(storage, sub_any, chains[0].desc, stream, pdl);
+    if (e == cudaSuccess && sub_any) e = halo_refresh(-1, pdl);
+    return e;
+  }
+
+  // The launches of a chunk; each(kind, launch) runs one.
+  template <class F>
+  su3_status launch_chunk(const Chunk &c, int grid, F &&each) {
+    const ChainDesc &d = chains[0].desc;
+    for (int i = 0; i < c.m; ++i)
+      for (int st = 0; st < 2 * d.D; ++st) {
+        UpdateStep u{};
+        u.colour = st / d.D;
+        u.mu = st % d.D;
+        u.offset = (uint32_t)i;
+        u.first = i == 0 && st == 0;
+        u.advance = i == c.m - 1 && st == 2 * d.D - 1 ? (uint32_t)c.m : 0u;
+        u.tiles = total_tiles;
+        TRY(each(0, [&]() -> cudaError_t {
+          cudaError_t e = launch_update(storage, kernel_variant(), weighted_any, sub_any, torus_all, d, d_ctl, u, grid,
+                                        block, stream, pdl);
+          if (e == cudaSuccess && sub_any) e = halo_refresh(st, pdl);
+          return e;
+        }));
+      }
+    if (c.reunit) TRY(each(1, [&] { return reunit_all(); }));
+    if (c.measure) TRY(each(2, [&] { return measure_recorded(); }));
+    return SU3_OK;
+  }
+
+  // Capture a chunk; cudaErrorNotSupported etc. come back for a second try
+  // without programmatic launches.
+  cudaError_t capture_chunk(const Chunk &c, int grid, cudaGraphExec_t *out) {
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal), le = cudaSuccess;
+    if (e != cudaSuccess) return e;
+    launch_chunk(c, grid, [&](int, auto &&launch) -> su3_status {
+      if (le == cudaSuccess) le = launch();
+      return SU3_OK;
+    });
+    e = cudaStreamEndCapture(stream, &g);
+    if (le != cudaSuccess) e = le;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(out, g, 0);
+    if (g) cudaGraphDestroy(g);
+    if (e != cudaSuccess) *out = nullptr;
+    return e;
+  }
+
+  su3_status run_chunk(const Chunk &c) {
+    int grid = 0;
+    TRY(grid_size(&grid));
+    if (use_graph && !profiling) {
+      cudaGraphExec_t &g = chunk_graph[c.kind()];
+      if (!g) {
+        cudaError_t e = capture_chunk(c, grid, &g);
+        if (e != cudaSuccess && pdl) {  // programmatic edges not capturable here: plain ones
+          cudaGetLastError();
+          pdl = false;
+          e = capture_chunk(c, grid, &g);
+        }
+        if (e != cudaSuccess) return fail(SU3_ECUDA, "graph capture of %d sweeps: %s", c.m, cudaGetErrorString(e));
+      }
+      CU(cudaGraphLaunch(g, stream));
+      return SU3_OK;
+    }
+    return launch_chunk(c, grid, [&](int kind, auto &&launch) -> su3_status {
+      auto once = [&]() -> su3_status {
+        cudaError_t e = launch();
+        if (e != cudaSuccess && pdl) {  // not offered here: plain launches from now on
+          cudaGetLastError();
+          pdl = false;
+          drop_graph();
+          e = launch();
+        }
+        CU(e);
+        return SU3_OK;
+      };
+      return profiling ? profiled(kind, once) : once();
+    });
+  }
+
+  // n sweeps of the chain.  The mirror follows the launches queued.
+  su3_status run_schedule(int n) {
+    Chain &ch = chains[0];
+    while (n > 0) {
+      const Chunk c = next_chunk(n);
+      TRY(run_chunk(c));
+      ch.state.sweep += (uint32_t)c.m;
+      if (c.measure) {
+        ch.state.n_meas += 1;
+        ch.state.anchor = 0;  // the measurement restarted the bookkeeping
+      }
+      n -= c.m;
+    }
+    return SU3_OK;
   }
 
   // Host mirror: ticks until every chain in `which` is idle again.
@@ -1000,6 +1147,7 @@ struct Engine {
     if (n < 0) return fail(SU3_EINVAL, "negative sweep count %d", n);
     if (n == 0) return SU3_OK;
     if (tiles_dirty) TRY(rebuild());
+    if (fixed) return run_schedule(n);
     for (auto &ch : chains) {
       ch.state.target = ch.state.sweep + (uint32_t)n;
       ch.state.active = 1;
@@ -1013,15 +1161,21 @@ struct Engine {
     return SU3_OK;
   }
 
+  // Measure a chain's links (divided: gathered into the undivided layout)
+  // into device memory, queued.
+  su3_status measure_into(size_t c, double *device_out) {
+    ChainDesc *dd = nullptr;
+    TRY(io_desc(c, &dd));
+    CU(launch_measure(storage, false, chains[c].sub ? chains[c].pdesc : chains[c].desc, device_out, d_ctl, stream, false));
+    return SU3_OK;
+  }
+
   su3_status measure_chain(size_t c, double *host_out /* 5*(layers+1) */) {
     if (tiles_dirty) TRY(rebuild());
     Chain &ch = chains[c];
     const int nvals = (ch.desc.nlayers + 1) * kMeasVals;
     if (!d_meas_out) CU(cudaMalloc(&d_meas_out, 3 * kMeasVals * sizeof(double)));
-    ChainDesc *dd = nullptr;
-    TRY(io_desc(c, &dd));
-    const ChainDesc &md = ch.sub ? ch.pdesc : ch.desc;
-    CU(launch_measure(storage, dd, md.nlayers * md.tiles_per_layer, block, d_meas_out, stream));
+    TRY(measure_into(c, d_meas_out));
     CU(cudaMemcpyAsync(h_pinned, d_meas_out, nvals * sizeof(double), cudaMemcpyDeviceToHost, stream));
     CU(cudaStreamSynchronize(stream));
     std::memcpy(host_out, h_pinned, nvals * sizeof(double));
@@ -1084,21 +1238,25 @@ struct Engine {
     return SU3_OK;
   }
 
+  // The mirror's bookkeeping-restart flag of a chain, in stream order.
+  su3_status set_anchor(size_t c) {
+    if (fixed) return upload_ctl();
+    CU(launch_set_anchor(d_state + 2 * c, chains[c].state.anchor, stream));
+    return SU3_OK;
+  }
+
   // The bookkeeping restarts from the current links: clear the booked
   // changes and measure the reference action on the device, in stream
   // order and without waiting (su3_action reads the reference).
   su3_status action_reset(size_t c) {
     Chain &ch = chains[c];
     if (ch.state.anchor) {  // restarting now: no restart at the next measurement
-      CU(launch_set_anchor(d_state + 2 * c, 0, stream));
       ch.state.anchor = 0;
+      TRY(set_anchor(c));
     }
     CU(cudaMemsetAsync(ch.action_slots, 0, (size_t)ch.n_action_slots * sizeof(double), stream));
     if (!ch.desc.weighted) {
-      ChainDesc *dd = nullptr;
-      TRY(io_desc(c, &dd));
-      const ChainDesc &md = ch.sub ? ch.pdesc : ch.desc;
-      CU(launch_measure(storage, dd, md.nlayers * md.tiles_per_layer, block, ch.ref_meas, stream));
+      TRY(measure_into(c, ch.ref_meas));
     }
     return SU3_OK;
   }
@@ -1110,9 +1268,8 @@ struct Engine {
   su3_status action_defer(size_t c) {
     Chain &ch = chains[c];
     if (ch.desc.weighted || ch.desc.measure_every <= 0) return action_reset(c);
-    CU(launch_set_anchor(d_state + 2 * c, 1, stream));
     ch.state.anchor = 1;
-    return SU3_OK;
+    return set_anchor(c);
   }
 
   // Action at the last reset (0 for the two-coupling DLT: its booked value
@@ -1134,10 +1291,12 @@ struct Engine {
   }
 
   su3_status counters(size_t c, uint64_t *prop, uint64_t *acc) {
-    CU(cudaMemcpyAsync(h_pinned, chains[c].counters, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, stream));
+    static_assert(kCounterBytes <= 4096, "h_pinned");
+    CU(cudaMemcpyAsync(h_pinned, chains[c].counters, kCounterBytes, cudaMemcpyDeviceToHost, stream));
     CU(cudaStreamSynchronize(stream));
-    unsigned long long v[2];
-    std::memcpy(v, h_pinned, sizeof v);
+    unsigned long long all[2 * kCounterSlots], v[2] = {0, 0};
+    std::memcpy(all, h_pinned, sizeof all);
+    for (int i = 0; i < 2 * kCounterSlots; ++i) v[i & 1] += all[i];
     if (prop) *prop = v[0];
     if (acc) *acc = v[1];
     return SU3_OK;
@@ -1189,6 +1348,7 @@ static su3_status make_lattice(const su3_config *cfg, su3_lattice **out) {
   *out = nullptr;
   TRY(validate(cfg));
   auto *lat = new su3_lattice();
+  lat->eng.fixed = true;
   su3_status st = lat->eng.init(cfg->storage, (cudaStream_t)cfg->stream);
   if (st == SU3_OK) {
     Chain ch;
@@ -1240,6 +1400,7 @@ extern "C" su3_status su3_sweep(su3_lattice *lat, int n, int hits) {
     ch.cfg.hits = hits;
     ch.desc.hits = hits;
     TRY(lat->eng.upload_desc(0));
+    lat->eng.drop_graph();  // the captured launches carry the descriptor
   }
   return lat->eng.sweep_all(n);
 }
@@ -1248,18 +1409,8 @@ extern "C" su3_status su3_reunitarize(su3_lattice *lat) {
   LAT_CHECK(lat);
   Engine &e = lat->eng;
   if (e.tiles_dirty) TRY(e.rebuild());
-  Chain &ch = e.chains[0];
-  // one re-unitarisation stage through the tick kernel
-  const ChainState saved = ch.state;
-  ch.state.stage = kStageReunit;
-  ch.state.active = 1;
-  ch.state.target = ch.state.sweep;  // idle again right after
-  TRY(e.upload_states());
-  TRY(e.tick_direct(1));
-  ch.state = saved;
-  ch.state.stage = 0;
-  ch.state.active = 0;
-  return e.upload_states();
+  CU(e.reunit_all());
+  return SU3_OK;
 }
 
 extern "C" su3_status su3_plaquette(su3_lattice *lat, int layer, double *total, double *space, double *time) {
@@ -1292,12 +1443,7 @@ extern "C" su3_status su3_measure_async(su3_lattice *lat, double *device_out) {
   if (!device_out) return fail(SU3_EINVAL, "device_out is NULL");
   Engine &e = lat->eng;
   if (e.tiles_dirty) TRY(e.rebuild());
-  Chain &ch = e.chains[0];
-  ChainDesc *dd = nullptr;
-  TRY(e.io_desc(0, &dd));
-  const ChainDesc &md = ch.sub ? ch.pdesc : ch.desc;
-  CU(launch_measure(e.storage, dd, md.nlayers * md.tiles_per_layer, e.block, device_out, e.stream));
-  return SU3_OK;
+  return e.measure_into(0, device_out);
 }
 
 static su3_status chain_measurements(Engine &e, size_t c, double *host_out, size_t max, size_t *count) {
@@ -1523,10 +1669,10 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     }
   }
   std::vector<ChainState> saved_state;
-  std::vector<unsigned long long> saved_cnt(2 * e.chains.size());
+  std::vector<unsigned long long> saved_cnt(2 * kCounterSlots * e.chains.size());
   for (size_t c = 0; c < e.chains.size(); ++c) {
     saved_state.push_back(e.chains[c].state);
-    CU(cudaMemcpyAsync(&saved_cnt[2 * c], e.chains[c].counters, 16, cudaMemcpyDeviceToHost, e.stream));
+    CU(cudaMemcpyAsync(&saved_cnt[2 * kCounterSlots * c], e.chains[c].counters, kCounterBytes, cudaMemcpyDeviceToHost, e.stream));
   }
   CU(cudaStreamSynchronize(e.stream));
   const int saved_var = e.variant, saved_block = e.block, saved_ctas = e.ctas_per_sm;
@@ -1549,7 +1695,10 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     for (int t : cand_t) {
       if (t > tick_max_threads(e.storage, v)) continue;
       int occ = 0;
-      if (tick_occupancy(e.storage, e.coop ? 1 : v, e.weighted_any, e.sub_any, e.torus_form(), t, &occ) != cudaSuccess || occ < 1) continue;
+      const int kv = e.coop ? 1 : v;
+      const cudaError_t oe = e.fixed ? update_occupancy(e.storage, kv, e.weighted_any, e.sub_any, e.torus_all, t, &occ)
+                                     : tick_occupancy(e.storage, kv, e.weighted_any, e.torus_all, t, &occ);
+      if (oe != cudaSuccess || occ < 1) continue;
       // 0 = one CTA per tile, then persistent grids of 1, 2, 4, ..., occ CTAs per SM
       for (int c = 0; c <= occ && st == SU3_OK; c = (c == 0) ? 1 : ((c < occ && 2 * c > occ) ? occ : 2 * c)) {
         if ((st = e.set_launch(v, t, c)) != SU3_OK) break;
@@ -1583,7 +1732,7 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     if (slots[c])
       cudaMemcpyAsync(e.chains[c].action_slots, slots[c], (size_t)e.chains[c].n_action_slots * sizeof(double),
                       cudaMemcpyDeviceToDevice, e.stream);
-    cudaMemcpyAsync(e.chains[c].counters, &saved_cnt[2 * c], 16, cudaMemcpyHostToDevice, e.stream);
+    cudaMemcpyAsync(e.chains[c].counters, &saved_cnt[2 * kCounterSlots * c], kCounterBytes, cudaMemcpyHostToDevice, e.stream);
     e.chains[c].state = saved_state[c];
   }
   cudaStreamSynchronize(e.stream);
@@ -1654,6 +1803,7 @@ extern "C" su3_status su3_ensemble_create(const su3_config *cfgs, int nchains, v
     if (divided(&cfgs[c])) return fail(SU3_EINVAL, "chain %d: ensembles take undivided lattices (ndiv)", c);
   }
   auto *ens = new su3_ensemble();
+  ens->eng.fixed = nchains == 1;
   su3_status st = ens->eng.init(cfgs[0].storage, (cudaStream_t)stream);
   for (int c = 0; c < nchains && st == SU3_OK; ++c) {
     su3_config cfg = cfgs[c];
@@ -1792,7 +1942,8 @@ static size_t job_bytes(const su3_config &c) {
   const size_t layers = c.boundary == SU3_DLT ? 2 : 1;
   const size_t tiles = layers * ((V / 2 + 31) / 32);
   const size_t cap = c.measure_capacity > 0 ? (size_t)c.measure_capacity : 1024;
-  return link_bytes_of(&c) + tiles * kPartVals * 8 + cap * (layers + 1) * kMeasVals * 8 + 16 + tiles * 8;
+  return link_bytes_of(&c) + std::max(tiles, layers * kMeasureCtas) * kPartVals * 8 + cap * (layers + 1) * kMeasVals * 8 +
+         kCounterBytes + tiles * 8;
 }
 
 extern "C" su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, su3_server **out) {
@@ -1821,7 +1972,7 @@ extern "C" su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, 
     // persistent grid: its size does not depend on the resident jobs, so the
     // captured graph of ticks survives admissions and retirements
     int occ = 0;
-    if (tick_occupancy(SU3_FP32_12, srv->eng.variant, false, false, 0, srv->eng.block, &occ) != cudaSuccess || occ < 1) occ = 1;
+    if (tick_occupancy(SU3_FP32_12, srv->eng.variant, false, false, srv->eng.block, &occ) != cudaSuccess || occ < 1) occ = 1;
     srv->eng.ctas_per_sm = occ;
   }
   if (cudaEventCreate(&srv->round_ev[0]) != cudaSuccess || cudaEventCreate(&srv->round_ev[1]) != cudaSuccess) {

@@ -46,6 +46,11 @@ constexpr float kAlphaAccurateLog = 2.0f;
 constexpr int kCoopLanes = 8;
 constexpr int kCoopSites = 8192;
 
+// Pairs of FHKP counters per chain (their sums are the totals).
+constexpr int kCounterSlots = 32;
+// A measurement's partial sums: at most this many CTAs per layer.
+constexpr int kMeasureCtas = 1024;
+
 // Results per measurement slot: [total, space, time, poly_re, poly_im].
 constexpr int kMeasVals = 5;
 // Partial sums per tile in a measurement: [space, time, poly_re, poly_im].
@@ -55,7 +60,7 @@ struct ChainDesc {
   void *links;               // storage base (Vec units, see su3_device.cuh)
   double *results;           // [result_cap][nlayers + 1][kMeasVals]
   double *partials;          // [tiles][kPartVals]
-  unsigned long long *counters;  // [proposals, accepts]
+  unsigned long long *counters;  // [kCounterSlots][proposals, accepts]
   double *action_slots;      // booked action changes, one slot per warp of sites: [layer][ceil(Vh/32)]
   double *ref_meas;          // the measurement the booked changes count from: [nlayers + 1][kMeasVals]
   int32_t n_action_slots;
@@ -118,6 +123,27 @@ struct ChainState {
   int32_t prev_stage;      // stage run by the last tick (-1: none); read by the halo refresh
   int32_t anchor;          // 1: the next measurement restarts the action bookkeeping
   int32_t pad;
+};
+
+// The device side of a one-chain engine's fixed schedule.  The sweep counter
+// has two copies: the launches of one graph read `cur` (its first launch
+// copies `nxt` there), and its last launch writes `nxt`, so that no launch
+// reads a word that its own CTAs write.
+struct ChainCtl {
+  uint32_t cur, nxt;
+  uint32_t n_meas;         // measurements recorded
+  int32_t anchor;          // 1: the next measurement restarts the action bookkeeping
+  uint32_t done;           // CTAs of a measurement that have written their partial sums
+  int32_t pad[3];
+};
+
+// One update phase of a fixed schedule.
+struct UpdateStep {
+  int32_t colour, mu;
+  uint32_t offset;         // sweeps completed since the schedule's first launch
+  uint32_t advance;        // last launch: sweeps to add to the counter (0: not the last)
+  int32_t first;           // 1: the schedule's first launch
+  int32_t tiles;
 };
 
 struct EngineHeader {

@@ -38,7 +38,7 @@
 #include <initializer_list>
 
 #ifdef __CUDACC__
-#define SU3_HD __host__ __device__ __forceinline__
+#define SU3_HD __device__ __forceinline__
 #define SU3_TABLE static __device__ const
 #else
 #define SU3_HD inline

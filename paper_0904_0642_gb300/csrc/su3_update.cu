@@ -1,0 +1,219 @@
+// su3_update.cu -- kernels of one chain (sm_103a): the update phases, the
+// re-unitarisation and the measurement of a lattice whose schedule the host
+// knows.  The descriptor is a kernel parameter: geometry and pointers are
+// uniform values from the constant bank, nothing is loaded before the links.
+#include "su3_launch.h"
+#include "su3_site.cuh"
+
+namespace su3g {
+
+// Every kernel may be scheduled before the previous one of the stream has
+// finished (programmatic launch): wait for its completion and memory before
+// touching anything, then let the next kernel be scheduled.  Both are no-ops
+// for an ordinary launch.
+__device__ __forceinline__ void wait_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class S, int V, bool WT, bool SUB, bool TOR>
+__global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBlocks)
+    k_update(const __grid_constant__ ChainDesc d, ChainCtl *ctl, const UpdateStep u) {
+  wait_previous();
+  const uint32_t base = __ldcg(u.first ? &ctl->nxt : &ctl->cur);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (u.first) ctl->cur = base;
+    if (u.advance) ctl->nxt = base + u.advance;
+  }
+  uint32_t np = 0, na = 0;
+  for (int lt = blockIdx.x; lt < u.tiles; lt += gridDim.x)
+    update_tile<S, V, WT, SUB, TOR>(d, base + u.offset, u.colour, u.mu, lt, np, na);
+  flush_counters(d, np, na);
+}
+
+// One thread per checkerboard index of a (virtual) layer.
+template <class S, bool SUB>
+__global__ void __launch_bounds__(128) k_reunit(const __grid_constant__ ChainDesc d) {
+  wait_previous();
+  const int jj = blockIdx.x * blockDim.x + threadIdx.x;
+  if (jj < d.Vn) reunit_site<S, SUB>(d, blockIdx.y, jj);
+}
+
+// Plaquettes (one site per thread) and Polyakov lines (one per thread) of
+// layer blockIdx.y, the lines first: the longest work starts first.  The last
+// CTA to finish sums the CTAs' partial sums in a fixed order.
+template <class S, bool SUB>
+__global__ void __launch_bounds__(128) k_measure(const __grid_constant__ ChainDesc d, double *out, ChainCtl *ctl,
+                                                 int record) {
+  __shared__ double s_red[32 * kPartVals];
+  __shared__ int s_last;
+  wait_previous();
+  const int layer = blockIdx.y, T = d.D - 1;
+  const int nl = (SUB && d.hpad[T]) ? 0 : d.Vn / d.idims[T];  // lines per colour of a box
+  const int ltiles = (nl + 127) / 128, tiles = ltiles + (d.Vn + 127) / 128;
+  double v[kPartVals] = {0, 0, 0, 0};
+  for (int t = blockIdx.x; t < d.nb * 2 * tiles; t += gridDim.x) {
+    int r = t;
+    const bool line = r < d.nb * 2 * ltiles;
+    if (!line) r -= d.nb * 2 * ltiles;
+    const int per = line ? ltiles : tiles - ltiles;
+    const int cb = r / per, jj = (r - cb * per) * 128 + threadIdx.x;
+    const int colour = cb & 1, vl = layer * d.nb + (cb >> 1);
+    if (jj >= (line ? nl : d.Vn)) continue;
+    const SiteGeo g = site_of<SUB>(d, vl, colour, jj);
+    if (line) {
+      const C<typename S::R> p = polyakov_line<S, SUB>(d, g, colour);
+      v[2] += to_double(p.re);
+      v[3] += to_double(p.im);
+    } else {
+      typename S::R ps, pt;
+      site_plaquettes<S, SUB>(d, g, colour, ps, pt);
+      v[0] += to_double(ps);
+      v[1] += to_double(pt);
+    }
+  }
+  block_reduce(v, s_red);
+  if (threadIdx.x == 0) {
+    const int slot = layer * gridDim.x + blockIdx.x;
+    if (in_bounds(slot, d.nlayers * kMeasureCtas, kBoundsPartial))
+      for (int k = 0; k < kPartVals; ++k) d.partials[(size_t)slot * kPartVals + k] = v[k];
+    __threadfence();
+    s_last = atomicAdd(&ctl->done, 1u) == gridDim.x * gridDim.y - 1;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  const uint32_t slot = ctl->n_meas;
+  if (record) out = d.results + (size_t)(slot % (uint32_t)d.result_cap) * (d.nlayers + 1) * kMeasVals;
+  double whole[kPartVals] = {0, 0, 0, 0};
+  for (int l = 0; l < d.nlayers; ++l) {
+    double w[kPartVals] = {0, 0, 0, 0};
+    for (int b = threadIdx.x; b < gridDim.x; b += 128)
+#pragma unroll
+      for (int k = 0; k < kPartVals; ++k) w[k] += __ldcg(d.partials + (size_t)(l * gridDim.x + b) * kPartVals + k);
+    block_reduce(w, s_red);
+    if (threadIdx.x == 0) {
+      measured_values(d, w, 1.0, out + l * kMeasVals);
+      for (int k = 0; k < kPartVals; ++k) whole[k] += w[k];
+    }
+  }
+  if (threadIdx.x == 0) {
+    measured_values(d, whole, (double)d.nlayers, out + d.nlayers * kMeasVals);
+    ctl->done = 0;
+  }
+  if (!record) return;
+  // a chain whose links were replaced restarts its action bookkeeping here
+  const int anchor = ctl->anchor;
+  __syncthreads();
+  if (anchor) {
+    for (int i = threadIdx.x; i < (d.nlayers + 1) * kMeasVals; i += 128) d.ref_meas[i] = out[i];
+    for (int i = threadIdx.x; i < d.n_action_slots; i += 128) d.action_slots[i] = 0.0;
+  }
+  if (threadIdx.x == 0) {
+    ctl->n_meas = slot + 1;
+    ctl->anchor = 0;
+  }
+}
+
+__global__ void k_set_ctl(ChainCtl *ctl, uint32_t sweep, uint32_t n_meas, int anchor) {
+  *ctl = ChainCtl{sweep, sweep, n_meas, anchor, 0u, {0, 0, 0}};
+}
+
+// ------------------------------------------------------------------ launchers
+
+constexpr int kSubVariant = 3;  // the FP32 variant of a divided chain
+
+template <class S, int V, bool WT, bool SUB, bool TOR>
+struct UpdateLaunch {
+  static cudaError_t run(const ChainDesc *d, ChainCtl *ctl, const UpdateStep *u, int grid, int block, cudaStream_t st,
+                         bool pdl) {
+    return launch_ex(k_update<S, V, WT, SUB, TOR>, dim3((unsigned)grid), block, st, pdl, *d, ctl, *u);
+  }
+};
+template <class S, int V, bool WT, bool SUB, bool TOR>
+struct UpdateOccupancy {
+  static cudaError_t run(int block, int *ctas) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_update<S, V, WT, SUB, TOR>, block, 0);
+  }
+};
+
+// One switch for launching and for occupancy queries: OP<S, V, WT, SUB, TOR>.
+template <template <class, int, bool, bool, bool> class OP, bool WT, class... A>
+static cudaError_t update_dispatch(int storage, int variant, bool sub, bool torus, A... a) {
+  constexpr bool kT = !WT;
+  const bool tor = torus && !WT;
+  if (storage == 0) {
+    if (variant == 1 && !WT)
+      return sub ? OP<StoreF64x18, kCoopVariant, false, true, false>::run(a...)
+                 : OP<StoreF64x18, kCoopVariant, false, false, false>::run(a...);
+    return sub ? OP<StoreF64x18, 10, WT, true, false>::run(a...) : OP<StoreF64x18, 10, WT, false, false>::run(a...);
+  }
+  if (storage == 2) {
+    if (sub) return OP<StoreF32x18, kSubVariant, WT, true, false>::run(a...);
+    return tor ? OP<StoreF32x18, 0, false, false, kT>::run(a...) : OP<StoreF32x18, 0, WT, false, false>::run(a...);
+  }
+  if (sub) return OP<StoreF32x12, kSubVariant, WT, true, false>::run(a...);
+  switch (variant) {
+    case 0: return tor ? OP<StoreF32x12, 0, false, false, kT>::run(a...) : OP<StoreF32x12, 0, WT, false, false>::run(a...);
+    case 1: return tor ? OP<StoreF32x12, 1, false, false, kT>::run(a...) : OP<StoreF32x12, 1, WT, false, false>::run(a...);
+    case 2: return OP<StoreF32x12, 2, WT, false, false>::run(a...);
+    case 3: return OP<StoreF32x12, 3, WT, false, false>::run(a...);
+    default: return OP<StoreF32x12, 4, WT, false, false>::run(a...);
+  }
+}
+
+cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, bool torus, const ChainDesc &d,
+                          ChainCtl *ctl, const UpdateStep &step, int grid, int block, cudaStream_t st, bool pdl) {
+  if (sub && storage != 0) variant = kSubVariant;
+  if (block > tick_max_threads(storage, variant)) return cudaErrorInvalidConfiguration;
+  const ChainDesc *pd = &d;
+  const UpdateStep *pu = &step;
+  return weighted ? update_dispatch<UpdateLaunch, true>(storage, variant, sub, torus, pd, ctl, pu, grid, block, st, pdl)
+                  : update_dispatch<UpdateLaunch, false>(storage, variant, sub, torus, pd, ctl, pu, grid, block, st, pdl);
+}
+
+cudaError_t update_occupancy(int storage, int variant, bool weighted, bool sub, bool torus, int block,
+                             int *ctas_per_sm) {
+  *ctas_per_sm = 0;
+  if (sub && storage != 0) variant = kSubVariant;
+  if (block > tick_max_threads(storage, variant)) return cudaSuccess;
+  return weighted ? update_dispatch<UpdateOccupancy, true>(storage, variant, sub, torus, block, ctas_per_sm)
+                  : update_dispatch<UpdateOccupancy, false>(storage, variant, sub, torus, block, ctas_per_sm);
+}
+
+cudaError_t launch_reunit(int storage, bool sub, const ChainDesc &d, cudaStream_t st, bool pdl) {
+  const dim3 grid((unsigned)((d.Vn + 127) / 128), (unsigned)(d.nlayers * d.nb));
+  return by_storage(storage, [&](auto s) {
+    using S = decltype(s);
+    return sub ? launch_ex(k_reunit<S, true>, grid, 128, st, pdl, d) : launch_ex(k_reunit<S, false>, grid, 128, st, pdl, d);
+  });
+}
+
+cudaError_t launch_measure(int storage, bool sub, const ChainDesc &d, double *out, ChainCtl *ctl, cudaStream_t st,
+                           bool pdl) {
+  const int T = d.D - 1, nl = (sub && d.hpad[T]) ? 0 : d.Vn / d.idims[T];
+  const long long tiles = (long long)d.nb * 2 * ((nl + 127) / 128 + (d.Vn + 127) / 128);
+  const dim3 grid((unsigned)(tiles < kMeasureCtas ? tiles : kMeasureCtas), (unsigned)d.nlayers);
+  const int record = out ? 0 : 1;
+  return by_storage(storage, [&](auto s) {
+    using S = decltype(s);
+    return sub ? launch_ex(k_measure<S, true>, grid, 128, st, pdl, d, out, ctl, record)
+               : launch_ex(k_measure<S, false>, grid, 128, st, pdl, d, out, ctl, record);
+  });
+}
+
+cudaError_t launch_set_ctl(ChainCtl *ctl, uint32_t sweep, uint32_t n_meas, int anchor, cudaStream_t st) {
+  k_set_ctl<<<1, 1, 0, st>>>(ctl, sweep, n_meas, anchor);
+  return cudaGetLastError();
+}
+
+cudaError_t bounds_record_update(unsigned long long out[3]) {
+  out[0] = out[1] = out[2] = 0;
+#ifdef SU3_DEBUG_BOUNDS
+  return cudaMemcpyFromSymbol(out, g_bounds, 3 * sizeof(unsigned long long));
+#else
+  return cudaSuccess;
+#endif
+}
+
+}  // namespace su3g
