@@ -48,8 +48,12 @@ constexpr int kCoopSites = 8192;
 
 // Pairs of FHKP counters per chain (their sums are the totals).
 constexpr int kCounterSlots = 32;
-// A measurement's partial sums: at most this many CTAs per layer.
-constexpr int kMeasureCtas = 1024;
+// A measurement's partial sums: at most this many CTAs per layer (one wave: 5
+// per SM, FP64 3).
+constexpr int kMeasureCtas = 760, kMeasureCtasF64 = 456;
+// Float measurements of at most this many sites per colour take eight lanes
+// per site.
+constexpr int kSplitSites = 4096;
 
 // Results per measurement slot: [total, space, time, poly_re, poly_im].
 constexpr int kMeasVals = 5;

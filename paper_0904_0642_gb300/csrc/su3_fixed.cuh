@@ -48,8 +48,9 @@
 
 namespace su3g {
 
-// The high word of the largest accepted double magnitude (1.0625).
-constexpr uint32_t kElemMaxHi = 0x3FF10000u;
+// The high word of the largest accepted double magnitude (1.0625), and its
+// bits as a float.
+constexpr uint32_t kElemMaxHi = 0x3FF10000u, kElemMaxFloat = 0x3F880000u;
 // The same bound on the high limb (units 2^-28), a margin of one for l < 0.
 constexpr int32_t kElemMaxLimb = (17 << 24) + 1;
 
@@ -80,6 +81,7 @@ struct FxRange {
   int32_t dpos = 0;
   uint32_t dneg = 0;
   int32_t hmax = 0, hmin = 0;
+  // high words of doubles, or floats
   SU3_HD void doubles(int32_t hi0, int32_t hi1) {
 #ifdef __CUDA_ARCH__
     dpos = __vimax3_s32(dpos, hi0, hi1);
@@ -102,9 +104,9 @@ struct FxRange {
     }
 #endif
   }
-  SU3_HD bool ok() const {
-    return dpos <= (int32_t)kElemMaxHi && dneg <= (0x80000000u | kElemMaxHi) && hmax <= kElemMaxLimb &&
-           hmin >= -kElemMaxLimb;
+  // top: the high word of the largest accepted double, or its bits as a float
+  SU3_HD bool ok(uint32_t top = kElemMaxHi) const {
+    return dpos <= (int32_t)top && dneg <= (0x80000000u | top) && hmax <= kElemMaxLimb && hmin >= -kElemMaxLimb;
   }
 };
 
@@ -167,16 +169,33 @@ SU3_HD int clz32(uint32_t x) {
 // 1026 - e (zero and subnormals shift out), negative values as the ones'
 // complement.  The conversion instruction is emulated on this GPU in about
 // four times as many instructions.
-SU3_HD Fx fx_of(double x) {
-  const uint32_t hi = (uint32_t)dbl_hi(x), lo = dbl_lo(x);
-  const int q = 1026 - (int)((hi >> 20) & 0x7FFu);
-  const uint32_t H = (hi << 11 | lo >> 21) | 0x80000000u, L = lo << 11;
-  const uint32_t s = (uint32_t)((int32_t)hi >> 31);
+SU3_HD Fx fx_of_mantissa(uint32_t H, uint32_t L, int q, uint32_t s) {
   const int q2 = q > 32 ? q - 32 : 0;
   const uint32_t vh = shr0(H, (uint32_t)q) ^ s;
   const uint32_t vl = shr0(shift_r(L, H, (uint32_t)(q < 32 ? q : 32)), (uint32_t)q2) ^ s;
   return {(int32_t)(vh + (vl >> 31)), (int32_t)vl};
 }
+SU3_HD Fx fx_of(double x) {
+  const uint32_t hi = (uint32_t)dbl_hi(x), lo = dbl_lo(x);
+  return fx_of_mantissa((hi << 11 | lo >> 21) | 0x80000000u, lo << 11, 1026 - (int)((hi >> 20) & 0x7FFu),
+                        (uint32_t)((int32_t)hi >> 31));
+}
+// The same for a float.
+SU3_HD uint32_t flt_bits(float x) {
+  uint32_t u;
+#ifdef __CUDA_ARCH__
+  u = __float_as_uint(x);
+#else
+  std::memcpy(&u, &x, 4);
+#endif
+  return u;
+}
+SU3_HD Fx fx_of(float x) {
+  const uint32_t u = flt_bits(x);
+  return fx_of_mantissa((u << 8) | 0x80000000u, 0u, 130 - (int)((u >> 23) & 0xFFu), (uint32_t)((int32_t)u >> 31));
+}
+// v 2^-60 as a float, rounded to nearest even.
+SU3_HD float flt_of(int64_t v) { return (float)v * 0x1p-60f; }
 
 // v 2^-e as a double, rounded to nearest (halves away from zero).
 SU3_HD double dbl_of(int64_t v, int e) {
@@ -364,6 +383,29 @@ SU3_HD void staple_f(FSum &A, const Fc (&X)[2][3], const FM3 &Y, const FM3 &G, b
   acc_su3_2rows_f(A, P, rg);
 }
 
+// Re Tr(P Q^+) of two SU(3) matrices given by rows 0, 1 (plaquette_at in
+// su3_site.cuh), in units 2^-60.
+SU3_HD int64_t trace_nd_f(const FM3 &P, const FM3 &Q, FxRange &rg) {
+  Fc G[2][2];  // <P_k, Q_l>
+#pragma unroll
+  for (int l = 0; l < 2; ++l) {
+    const FcN q[3] = {with_neg_re(Q.e[l][0]), with_neg_re(Q.e[l][1]), with_neg_re(Q.e[l][2])};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      FxAcc re = {0, kHalf60}, im = {0, kHalf60};
+#pragma unroll
+      for (int j = 0; j < 3; ++j) cmac_nc_f(re, im, q[j], P.e[k][j]);
+      store60(G[k][l], re, im, rg);
+    }
+  }
+  FxAcc t = {0, kHalf60};
+  fmac(t, G[0][0].re, G[1][1].re);
+  fmac(t, fx_neg(G[0][0].im), G[1][1].im);
+  fmac(t, fx_neg(G[0][1].re), G[1][0].re);
+  fmac(t, G[0][1].im, G[1][0].im);
+  return fold60(t) + fx_val(G[0][0].re) + fx_val(G[1][1].re);
+}
+
 // The staple sum as a factor: units 2^-56, so that the twelve products of a
 // projection stay inside 64 bits.
 SU3_HD FM3 factor56(const FSum &A) {
@@ -528,6 +570,100 @@ SU3_HD int64_t sqrt_u64(uint64_t p, int &e) {
   const Fx n = fx_split((int64_t)((p << z) >> 4));  // [1/4, 1)
   e = z >> 1;
   return fx_mul(n, fx_split(rsqrt_fx(n)));
+}
+
+// ------------------------------------------------------------------ re-unitarisation
+// Gram-Schmidt of rows 0, 1; false when a squared norm leaves [1/4, 4).
+
+SU3_HD int64_t norm2_f(const Fc (&a)[3]) {
+  FxAcc n = {0, kHalf60};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    fmac(n, a[k].re, a[k].re);
+    fmac(n, a[k].im, a[k].im);
+  }
+  return fold60(n);
+}
+SU3_HD bool norm2_ok(int64_t n) { return n >= (1ll << 58) && n < (1ll << 62); }
+
+// q = sum_k conj(a_k) b_k
+SU3_HD void inner_f(const Fc (&a)[3], const Fc (&b)[3], int64_t &qr, int64_t &qi) {
+  FxAcc re = {0, kHalf60}, im = {0, kHalf60};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    fmac(re, a[k].re, b[k].re);
+    fmac(re, a[k].im, b[k].im);
+    fmac(im, a[k].re, b[k].im);
+    fmac(im, fx_neg(a[k].im), b[k].re);
+  }
+  qr = fold60(re);
+  qi = fold60(im);
+}
+
+// n^(-1/2): to rounding level (FLOAT = false), or as the double-precision form
+// takes it for float storage - a float seed and one Newton step, exact to
+// ~1e-13 - so that the stored floats are that form's.
+template <bool FLOAT>
+SU3_HD int64_t reunit_rsqrt_fx(int64_t n) {
+  const Fx nf = fx_split(n);
+  if (!FLOAT) return rsqrt_fx(nf);
+  const int64_t y = fx_val(fx_of(rsqrt_seed(flt_of(n))));
+  const Fx yf = fx_split(y);
+  const int64_t e = (1ll << 60) - fx_mul(fx_split(fx_mul(nf, yf)), yf);  // 1 - n y^2
+  return y + fx_mul(fx_split(e >> 1), yf);
+}
+
+template <bool FLOAT>
+SU3_HD bool reunit_f(FM3 &m, FxRange &rg) {
+  Fc(&a)[3] = m.e[0], (&b)[3] = m.e[1];
+  const int64_t n1 = norm2_f(a);
+  if (!norm2_ok(n1)) return false;
+  const Fx s1 = fx_split(reunit_rsqrt_fx<FLOAT>(n1));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) a[k] = {fx_split(fx_mul(a[k].re, s1)), fx_split(fx_mul(a[k].im, s1))};
+  int64_t qr, qi;
+  inner_f(a, b, qr, qi);
+  const Fx pr = fx_split(-qr), pi = fx_split(-qi), pn = fx_split(qi);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {  // b - q a
+    FxAcc re = {0, kHalf60}, im = {0, kHalf60};
+    fmac(re, pr, a[k].re);
+    fmac(re, pn, a[k].im);
+    fmac(im, pr, a[k].im);
+    fmac(im, pi, a[k].re);
+    b[k] = {fx_split(fx_val(b[k].re) + fold60(re)), fx_split(fx_val(b[k].im) + fold60(im))};
+  }
+  const int64_t n2 = norm2_f(b);
+  if (!norm2_ok(n2)) return false;
+  const Fx s2 = fx_split(reunit_rsqrt_fx<FLOAT>(n2));
+#pragma unroll
+  for (int k = 0; k < 3; ++k) b[k] = {fx_split(fx_mul(b[k].re, s2)), fx_split(fx_mul(b[k].im, s2))};
+  third_row_f(m, rg);
+  return true;
+}
+
+// The factors of reunit_rows2_f (su3_site.cuh) from two float rows: e1 = s1 -
+// 1, p = s1 <r1, r2>, e2 = s2 - 1 with s1 = n1^(-1/2), s2 = (n2 - |p|^2)^(-1/2).
+SU3_HD bool reunit_factors_f(const Fc (&a)[3], const Fc (&b)[3], float &e1, float &pr, float &pi, float &e2) {
+  const int64_t n1 = norm2_f(a);
+  if (!norm2_ok(n1)) return false;
+  const int64_t s1 = reunit_rsqrt_fx<true>(n1);
+  int64_t qr, qi;
+  inner_f(a, b, qr, qi);
+  const Fx s1f = fx_split(s1);
+  const int64_t vr = fx_mul(fx_split(qr), s1f), vi = fx_mul(fx_split(qi), s1f);
+  FxAcc p2 = {0, kHalf60};
+  const Fx fr = fx_split(vr), fi = fx_split(vi);
+  fmac(p2, fr, fr);
+  fmac(p2, fi, fi);
+  const int64_t n2 = norm2_f(b) - fold60(p2);
+  if (!norm2_ok(n2)) return false;
+  const int64_t s2 = reunit_rsqrt_fx<true>(n2);
+  e1 = flt_of(s1 - (1ll << 60));
+  pr = flt_of(vr);
+  pi = flt_of(vi);
+  e2 = flt_of(s2 - (1ll << 60));
+  return true;
 }
 
 // ------------------------------------------------------------------ the draw

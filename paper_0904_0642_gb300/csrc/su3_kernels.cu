@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
   __shared__ ChainDesc sd;
   __shared__ ChainState ss;  // the current chain's current state
   __shared__ int s_par;      // the state slot that holds the current states
-  __shared__ double s_red[32 * kPartVals];
+  __shared__ double s_red[32];
   // Launched as a programmatic dependent (pdl), this tick may be scheduled
   // before the previous kernel of the stream has finished: wait for its
   // completion and memory before touching anything, then let the next tick
@@ -606,7 +606,7 @@ static __device__ __align__(256) double g_noalloc_partials[kNoAllocTiles * kPart
 
 template <class S>
 __global__ void __launch_bounds__(256) k_measure_noalloc(ChainDesc d, double *partials) {
-  __shared__ double s_red[32 * kPartVals];
+  __shared__ double s_red[32];
   const int total = d.tiles_per_layer * d.nlayers;
   for (int lt = blockIdx.x; lt < total; lt += gridDim.x) {
     const int layer = lt / d.tiles_per_layer;

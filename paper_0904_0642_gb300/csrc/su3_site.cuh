@@ -796,6 +796,23 @@ __device__ __forceinline__ M3<double> load_rows2_d(const typename S::Vec *p, int
   return m;
 }
 
+// The end of reunit_rows2_f: the corrections applied in float.
+__device__ __forceinline__ void reunit_apply_f(M3<float> &m, float e1, float pr, float pi, float e2) {
+  C<float> *r1 = m.e[0], *r2 = m.e[1];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const C<float> a = r1[k];
+    r1[k] = {fm(a.re, e1, a.re), fm(a.im, e1, a.im)};
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    // c = -p r1'_k, then r2''_k = r2_k + (c (1 + e2) + r2_k e2), one rounding
+    const C<float> a = r1[k], b = r2[k];
+    const float cr = fm(pi, a.im, -pr * a.re), ci = fm(-pi, a.re, -pr * a.im);
+    r2[k] = {b.re + fm(b.re, e2, fm(cr, e2, cr)), b.im + fm(b.im, e2, fm(ci, e2, ci))};
+  }
+}
+
 // The double-precision Gram-Schmidt of two float rows r1, r2, applied in
 // float.  The norms and the inner product are summed in double from the
 // float elements (products of floats are exact in double):
@@ -838,71 +855,78 @@ __device__ __forceinline__ void reunit_rows2_f(M3<float> &m) {
   n2 = fm(-pdr, pdr, n2);
   n2 = fm(-pdi, pdi, n2);
   const double s2 = rsqrt_d<1>(n2);
-  const float e1 = d2f_bits(s1 - 1.0), e2 = d2f_bits(s2 - 1.0);
-  const float pr = d2f_bits(pdr), pi = d2f_bits(pdi);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const C<float> a = r1[k];
-    r1[k] = {fm(a.re, e1, a.re), fm(a.im, e1, a.im)};
-  }
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    // c = -p r1'_k, then r2''_k = r2_k + (c (1 + e2) + r2_k e2), one rounding
-    const C<float> a = r1[k], b = r2[k];
-    const float cr = fm(pi, a.im, -pr * a.re), ci = fm(-pi, a.re, -pr * a.im);
-    r2[k] = {b.re + fm(b.re, e2, fm(cr, e2, cr)), b.im + fm(b.im, e2, fm(ci, e2, ci))};
+  reunit_apply_f(m, d2f_bits(s1 - 1.0), d2f_bits(pdr), d2f_bits(pdi), d2f_bits(s2 - 1.0));
+}
+
+// One stored link in double precision, out of line: links whose rows are far
+// from orthonormal (reunit_link) only.
+template <class S>
+static __device__ __noinline__ void reunit_link_general(typename S::Vec *p, int Vh, int js) {
+  if constexpr (S::kTwoRows) {
+    M3<float> m = S::load2(p, Vh, js);
+    reunit_rows2_f(m);
+    S::store(p, Vh, js, m);
+  } else {
+    constexpr int kNewton = sizeof(typename S::R) == 4 ? 1 : 2;  // float storage: one Newton step suffices
+    M3<double> m = load_rows2_d<S>(p, Vh, js);
+    reunit_d<kNewton, true>(m);
+    S::store(p, Vh, js, to_storage<typename S::R>(m));
   }
 }
 
-// Two links per step: their Gram-Schmidt chains are independent.
-template <class S, bool SUB = false>
-__device__ __forceinline__ void reunit_site(const ChainDesc &d, int layer, int jj) {
-  constexpr bool kTwoRows = S::kTwoRows;  // the 12-real form keeps rows 1, 2 only
-  constexpr int kNewton = sizeof(typename S::R) == 4 ? 1 : 2;  // float storage: one Newton step suffices
-  const int Vh = d.Vh;
-  if constexpr (std::is_same<S, StoreF32x12>::value) {
-    // two-row float storage: the double Gram-Schmidt applied in float
-    for (int colour = 0; colour < 2; ++colour) {
-      const int js = SUB ? (site_of<true>(d, layer, colour, jj).s >> 1) : jj;
-      int mu = 0;
-#pragma unroll 1
-      for (; mu + 1 < d.D; mu += 2) {
-        typename S::Vec *p0 = plane_ptr<S>(d, layer, colour, mu), *p1 = plane_ptr<S>(d, layer, colour, mu + 1);
-        M3<float> m0 = S::load2(p0, Vh, js), m1 = S::load2(p1, Vh, js);
-        reunit_rows2_f(m0);
-        reunit_rows2_f(m1);
-        S::store(p0, Vh, js, m0);
-        S::store(p1, Vh, js, m1);
-      }
-      if (mu < d.D) {
-        typename S::Vec *p = plane_ptr<S>(d, layer, colour, mu);
-        M3<float> m = S::load2(p, Vh, js);
-        reunit_rows2_f(m);
-        S::store(p, Vh, js, m);
+// Re-unitarise one stored link: the sums, products and reciprocal square roots
+// in fixed point (errors below 2^-57, absolute; the double-precision pipe ran
+// at 90 % of its rate here), the result rounded to the storage precision, or
+// applied to two-row float storage as in reunit_rows2_f.
+template <class S>
+__device__ __forceinline__ void reunit_link(typename S::Vec *p, int Vh, int js) {
+  using R = typename S::R;
+  M3<R> m = S::load2(p, Vh, js);
+  FxRange rg;
+  FM3 f;
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if constexpr (sizeof(R) == 4) {
+        rg.doubles(__float_as_int(m.e[i][k].re), __float_as_int(m.e[i][k].im));
+        f.e[i][k] = {fx_of(m.e[i][k].re), fx_of(m.e[i][k].im)};
+      } else {
+        f.e[i][k] = fc_of(m.e[i][k].re, m.e[i][k].im, rg);
       }
     }
-  } else {
-    for (int colour = 0; colour < 2; ++colour) {
-      const int js = SUB ? (site_of<true>(d, layer, colour, jj).s >> 1) : jj;
-      int mu = 0;
-#pragma unroll 1
-      for (; mu + 1 < d.D; mu += 2) {
-        typename S::Vec *p0 = plane_ptr<S>(d, layer, colour, mu), *p1 = plane_ptr<S>(d, layer, colour, mu + 1);
-        M3<double> m0 = load_rows2_d<S>(p0, Vh, js);
-        M3<double> m1 = load_rows2_d<S>(p1, Vh, js);
-        reunit_d<kNewton, !kTwoRows>(m0);
-        reunit_d<kNewton, !kTwoRows>(m1);
-        S::store(p0, Vh, js, to_storage<typename S::R>(m0));
-        S::store(p1, Vh, js, to_storage<typename S::R>(m1));
-      }
-      if (mu < d.D) {
-        typename S::Vec *p = plane_ptr<S>(d, layer, colour, mu);
-        M3<double> m = load_rows2_d<S>(p, Vh, js);
-        reunit_d<kNewton, !kTwoRows>(m);
-        S::store(p, Vh, js, to_storage<typename S::R>(m));
-      }
+  const bool in = rg.ok(sizeof(R) == 4 ? kElemMaxFloat : kElemMaxHi);
+  FxRange rr;
+  if constexpr (S::kTwoRows) {
+    float e1, pr, pi, e2;
+    if (in && reunit_factors_f(f.e[0], f.e[1], e1, pr, pi, e2)) {
+      reunit_apply_f(m, e1, pr, pi, e2);
+      S::store(p, Vh, js, m);
+      return;
     }
+  } else if (in && reunit_f<sizeof(R) == 4>(f, rr) && rr.ok()) {
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int64_t re = fx_val(f.e[i][k].re), im = fx_val(f.e[i][k].im);
+        if constexpr (sizeof(R) == 4)
+          m.e[i][k] = {flt_of(re), flt_of(im)};
+        else
+          m.e[i][k] = {dbl_of(re, 60), dbl_of(im, 60)};
+      }
+    S::store(p, Vh, js, m);
+    return;
   }
+  reunit_link_general<S>(p, Vh, js);
+}
+
+// All links of the two sites of a checkerboard index (many-chain launches).
+template <class S>
+__device__ __forceinline__ void reunit_site(const ChainDesc &d, int layer, int jj) {
+#pragma unroll 1
+  for (int cm = 0; cm < 2 * d.D; ++cm)
+    reunit_link<S>(plane_ptr<S>(d, layer, cm / d.D, cm % d.D), d.Vh, jj);
 }
 
 // ------------------------------------------------------------------ measurements
@@ -947,6 +971,65 @@ __device__ __forceinline__ typename S::R plaquette_at(const ChainDesc &d, const 
   return tr;
 }
 
+// plaquette_at for FP64 links in fixed point: Re Tr in units 2^-60, one
+// plaquette at a time (mu, nu are run-time values: the code is short).
+// false: a link is out of the fixed-point range.
+template <bool SUB>
+__device__ __forceinline__ bool plaquette_fixed(const ChainDesc &d, const SiteGeo &g, int colour, int mu, int nu,
+                                                int64_t &tr) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh, layer = g.layer, js = g.s >> 1, oc = colour ^ 1;
+  int offp, flp, offn, fln;
+  step_fwd(d, sel(g.x, mu), mu, offp, flp);
+  step_fwd(d, sel(g.x, nu), nu, offn, fln);
+  const S::Vec *pm = plane_ptr<S>(d, layer, colour, mu), *pn = plane_ptr<S>(d, layer, colour, nu);
+  FxRange rg;
+  FM3 Y, P, Q;
+  Fc row[3];
+  load_f(plane_ptr<S>(d, lflip<SUB>(d, layer, flp), oc, nu), Vh, (g.s + offp) >> 1, Y, rg);  // U_nu(x+mu)
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    load_row_f(pm, Vh, js, i, row, rg);
+    row_nn_f(P, i, row, Y, rg);
+  }
+  load_f(plane_ptr<S>(d, lflip<SUB>(d, layer, fln), oc, mu), Vh, (g.s + offn) >> 1, Y, rg);  // U_mu(x+nu)
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    load_row_f(pn, Vh, js, i, row, rg);
+    row_nn_f(Q, i, row, Y, rg);
+  }
+  tr = trace_nd_f(P, Q, rg);
+  return rg.ok();
+}
+
+// The same in double, out of line.
+template <bool SUB>
+static __device__ __noinline__ double plaquette_general(const ChainDesc *d, int layer, int colour, int jj, int mu,
+                                                        int nu) {
+  using S = StoreF64x18;
+  const SiteGeo g = site_of<SUB>(*d, layer, colour, jj);
+  return plaquette_at<S, SUB>(*d, g, colour, mu, nu, sel(g.x, mu), sel(g.x, nu),
+                              S::load2(plane_ptr<S>(*d, layer, colour, mu), d->Vh, g.s >> 1));
+}
+
+// Sums of plaquettes: integers in units 2^-48 (at most 2^11 plaquettes per
+// sum), and in double those of links out of range.
+struct PlaquetteSum {
+  int64_t v = 0;
+  double general = 0.0;
+  __device__ __forceinline__ double value() const { return dbl_of(v, 48) + general; }
+};
+
+template <bool SUB>
+__device__ __forceinline__ void add_plaquette(const ChainDesc &d, const SiteGeo &g, int colour, int jj, int mu, int nu,
+                                              PlaquetteSum &s) {
+  int64_t tr;
+  if (plaquette_fixed<SUB>(d, g, colour, mu, nu, tr))
+    s.v += (tr + (1 << 11)) >> 12;
+  else
+    s.general += plaquette_general<SUB>(&d, g.layer, colour, jj, mu, nu);
+}
+
 // The plaquettes of one site: Re Tr summed in the storage precision, split
 // into space-like and time-like (the 1/3 is applied with the counts).  The
 // loop over mu is unrolled so that the loads of several plaquettes are in
@@ -970,6 +1053,32 @@ __device__ __forceinline__ void site_plaquettes(const ChainDesc &d, const SiteGe
       if (nu == D - 1) pt += p; else ps += p;
     }
   }
+}
+
+// The same with eight lanes per site: lane p takes plane p (its indices are
+// run-time values), the sums are taken in the order of site_plaquettes.
+// Called by whole warps; valid false: the lane's site is a repeated one.
+template <class S, bool SUB = false>
+__device__ __forceinline__ void site_plaquettes_split(const ChainDesc &d, const SiteGeo &g, int colour,
+                                                      typename S::R &ps, typename S::R &pt) {
+  using R = typename S::R;
+  const int D = d.D, lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
+  const int np = D * (D - 1) / 2;
+  int mu = 0, nu = l8 < np ? l8 + 1 : 1;  // planes (0,1), (0,2), .., (1,2), ..
+  while (nu >= D) {
+    nu -= D - 2 - mu;
+    ++mu;
+  }
+  const R p = plaquette_at<S, SUB>(d, g, colour, mu, nu, sel(g.x, mu), sel(g.x, nu),
+                                   S::load2(plane_ptr<S>(d, g.layer, colour, mu), d.Vh, g.s >> 1));
+  ps = R(0);
+  pt = R(0);
+  int k = 0;
+  for (int m = 0; m + 1 < D; ++m)
+    for (int n = m + 1; n < D; ++n, ++k) {
+      const R q = __shfl_sync(0xffffffffu, p, base + k);
+      if (n == D - 1) pt += q; else ps += q;
+    }
 }
 
 // Tr of the Polyakov line through a site with x^D = 0 (the line follows the
@@ -1005,6 +1114,62 @@ __device__ __forceinline__ C<typename S::R> polyakov_line(const ChainDesc &d, co
   return {P.e[0][0].re + P.e[1][1].re + p33.re, P.e[0][0].im + P.e[1][1].im + p33.im};
 }
 
+// The same for FP64 links in fixed point (units 2^-60); false: out of range.
+template <bool SUB>
+__device__ __forceinline__ bool polyakov_fixed(const ChainDesc &d, const SiteGeo &g, int colour, int64_t &re,
+                                               int64_t &im) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh, t = d.D - 1, layer = g.layer;
+  FxRange rg;
+  FM3 P, Y;
+  load_row_f(plane_ptr<S>(d, layer, colour, t), Vh, g.s >> 1, 0, P.e[0], rg);
+  load_row_f(plane_ptr<S>(d, layer, colour, t), Vh, g.s >> 1, 1, P.e[1], rg);
+  int cs = g.s, cl = layer, cc = colour, xt = 0;
+#pragma unroll 1
+  while (true) {
+    int off, fl;
+    step_fwd(d, xt, t, off, fl);
+    cs += off;
+    cl = lflip<SUB>(d, cl, fl);
+    cc ^= 1;
+    xt = (xt == d.dims[t] - 1) ? 0 : xt + 1;
+    if (cs == g.s && cl == layer) break;
+    load_f(plane_ptr<S>(d, cl, cc, t), Vh, cs >> 1, Y, rg);
+    FM3 N;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) row_nn_f(N, i, P.e[i], Y, rg);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) P.e[i][k] = N.e[i][k];
+  }
+  // conj(P_11 P_22 - P_12 P_21)
+  FxAcc x = {0, kHalf60}, y = {0, kHalf60};
+  const Fc r = P.e[0][1];
+  cross_f(x, y, P.e[0][0], fx_neg(P.e[0][0].im), P.e[1][1], r, fx_neg(r.re), fx_neg(r.im), P.e[1][0]);
+  re = fx_val(P.e[0][0].re) + fx_val(P.e[1][1].re) + fold60(x);
+  im = fx_val(P.e[0][0].im) + fx_val(P.e[1][1].im) - fold60(y);
+  return rg.ok();
+}
+
+template <bool SUB>
+static __device__ __noinline__ C<double> polyakov_general(const ChainDesc *d, int layer, int colour, int jj) {
+  return polyakov_line<StoreF64x18, SUB>(*d, site_of<SUB>(*d, layer, colour, jj), colour);
+}
+
+// A line's trace in double.
+template <class S, bool SUB = false>
+__device__ __forceinline__ C<double> line_trace(const ChainDesc &d, const SiteGeo &g, int colour, int jj) {
+  if constexpr (std::is_same<S, StoreF64x18>::value) {
+    int64_t re, im;
+    if (polyakov_fixed<SUB>(d, g, colour, re, im)) return {dbl_of(re, 60), dbl_of(im, 60)};
+    return polyakov_general<SUB>(&d, g.layer, colour, jj);
+  } else {
+    const C<typename S::R> l = polyakov_line<S, SUB>(d, g, colour);
+    return {to_double(l.re), to_double(l.im)};
+  }
+}
+
 // Per thread: the two sites of checkerboard index jj (both colours), and the
 // Polyakov lines that start at them; accumulated in double.
 template <class S>
@@ -1013,55 +1178,67 @@ __device__ __forceinline__ void measure_site(const ChainDesc &d, int layer, int 
 #pragma unroll 1
   for (int colour = 0; colour < 2; ++colour) {
     const SiteGeo g = site_of<false>(d, layer, colour, jj);
-    R ps, pt;
-    site_plaquettes<S>(d, g, colour, ps, pt);
-    acc[0] += to_double(ps);
-    acc[1] += to_double(pt);
+    if constexpr (std::is_same<S, StoreF64x18>::value) {
+      PlaquetteSum ps, pt;
+#pragma unroll 1
+      for (int mu = 0; mu + 1 < d.D; ++mu)
+#pragma unroll 1
+        for (int nu = mu + 1; nu < d.D; ++nu) add_plaquette<false>(d, g, colour, jj, mu, nu, nu == d.D - 1 ? pt : ps);
+      acc[0] += ps.value();
+      acc[1] += pt.value();
+    } else {
+      R ps, pt;
+      site_plaquettes<S>(d, g, colour, ps, pt);
+      acc[0] += to_double(ps);
+      acc[1] += to_double(pt);
+    }
     if (sel(g.x, d.D - 1) == 0) {
-      const C<R> l = polyakov_line<S>(d, g, colour);
-      acc[2] += to_double(l.re);
-      acc[3] += to_double(l.im);
+      const C<double> l = line_trace<S>(d, g, colour, jj);
+      acc[2] += l.re;
+      acc[3] += l.im;
     }
   }
 }
 
-// Block reduction of kPartVals doubles in a fixed order (warp shuffles, then
-// warp 0 over the warp sums).  Result valid in thread 0.
-__device__ __forceinline__ void block_reduce(double v[kPartVals], double *smem /* [32][kPartVals] */) {
+// Block reduction of kPartVals doubles in a fixed order.  Result valid in
+// thread 0.  Within a warp the four values are spread over the lanes while
+// they are summed (six additions instead of twenty: a double addition takes
+// 16 clocks of the SM per warp); then warp 0 sums the warps (at most eight).
+__device__ __forceinline__ void block_reduce(double v[kPartVals], double *smem /* [32] */) {
+  static_assert(kPartVals == 4, "the value index is two lane bits");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+  const bool b1 = lane & 16, b0 = lane & 8;
+  double x0 = b1 ? v[2] : v[0], x1 = b1 ? v[3] : v[1];
+  x0 += __shfl_xor_sync(0xffffffffu, b1 ? v[0] : v[2], 16);
+  x1 += __shfl_xor_sync(0xffffffffu, b1 ? v[1] : v[3], 16);
+  double x = b0 ? x1 : x0;
+  x += __shfl_xor_sync(0xffffffffu, b0 ? x0 : x1, 8);
 #pragma unroll
-  for (int k = 0; k < kPartVals; ++k)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < kPartVals; ++k) smem[warp * kPartVals + k] = v[k];
+  for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if ((lane & 7) == 0) smem[warp * kPartVals + (b1 ? 2 : 0) + (b0 ? 1 : 0)] = x;
   __syncthreads();
   if (warp == 0) {
+    double y = lane < nw * kPartVals ? smem[lane] : 0.0;
 #pragma unroll
-    for (int k = 0; k < kPartVals; ++k) {
-      double x = lane < nw ? smem[lane * kPartVals + k] : 0.0;
+    for (int o = kPartVals; o < 32; o <<= 1)
+      if (o < nw * kPartVals) y += __shfl_xor_sync(0xffffffffu, y, o);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      v[k] = x;
-    }
+    for (int k = 0; k < kPartVals; ++k) v[k] = __shfl_sync(0xffffffffu, y, k);
   }
   __syncthreads();
 }
 
-// The measured values [total, space, time, poly_re, poly_im] from the sums
-// over `layers` layers (they hold Re Tr and Tr: the counts carry the factor 3).
-__device__ __forceinline__ void measured_values(const ChainDesc &d, const double v[kPartVals], double layers,
-                                                double *o) {
+// Value k of [total, space, time, poly_re, poly_im] from the sums over
+// `layers` layers (they hold Re Tr and Tr: the counts carry the factor 3).
+__device__ __forceinline__ double measured_value(const ChainDesc &d, const double v[kPartVals], double layers, int k) {
   const int D = d.D;
   const double np_s = 3.0 * d.V * (D - 1) * (D - 2) / 2, np_t = 3.0 * d.V * (D - 1);
-  // Polyakov lines are not taken inside sublattice boxes with divided time
+  // Polyakov lines are not taken inside sublattice boxes with divided time:
+  // the values are NaN
   const double nl = d.hpad[D - 1] ? __longlong_as_double(0x7ff8000000000000ll) : 3.0 * d.spatial_per_layer;
-  o[0] = (v[0] + v[1]) / (layers * (np_s + np_t));
-  o[1] = np_s > 0 ? v[0] / (layers * np_s) : 0.0;
-  o[2] = v[1] / (layers * np_t);
-  o[3] = v[2] / (layers * nl);  // NaN when nl is
-  o[4] = v[3] / (layers * nl);
+  const double num = k == 0 ? v[0] + v[1] : (k == 1 ? v[0] : (k == 2 ? v[1] : (k == 3 ? v[2] : v[3])));
+  const double den = k == 0 ? np_s + np_t : (k == 1 ? np_s : (k == 2 ? np_t : nl));
+  return k == 1 && !(np_s > 0) ? 0.0 : num / (layers * den);
 }
 
 // Sum the tile partials of one chain per layer (one warp, fixed order) and
@@ -1081,15 +1258,15 @@ __device__ __forceinline__ void finalize_measure(const ChainDesc &d, const doubl
       v[k] = __shfl_sync(0xffffffffu, v[k], 0);
       whole[k] += v[k];
     }
-    if (lane == 0) measured_values(d, v, 1.0, out + layer * kMeasVals);
+    if (lane < kMeasVals) out[layer * kMeasVals + lane] = measured_value(d, v, 1.0, lane);
   }
-  if (lane == 0) measured_values(d, whole, (double)d.nlayers, out + d.nlayers * kMeasVals);
+  if (lane < kMeasVals) out[d.nlayers * kMeasVals + lane] = measured_value(d, whole, (double)d.nlayers, lane);
 }
 
 // The action bookkeeping restarts at this measurement (a chain whose links
 // were replaced asks for it): the measurement becomes the reference and
 // the booked changes restart from zero.  Warp-collective; the measurement
-// was written by lane 0 of this warp.
+// was written by lanes of this warp.
 __device__ __forceinline__ void restart_bookkeeping(const ChainDesc &d, const double *out) {
   __syncwarp();
   const int lane = threadIdx.x & 31;
