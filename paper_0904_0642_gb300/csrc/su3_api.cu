@@ -276,6 +276,7 @@ struct Chain {
   ChainState state{};
   void *links = nullptr;
   bool own_links = false;
+  void *scratch = nullptr;  // one block: the five arrays below
   double *results = nullptr;
   double *partials = nullptr;
   unsigned long long *counters = nullptr;
@@ -602,28 +603,76 @@ struct Engine {
     d_tile_chain = nullptr;
     d_meas_out = nullptr;
     h_pinned = nullptr;
+    if (pool) {
+      if (stream) cudaStreamSynchronize(stream);
+      cudaMemPoolDestroy(pool);
+    }
+    pool = nullptr;
     if (own_stream && stream) cudaStreamDestroy(stream);
     stream = nullptr;
     own_stream = false;
   }
 
-  static void free_chain(Chain &ch) {
-    if (ch.own_links) cudaFree(ch.links);
+  // A server's chains come and go: their memory comes from a pool of its own
+  // (allocations and frees in stream order, no device-wide waits), which
+  // keeps at most `kPoolKept` bytes and is destroyed with the server.
+  cudaMemPool_t pool = nullptr;
+  static constexpr uint64_t kPoolKept = 1ull << 30;
+
+  su3_status make_pool(size_t most) {
+    int dev = 0;
+    CU(cudaGetDevice(&dev));
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    CU(cudaMemPoolCreate(&pool, &props));
+    uint64_t keep = std::min<uint64_t>(kPoolKept, most);
+    CU(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+    return SU3_OK;
+  }
+
+  template <class T>
+  cudaError_t chain_alloc(T **p, size_t bytes) {
+    void *v = nullptr;
+    cudaError_t e;
+    if (!pool) {
+      e = cudaMalloc(&v, bytes);
+    } else {
+      e = cudaMallocFromPoolAsync(&v, bytes, pool, stream);
+      if (e == cudaErrorMemoryAllocation) {  // what the pool keeps in pieces may be enough in one
+        cudaGetLastError();
+        cudaStreamSynchronize(stream);
+        cudaMemPoolTrimTo(pool, 0);
+        e = cudaMallocFromPoolAsync(&v, bytes, pool, stream);
+      }
+    }
+    *p = static_cast<T *>(v);
+    return e;
+  }
+  // Staging for link input and output, freed in stream order.
+  cudaError_t canon_alloc(double **p, size_t bytes) {
+    return pool ? chain_alloc(p, bytes) : cudaMallocAsync(p, bytes, stream);
+  }
+  void chain_free(void *p) {
+    if (!p) return;
+    if (pool)
+      cudaFreeAsync(p, stream);
+    else
+      cudaFree(p);
+  }
+
+  void free_chain(Chain &ch) {
+    if (ch.own_links) chain_free(ch.links);
+    chain_free(ch.scratch);
     cudaFree(ch.plain);
     cudaFree(ch.d_pdesc);
     cudaFree(ch.d_halo);
     ch.plain = nullptr;
     ch.d_pdesc = nullptr;
     ch.d_halo = nullptr;
-    cudaFree(ch.results);
-    cudaFree(ch.partials);
-    cudaFree(ch.counters);
-    cudaFree(ch.action_slots);
-    ch.action_slots = nullptr;
-    cudaFree(ch.ref_meas);
-    ch.ref_meas = nullptr;
-    ch.links = nullptr;
-    ch.results = ch.partials = nullptr;
+    ch.scratch = ch.links = nullptr;
+    ch.results = ch.partials = ch.action_slots = ch.ref_meas = nullptr;
     ch.counters = nullptr;
   }
 
@@ -640,7 +689,7 @@ struct Engine {
     CU(cudaMemsetAsync(d_hdr, 0, sizeof(EngineHeader), stream));
     CU(cudaMalloc(&d_ctl, sizeof(ChainCtl)));
     CU(cudaMemsetAsync(d_ctl, 0, sizeof(ChainCtl), stream));
-    CU(cudaMallocHost(&h_pinned, 4096));
+    CU(cudaMallocHost(&h_pinned, kRetireBatch * kRetireDoubles * sizeof(double)));
     return SU3_OK;
   }
 
@@ -676,7 +725,7 @@ struct Engine {
       ch.links = cfg.link_buffer;
       ch.own_links = false;
     } else {
-      cudaError_t e = cudaMalloc(&ch.links, ch.link_bytes);
+      cudaError_t e = chain_alloc(&ch.links, ch.link_bytes);
       if (e != cudaSuccess) {
         free_chain(ch);
         return fail(SU3_ENOMEM, "cudaMalloc of %zu link bytes: %s", ch.link_bytes, cudaGetErrorString(e));
@@ -695,28 +744,23 @@ struct Engine {
     }
     const size_t npart = std::max(ntiles, (size_t)ch.desc.nlayers * kMeasureCtas) * kPartVals;
     const size_t nres = (size_t)ch.desc.result_cap * (ch.desc.nlayers + 1) * kMeasVals;
-    cudaError_t e1 = cudaMalloc(&ch.partials, npart * sizeof(double));
-    cudaError_t e2 = cudaMalloc(&ch.results, nres * sizeof(double));
-    cudaError_t e3 = cudaMalloc(&ch.counters, kCounterBytes);
-    if (e1 != cudaSuccess || e2 != cudaSuccess || e3 != cudaSuccess) {
-      free_chain(ch);
-      return fail(SU3_ENOMEM, "scratch allocation failed");
-    }
-    ch.bytes_total += npart * sizeof(double) + nres * sizeof(double) + kCounterBytes;
+    // one block of scratch: what starts at zero (counters, booked changes,
+    // reference, results) first, then the partial sums
     ch.n_action_slots = ch.desc.nlayers * ch.desc.nb * ((ch.desc.Vn + narrow - 1) / narrow);
-    if (cudaMalloc(&ch.action_slots, (size_t)ch.n_action_slots * sizeof(double)) != cudaSuccess) {
+    const size_t nref = 3 * kMeasVals, n0 = kCounterBytes / sizeof(double);
+    const size_t zero = n0 + (size_t)ch.n_action_slots + nref + nres, bytes = (zero + npart) * sizeof(double);
+    if (chain_alloc(&ch.scratch, bytes) != cudaSuccess) {
       free_chain(ch);
-      return fail(SU3_ENOMEM, "action bookkeeping allocation failed");
+      return fail(SU3_ENOMEM, "scratch allocation of %zu bytes failed", bytes);
     }
-    CU(cudaMemsetAsync(ch.action_slots, 0, (size_t)ch.n_action_slots * sizeof(double), stream));
-    ch.bytes_total += (size_t)ch.n_action_slots * sizeof(double);
-    if (cudaMalloc(&ch.ref_meas, 3 * kMeasVals * sizeof(double)) != cudaSuccess) {
-      free_chain(ch);
-      return fail(SU3_ENOMEM, "action reference allocation failed");
-    }
-    CU(cudaMemsetAsync(ch.ref_meas, 0, 3 * kMeasVals * sizeof(double), stream));
-    CU(cudaMemsetAsync(ch.counters, 0, kCounterBytes, stream));
-    CU(cudaMemsetAsync(ch.results, 0, nres * sizeof(double), stream));
+    ch.bytes_total += bytes;
+    double *p = static_cast<double *>(ch.scratch);
+    ch.counters = reinterpret_cast<unsigned long long *>(p);
+    ch.action_slots = p + n0;
+    ch.ref_meas = ch.action_slots + ch.n_action_slots;
+    ch.results = ch.ref_meas + nref;
+    ch.partials = ch.results + nres;
+    CU(cudaMemsetAsync(ch.scratch, 0, zero * sizeof(double), stream));
     fill_desc(ch, block);
     if (ch.sub) fill_plain(ch, block);
     ch.state = ChainState{};
@@ -726,21 +770,22 @@ struct Engine {
     return SU3_OK;
   }
 
-  // Write a chain's start configuration through a scratch descriptor.
+  // Write a chain's start configuration, in stream order.
   su3_status start_chain(Chain &ch) {
+    const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
+    const int hot = ch.cfg.start == SU3_START_HOT;
+    if (!ch.sub) {
+      CU(launch_start(storage, ch.desc, nlinks, hot, stream));
+      return SU3_OK;
+    }
+    // start the undivided layout, scatter it into the boxes, fill every halo
     ChainDesc *dd = nullptr;
     CU(cudaMallocAsync(&dd, sizeof(ChainDesc), stream));
     CU(cudaMemcpyAsync(dd, &ch.desc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
-    const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
-    if (ch.sub) {
-      // start the undivided layout, scatter it into the boxes, fill every halo
-      CU(cudaMemcpyAsync(ch.d_pdesc, &ch.pdesc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
-      CU(launch_start(storage, ch.d_pdesc, nlinks, ch.cfg.start == SU3_START_HOT, stream));
-      CU(launch_sub_copy(storage, dd, ch.d_pdesc, nlinks, 1, stream));
-      CU(launch_halo(storage, ch.desc, -1, ch.halo_n[0] + ch.halo_n[1], stream));
-    } else {
-      CU(launch_start(storage, dd, nlinks, ch.cfg.start == SU3_START_HOT, stream));
-    }
+    CU(cudaMemcpyAsync(ch.d_pdesc, &ch.pdesc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
+    CU(launch_start(storage, ch.pdesc, nlinks, hot, stream));
+    CU(launch_sub_copy(storage, dd, ch.d_pdesc, nlinks, 1, stream));
+    CU(launch_halo(storage, ch.desc, -1, ch.halo_n[0] + ch.halo_n[1], stream));
     CU(cudaFreeAsync(dd, stream));
     CU(cudaStreamSynchronize(stream));  // the host ChainDesc copy is freed with it
     return SU3_OK;
@@ -922,16 +967,12 @@ struct Engine {
     return SU3_OK;
   }
 
-  // The descriptor that measurement and link I/O kernels read: the chain's
-  // own, or (divided chain) its undivided copy after a gather.
-  su3_status io_desc(size_t c, ChainDesc **dd) {
+  // The descriptor that measurements and link output read: the chain's own, or
+  // (divided chain) its undivided copy after a gather.
+  su3_status io_desc(size_t c, const ChainDesc **d) {
     Chain &ch = chains[c];
-    if (!ch.sub) {
-      *dd = d_desc + c;
-      return SU3_OK;
-    }
-    TRY(sub_sync(c, 0));
-    *dd = ch.d_pdesc;
+    if (ch.sub) TRY(sub_sync(c, 0));
+    *d = ch.sub ? &ch.pdesc : &ch.desc;
     return SU3_OK;
   }
 
@@ -1164,17 +1205,44 @@ struct Engine {
   // Measure a chain's links (divided: gathered into the undivided layout)
   // into device memory, queued.
   su3_status measure_into(size_t c, double *device_out) {
-    ChainDesc *dd = nullptr;
-    TRY(io_desc(c, &dd));
-    CU(launch_measure(storage, false, chains[c].sub ? chains[c].pdesc : chains[c].desc, device_out, d_ctl, stream, false));
+    const ChainDesc *d = nullptr;
+    TRY(io_desc(c, &d));
+    CU(launch_measure(storage, false, *d, device_out, d_ctl, stream, false));
     return SU3_OK;
+  }
+
+  // Measurement (3 kMeasVals doubles each) and counters of up to kRetireBatch
+  // chains with one wait.
+  static constexpr int kRetireBatch = 32, kRetireDoubles = 3 * kMeasVals + 2 * kCounterSlots;
+  su3_status measure_many(const size_t *c, int n, double (*vals)[3 * kMeasVals], uint64_t (*cnt)[2]) {
+    if (tiles_dirty) TRY(rebuild());
+    if (!d_meas_out) CU(cudaMalloc(&d_meas_out, kRetireBatch * 3 * kMeasVals * sizeof(double)));
+    double *hc = h_pinned + kRetireBatch * 3 * kMeasVals;
+    for (int i = 0; i < n; ++i) {
+      TRY(measure_into(c[i], d_meas_out + i * 3 * kMeasVals));
+      CU(cudaMemcpyAsync(hc + i * 2 * kCounterSlots, chains[c[i]].counters, kCounterBytes, cudaMemcpyDeviceToHost, stream));
+    }
+    CU(cudaMemcpyAsync(h_pinned, d_meas_out, n * 3 * kMeasVals * sizeof(double), cudaMemcpyDeviceToHost, stream));
+    CU(cudaStreamSynchronize(stream));
+    for (int i = 0; i < n; ++i) {
+      std::memcpy(vals[i], h_pinned + i * 3 * kMeasVals, sizeof vals[i]);
+      sum_counters(hc + i * 2 * kCounterSlots, cnt[i]);
+    }
+    return SU3_OK;
+  }
+
+  static void sum_counters(const double *words, uint64_t out[2]) {
+    unsigned long long all[2 * kCounterSlots];
+    std::memcpy(all, words, sizeof all);
+    out[0] = out[1] = 0;
+    for (int i = 0; i < 2 * kCounterSlots; ++i) out[i & 1] += all[i];
   }
 
   su3_status measure_chain(size_t c, double *host_out /* 5*(layers+1) */) {
     if (tiles_dirty) TRY(rebuild());
     Chain &ch = chains[c];
     const int nvals = (ch.desc.nlayers + 1) * kMeasVals;
-    if (!d_meas_out) CU(cudaMalloc(&d_meas_out, 3 * kMeasVals * sizeof(double)));
+    if (!d_meas_out) CU(cudaMalloc(&d_meas_out, kRetireBatch * 3 * kMeasVals * sizeof(double)));
     TRY(measure_into(c, d_meas_out));
     CU(cudaMemcpyAsync(h_pinned, d_meas_out, nvals * sizeof(double), cudaMemcpyDeviceToHost, stream));
     CU(cudaStreamSynchronize(stream));
@@ -1188,10 +1256,10 @@ struct Engine {
     const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
     if (!host || n < nlinks * 18) return fail(SU3_EINVAL, "host buffer holds %zu doubles, %zu needed", n, nlinks * 18);
     double *canon = nullptr;
-    ChainDesc *dd = nullptr;
-    TRY(io_desc(c, &dd));
-    CU(cudaMallocAsync(&canon, nlinks * 18 * sizeof(double), stream));
-    CU(launch_convert(storage, dd, nlinks, canon, 1, stream));
+    const ChainDesc *d = nullptr;
+    TRY(io_desc(c, &d));
+    CU(canon_alloc(&canon, nlinks * 18 * sizeof(double)));
+    CU(launch_convert(storage, *d, nlinks, canon, 1, stream));
     CU(cudaMemcpyAsync(host, canon, nlinks * 18 * sizeof(double), cudaMemcpyDeviceToHost, stream));
     CU(cudaFreeAsync(canon, stream));
     CU(cudaStreamSynchronize(stream));
@@ -1204,9 +1272,9 @@ struct Engine {
     const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
     if (!host || n < nlinks * 18) return fail(SU3_EINVAL, "host buffer holds %zu doubles, %zu needed", n, nlinks * 18);
     double *canon = nullptr;
-    CU(cudaMallocAsync(&canon, nlinks * 18 * sizeof(double), stream));
+    CU(canon_alloc(&canon, nlinks * 18 * sizeof(double)));
     CU(cudaMemcpyAsync(canon, host, nlinks * 18 * sizeof(double), cudaMemcpyHostToDevice, stream));
-    CU(launch_convert(storage, ch.sub ? ch.d_pdesc : d_desc + c, nlinks, canon, 0, stream));
+    CU(launch_convert(storage, ch.sub ? ch.pdesc : ch.desc, nlinks, canon, 0, stream));
     if (ch.sub) TRY(sub_sync(c, 1));  // scatter into the boxes, refresh every halo
     CU(cudaFreeAsync(canon, stream));
     CU(cudaStreamSynchronize(stream));
@@ -1230,7 +1298,7 @@ struct Engine {
 
   su3_status booked_change(size_t c, double *dS) {
     Chain &ch = chains[c];
-    if (!d_meas_out) CU(cudaMalloc(&d_meas_out, 3 * kMeasVals * sizeof(double)));
+    if (!d_meas_out) CU(cudaMalloc(&d_meas_out, kRetireBatch * 3 * kMeasVals * sizeof(double)));
     CU(launch_action_sum(ch.action_slots, ch.n_action_slots, d_meas_out, stream));
     CU(cudaMemcpyAsync(h_pinned, d_meas_out, sizeof(double), cudaMemcpyDeviceToHost, stream));
     CU(cudaStreamSynchronize(stream));
@@ -1291,12 +1359,10 @@ struct Engine {
   }
 
   su3_status counters(size_t c, uint64_t *prop, uint64_t *acc) {
-    static_assert(kCounterBytes <= 4096, "h_pinned");
     CU(cudaMemcpyAsync(h_pinned, chains[c].counters, kCounterBytes, cudaMemcpyDeviceToHost, stream));
     CU(cudaStreamSynchronize(stream));
-    unsigned long long all[2 * kCounterSlots], v[2] = {0, 0};
-    std::memcpy(all, h_pinned, sizeof all);
-    for (int i = 0; i < 2 * kCounterSlots; ++i) v[i & 1] += all[i];
+    uint64_t v[2];
+    sum_counters(h_pinned, v);
     if (prop) *prop = v[0];
     if (acc) *acc = v[1];
     return SU3_OK;
@@ -1562,11 +1628,11 @@ extern "C" su3_status su3_apply_links(su3_lattice *lat) {
   const int b = lat->pending;
   const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
   CU(cudaStreamWaitEvent(e.stream, lat->copied[b], 0));
-  ChainDesc *dd = ch.sub ? ch.d_pdesc : e.d_desc;
+  const ChainDesc &d = ch.sub ? ch.pdesc : ch.desc;
   if (lat->fmt[b] == SU3_LINKS_FP32_12)
-    CU(launch_convert_rows2(e.storage, dd, nlinks, reinterpret_cast<const float *>(lat->stage[b]), e.stream));
+    CU(launch_convert_rows2(e.storage, d, nlinks, reinterpret_cast<const float *>(lat->stage[b]), e.stream));
   else
-    CU(launch_convert(e.storage, dd, nlinks, lat->stage[b], 0, e.stream));
+    CU(launch_convert(e.storage, d, nlinks, lat->stage[b], 0, e.stream));
   if (ch.sub) TRY(e.sub_sync(0, 1));
   CU(cudaEventRecord(lat->consumed[b], e.stream));
   lat->used[b] = true;
@@ -1967,6 +2033,13 @@ extern "C" su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, 
     hbm_budget_bytes = (size_t)(0.8 * (double)fr);
   }
   srv->budget = hbm_budget_bytes;
+  if (srv->eng.make_pool(hbm_budget_bytes) != SU3_OK) {
+    const std::string msg = g_err;
+    srv->eng.release();
+    cudaStreamDestroy(st);
+    delete srv;
+    return fail(SU3_ECUDA, "%s", msg.c_str());
+  }
   srv->max_slots = max_slots;
   {
     // persistent grid: its size does not depend on the resident jobs, so the
@@ -2122,7 +2195,7 @@ void su3_server::loop() {
         eng.chains.push_back(ch);
         st = eng.start_chain(eng.chains.back());
         if (st != SU3_OK) {
-          Engine::free_chain(eng.chains.back());
+          eng.free_chain(eng.chains.back());
           eng.chains.pop_back();
         }
       }
@@ -2200,23 +2273,29 @@ void su3_server::loop() {
       if (!eng.chains[c].state.active) done.push_back(c);
     bool retired = !done.empty();
     std::vector<su3_result> results;
-    for (size_t c : done) {
+    double vals[Engine::kRetireBatch][3 * kMeasVals];
+    uint64_t cnt[Engine::kRetireBatch][2];
+    su3_status ms = SU3_OK;
+    for (size_t i = 0; i < done.size(); ++i) {
+      const size_t c = done[i];
+      const int at = (int)(i % Engine::kRetireBatch);
+      if (at == 0)
+        ms = eng.measure_many(&done[i], (int)std::min<size_t>(done.size() - i, Engine::kRetireBatch), vals, cnt);
       Chain &ch = eng.chains[c];
       su3_result r{};
       r.job_id = ch.job_id;
-      r.status = SU3_OK;
+      r.status = ms == SU3_OK ? SU3_OK : SU3_ECUDA;
       r.nlayers = ch.desc.nlayers;
-      double v[3 * kMeasVals];
-      if (eng.measure_chain(c, v) == SU3_OK) {
+      if (ms == SU3_OK) {
+        const double *v = vals[at];
         const int w = ch.desc.nlayers;
         for (int k = 0; k < 3; ++k) r.plaquette[k] = v[w * kMeasVals + k];
         r.polyakov[0] = v[w * kMeasVals + 3];
         r.polyakov[1] = v[w * kMeasVals + 4];
         for (int l = 0; l < ch.desc.nlayers; ++l) r.layer_plaquette[l] = v[l * kMeasVals];
-      } else {
-        r.status = SU3_ECUDA;
+        r.proposals = cnt[at][0];
+        r.accepts = cnt[at][1];
       }
-      eng.counters(c, &r.proposals, &r.accepts);
       double *lo = nullptr;
       {
         std::lock_guard<std::mutex> lk(mu);
@@ -2235,7 +2314,7 @@ void su3_server::loop() {
     for (size_t i = done.size(); i-- > 0;) {
       Chain &ch = eng.chains[done[i]];
       bytes[i] = job_bytes(ch.cfg);
-      Engine::free_chain(ch);
+      eng.free_chain(ch);
       eng.chains.erase(eng.chains.begin() + (long)done[i]);
     }
     if (retired) {

@@ -327,15 +327,6 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
 
 // ------------------------------------------------------------------ one-off kernels
 
-// The CTA's shared copy of a chain descriptor (a per-thread copy of the
-// struct would live in local memory).
-__device__ __forceinline__ void desc_to_shared(ChainDesc &dst, const ChainDesc *src) {
-  const uint32_t *s = reinterpret_cast<const uint32_t *>(src);
-  uint32_t *d = reinterpret_cast<uint32_t *>(&dst);
-  for (int i = threadIdx.x; i < (int)(sizeof(ChainDesc) / 4); i += blockDim.x) d[i] = s[i];
-  __syncthreads();
-}
-
 // Sum of a chain's booked action changes, one warp, fixed order.
 __global__ void k_action_sum(const double *slots, int n, double *out) {
   double v = 0.0;
@@ -386,9 +377,7 @@ cudaError_t launch_action_sum(const double *slots, int n, double *out, cudaStrea
 // ------------------------------------------------------------------ start configurations
 
 template <class S>
-__global__ void k_start(ChainDesc *desc_dev, int hot) {
-  __shared__ ChainDesc d;
-  desc_to_shared(d, desc_dev);
+__global__ void k_start(const __grid_constant__ ChainDesc d, int hot) {
   const size_t nl = (size_t)d.nlayers * 2 * d.D * d.Vh;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nl; i += (size_t)gridDim.x * blockDim.x) {
     const int jj = (int)(i % d.Vh);
@@ -433,9 +422,7 @@ __global__ void k_start(ChainDesc *desc_dev, int hot) {
 // ------------------------------------------------------------------ canonical layout <-> storage
 
 template <class S>
-__global__ void k_convert(ChainDesc *desc_dev, double *canon, int to_canonical) {
-  __shared__ ChainDesc d;
-  desc_to_shared(d, desc_dev);
+__global__ void k_convert(const __grid_constant__ ChainDesc d, double *canon, int to_canonical) {
   const size_t nlinks = (size_t)d.nlayers * d.V * d.D;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nlinks; i += (size_t)gridDim.x * blockDim.x) {
     const int mu = (int)(i % d.D);
@@ -564,9 +551,7 @@ __global__ void k_sub_copy(const ChainDesc *sub_dev, const ChainDesc *plain_dev,
 // Links given as rows 1 and 2 in float (12 per link, canonical site order:
 // [layer][i_s - 1][mu][row][col][re, im]); row 3 = conj(row1 x row2).
 template <class S>
-__global__ void k_convert_rows2(ChainDesc *desc_dev, const float *src) {
-  __shared__ ChainDesc d;
-  desc_to_shared(d, desc_dev);
+__global__ void k_convert_rows2(const __grid_constant__ ChainDesc d, const float *src) {
   const size_t nlinks = (size_t)d.nlayers * d.V * d.D;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nlinks; i += (size_t)gridDim.x * blockDim.x) {
     const int mu = (int)(i % d.D);
@@ -807,27 +792,27 @@ cudaError_t launch_sub_copy(int storage, const ChainDesc *sub_dev, const ChainDe
   });
 }
 
-cudaError_t launch_start(int storage, ChainDesc *desc_dev, size_t nlinks, int hot, cudaStream_t st) {
+cudaError_t launch_start(int storage, const ChainDesc &d, size_t nlinks, int hot, cudaStream_t st) {
   const int block = 256, grid = copy_grid(nlinks, block);
   return by_storage(storage, [&](auto s) {
-    k_start<decltype(s)><<<grid, block, 0, st>>>(desc_dev, hot);
+    k_start<decltype(s)><<<grid, block, 0, st>>>(d, hot);
     return cudaGetLastError();
   });
 }
 
-cudaError_t launch_convert_rows2(int storage, ChainDesc *desc_dev, size_t nlinks, const float *src, cudaStream_t st) {
+cudaError_t launch_convert_rows2(int storage, const ChainDesc &d, size_t nlinks, const float *src, cudaStream_t st) {
   const int block = 256, grid = copy_grid(nlinks, block);
   return by_storage(storage, [&](auto s) {
-    k_convert_rows2<decltype(s)><<<grid, block, 0, st>>>(desc_dev, src);
+    k_convert_rows2<decltype(s)><<<grid, block, 0, st>>>(d, src);
     return cudaGetLastError();
   });
 }
 
-cudaError_t launch_convert(int storage, ChainDesc *desc_dev, size_t nlinks, double *canon, int to_canonical,
+cudaError_t launch_convert(int storage, const ChainDesc &d, size_t nlinks, double *canon, int to_canonical,
                            cudaStream_t st) {
   const int block = 256, grid = copy_grid(nlinks, block);
   return by_storage(storage, [&](auto s) {
-    k_convert<decltype(s)><<<grid, block, 0, st>>>(desc_dev, canon, to_canonical);
+    k_convert<decltype(s)><<<grid, block, 0, st>>>(d, canon, to_canonical);
     return cudaGetLastError();
   });
 }

@@ -39,11 +39,11 @@ cudaError_t launch_set_ctl(ChainCtl *ctl, uint32_t sweep, uint32_t n_meas, int a
 cudaError_t launch_halo(int storage, const ChainDesc &d, int stage, int halo_sites, cudaStream_t st, bool pdl = false);
 cudaError_t launch_sub_copy(int storage, const ChainDesc *sub_dev, const ChainDesc *plain_dev, size_t nlinks,
                             int to_sub, cudaStream_t st);
-cudaError_t launch_start(int storage, ChainDesc *desc_dev, size_t nlinks, int hot, cudaStream_t st);
-cudaError_t launch_convert(int storage, ChainDesc *desc_dev, size_t nlinks, double *canon, int to_canonical,
+cudaError_t launch_start(int storage, const ChainDesc &d, size_t nlinks, int hot, cudaStream_t st);
+cudaError_t launch_convert(int storage, const ChainDesc &d, size_t nlinks, double *canon, int to_canonical,
                            cudaStream_t st);
 // Links from rows 1, 2 in float (12 per link, canonical order; 16-byte aligned).
-cudaError_t launch_convert_rows2(int storage, ChainDesc *desc_dev, size_t nlinks, const float *src, cudaStream_t st);
+cudaError_t launch_convert_rows2(int storage, const ChainDesc &d, size_t nlinks, const float *src, cudaStream_t st);
 void host_advance_stage(const ChainDesc &d, ChainState &s);
 // Fixed-order sum of n booked action-change slots into *out (device).
 cudaError_t launch_action_sum(const double *slots, int n, double *out, cudaStream_t st);
