@@ -451,18 +451,22 @@ struct Engine {
   bool weighted_any = false;  // some chain has two couplings: the update's weighted form
   bool sub_any = false;       // the (only) chain is divided into sublattice boxes
   bool torus_all = false;     // every chain is an undivided periodic 4-D torus, one coupling, default key
-  bool coop = false;          // FP64, too few links to fill the GPU: eight lanes per link
+  bool cluster = false;       // fixed, fewest links: whole sweeps per launch (k_sweeps)
+  bool coop = false;          // too few links to fill the GPU: eight lanes per link
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
-  int kernel_variant() const { return coop ? 1 : variant; }
+  int kernel_variant() const { return !coop ? variant : (storage == SU3_FP64_18 ? 1 : kFloatLanes); }
   // The links of one update phase of an FP64 chain that may take eight lanes
   // per link (others: more than any limit).
   long long coop_sites(const Chain &ch) const {
-    if (storage != SU3_FP64_18) return 1ll << 40;
+    return storage == SU3_FP64_18 ? phase_links(ch) : 1ll << 40;
+  }
+  static long long phase_links(const Chain &ch) {
     long long n = ch.cfg.boundary == SU3_DLT ? 2 : 1;
     for (int i = 0; i < ch.cfg.D; ++i) n *= ch.cfg.dims[i];
     return n / 2;
   }
-  static constexpr int kMaxChunk = 4;  // sweeps of one graph
+  static constexpr int kMaxChunk = 4;       // sweeps of one graph
+  static constexpr int kClusterChunk = 16;  // sweeps of one k_sweeps launch (no graph: it is one launch)
   cudaStream_t stream = nullptr;
   std::vector<Chain> chains;
   // device mirrors
@@ -734,8 +738,8 @@ struct Engine {
       ch.bytes_total += ch.link_bytes;
     }
     // partials and action slots sized for the narrowest tile
-    const bool coop = coop_sites(ch) <= kCoopSites;
-    const int narrow = coop ? 32 / kCoopLanes : 32;
+    const bool few = phase_links(ch) <= (storage == SU3_FP64_18 ? kCoopSites : kLanesLinks);
+    const int narrow = few ? 32 / kCoopLanes : 32;
     fill_desc(ch, narrow);
     size_t ntiles = (size_t)ch.desc.nlayers * ch.desc.tiles_per_layer;
     if (ch.sub) {
@@ -785,7 +789,7 @@ struct Engine {
     CU(cudaMemcpyAsync(ch.d_pdesc, &ch.pdesc, sizeof(ChainDesc), cudaMemcpyHostToDevice, stream));
     CU(launch_start(storage, ch.pdesc, nlinks, hot, stream));
     CU(launch_sub_copy(storage, dd, ch.d_pdesc, nlinks, 1, stream));
-    CU(launch_halo(storage, ch.desc, -1, ch.halo_n[0] + ch.halo_n[1], stream));
+    CU(launch_halo(storage, ch.desc, ch.halo_n[0] + ch.halo_n[1], stream));
     CU(cudaFreeAsync(dd, stream));
     CU(cudaStreamSynchronize(stream));  // the host ChainDesc copy is freed with it
     return SU3_OK;
@@ -802,7 +806,9 @@ struct Engine {
       sites += coop_sites(ch);
       weighted = weighted || ch.desc.weighted;
     }
-    const bool cp = sites <= kCoopSites && !weighted;
+    // eight lanes per link: FP64, and one-chain float engines, with few links
+    const bool cp = !weighted && (storage == SU3_FP64_18 ? sites <= kCoopSites
+                                                         : fixed && phase_links(chains[0]) <= kLanesLinks);
     if (cp != coop) drop_graph();
     coop = cp;
     for (auto &ch : chains) {
@@ -824,6 +830,7 @@ struct Engine {
     bool tor = !chains.empty();
     for (auto &ch : chains)
       tor = tor && ch.desc.nlayers == 1 && ch.desc.D == 4 && !ch.sub && !ch.desc.weighted && !ch.desc.custom_period;
+    cluster = fixed && !w && phase_links(chains[0]) <= kClusterLinks && sweeps_supported(storage, sb);
     if (w != weighted_any || sb != sub_any || tor != torus_all) {  // another kernel form: the captured graph is stale
       weighted_any = w;
       sub_any = sb;
@@ -939,10 +946,10 @@ struct Engine {
 
   EngineArgs args() const { return EngineArgs{d_desc, d_state, d_hdr, d_tile_chain, d_meas_list}; }
 
-  // Halo refresh of a divided chain (stage -1: all links).
-  cudaError_t halo_refresh(int stage, bool programmatic) const {
+  // Refresh every halo of a divided chain (update phases write their own).
+  cudaError_t halo_refresh(bool programmatic) const {
     const Chain &ch = chains[0];
-    return launch_halo(storage, ch.desc, stage, ch.halo_n[0] + ch.halo_n[1], stream, programmatic);
+    return launch_halo(storage, ch.desc, ch.halo_n[0] + ch.halo_n[1], stream, programmatic);
   }
 
   su3_status one_tick(int grid) {
@@ -963,7 +970,7 @@ struct Engine {
     Chain &ch = chains[c];
     const size_t nlinks = (size_t)ch.desc.nlayers * ch.desc.D * ch.desc.V;
     CU(launch_sub_copy(storage, d_desc + c, ch.d_pdesc, nlinks, to_sub, stream));
-    if (to_sub) CU(halo_refresh(-1, false));
+    if (to_sub) CU(halo_refresh(false));
     return SU3_OK;
   }
 
@@ -1043,7 +1050,8 @@ struct Engine {
   Chunk next_chunk(int n) const {
     const Chain &ch = chains[0];
     Chunk c{0, false, false};
-    while (c.m < n && c.m < kMaxChunk && !c.reunit && !c.measure) {
+    const int most = cluster ? kClusterChunk : kMaxChunk;
+    while (c.m < n && c.m < most && !c.reunit && !c.measure) {
       ++c.m;
       const uint32_t s = ch.state.sweep + (uint32_t)c.m;
       c.reunit = ch.desc.reunit_every > 0 && s % (uint32_t)ch.desc.reunit_every == 0;
@@ -1057,7 +1065,7 @@ struct Engine {
   }
   cudaError_t reunit_all() {
     cudaError_t e = launch_reunit(storage, sub_any, chains[0].desc, stream, pdl);
-    if (e == cudaSuccess && sub_any) e = halo_refresh(-1, pdl);
+    if (e == cudaSuccess && sub_any) e = halo_refresh(pdl);
     return e;
   }
 
@@ -1065,7 +1073,8 @@ struct Engine {
   template <class F>
   su3_status launch_chunk(const Chunk &c, int grid, F &&each) {
     const ChainDesc &d = chains[0].desc;
-    for (int i = 0; i < c.m; ++i)
+    if (cluster) TRY(each(0, [&] { return launch_sweeps(storage, sub_any, d, d_ctl, c.m, stream, pdl); }));
+    for (int i = 0; i < (cluster ? 0 : c.m); ++i)
       for (int st = 0; st < 2 * d.D; ++st) {
         UpdateStep u{};
         u.colour = st / d.D;
@@ -1074,11 +1083,9 @@ struct Engine {
         u.first = i == 0 && st == 0;
         u.advance = i == c.m - 1 && st == 2 * d.D - 1 ? (uint32_t)c.m : 0u;
         u.tiles = total_tiles;
-        TRY(each(0, [&]() -> cudaError_t {
-          cudaError_t e = launch_update(storage, kernel_variant(), weighted_any, sub_any, torus_all, d, d_ctl, u, grid,
-                                        block, stream, pdl);
-          if (e == cudaSuccess && sub_any) e = halo_refresh(st, pdl);
-          return e;
+        TRY(each(0, [&] {
+          return launch_update(storage, kernel_variant(), weighted_any, sub_any, torus_all, d, d_ctl, u, grid, block,
+                               stream, pdl);
         }));
       }
     if (c.reunit) TRY(each(1, [&] { return reunit_all(); }));
@@ -1107,7 +1114,7 @@ struct Engine {
   su3_status run_chunk(const Chunk &c) {
     int grid = 0;
     TRY(grid_size(&grid));
-    if (use_graph && !profiling) {
+    if (use_graph && !profiling && !cluster) {
       cudaGraphExec_t &g = chunk_graph[c.kind()];
       if (!g) {
         cudaError_t e = capture_chunk(c, grid, &g);
@@ -1761,7 +1768,7 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     for (int t : cand_t) {
       if (t > tick_max_threads(e.storage, v)) continue;
       int occ = 0;
-      const int kv = e.coop ? 1 : v;
+      const int kv = e.coop ? e.kernel_variant() : v;
       const cudaError_t oe = e.fixed ? update_occupancy(e.storage, kv, e.weighted_any, e.sub_any, e.torus_all, t, &occ)
                                      : tick_occupancy(e.storage, kv, e.weighted_any, e.torus_all, t, &occ);
       if (oe != cudaSuccess || occ < 1) continue;

@@ -376,7 +376,20 @@ __device__ __forceinline__ void acc_su3_2rows_w(M3<R> &A, const M3<R> &m, R w) {
 // Every form has load (3 rows), load2 (rows 1, 2; row 3 left unset), store
 // and copy (one link between two planes, for halo and box copies).
 
-struct StoreF32x12 {
+// COH: loads see what other CTAs of the same launch have written and
+// synchronised (through L2); otherwise they take the read-only path, which is
+// right for links that no CTA of the launch writes.
+
+template <bool COH, class T>
+__device__ __forceinline__ T ld_link(const T *p) {
+  if constexpr (COH)
+    return __ldcg(p);
+  else
+    return __ldg(p);
+}
+
+template <bool COH>
+struct StoreF32x12T {
   using R = float;
   using Vec = float4;
   static constexpr int NQ = 3;  // rows 1, 2: six complex numbers
@@ -385,7 +398,7 @@ struct StoreF32x12 {
   __device__ static __forceinline__ M3<float> load2(const Vec *plane, int Vh, int jj) {
     if (!in_bounds(jj, Vh, kBoundsIndex)) return m3_zero<float>();
     const Vec *p = plane + jj;
-    const float4 q0 = __ldg(p), q1 = __ldg(p + Vh), q2 = __ldg(p + 2 * Vh);
+    const float4 q0 = ld_link<COH>(p), q1 = ld_link<COH>(p + Vh), q2 = ld_link<COH>(p + 2 * Vh);
     M3<float> m;
     m.e[0][0] = {q0.x, q0.y};
     m.e[0][1] = {q0.z, q0.w};
@@ -410,7 +423,7 @@ struct StoreF32x12 {
   __device__ static __forceinline__ void copy(Vec *dst, int dVh, int dj, const Vec *src, int sVh, int sj) {
     if (!(in_bounds(dj, dVh, kBoundsIndex) && in_bounds(sj, sVh, kBoundsIndex))) return;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) dst[(size_t)q * dVh + dj] = src[(size_t)q * sVh + sj];
+    for (int q = 0; q < NQ; ++q) dst[(size_t)q * dVh + dj] = ld_link<COH>(src + (size_t)q * sVh + sj);
   }
 };
 
@@ -421,7 +434,8 @@ struct StoreF32x12 {
 // start on 16-byte boundaries because Vh is even (all extents are even).
 // Loads of rows 1, 2 are those of the 12-real form; row 3 costs two more
 // loads instead of the cross product.
-struct StoreF32x18 {
+template <bool COH>
+struct StoreF32x18T {
   using R = float;
   using Vec = float2;
   static constexpr int NQ = 9;  // float2 units per link
@@ -429,7 +443,7 @@ struct StoreF32x18 {
   __device__ static __forceinline__ M3<float> load2(const Vec *plane, int Vh, int jj) {
     if (!in_bounds(jj, Vh, kBoundsIndex)) return m3_zero<float>();
     const float4 *p = reinterpret_cast<const float4 *>(plane) + jj;
-    const float4 q0 = __ldg(p), q1 = __ldg(p + Vh), q2 = __ldg(p + 2 * Vh);
+    const float4 q0 = ld_link<COH>(p), q1 = ld_link<COH>(p + Vh), q2 = ld_link<COH>(p + 2 * Vh);
     M3<float> m;
     m.e[0][0] = {q0.x, q0.y};
     m.e[0][1] = {q0.z, q0.w};
@@ -442,8 +456,8 @@ struct StoreF32x18 {
   __device__ static __forceinline__ M3<float> load(const Vec *plane, int Vh, int jj) {
     M3<float> m = load2(plane, Vh, jj);
     if (!in_bounds(jj, Vh, kBoundsIndex)) return m;
-    const float4 q3 = __ldg(reinterpret_cast<const float4 *>(plane) + 3 * Vh + jj);
-    const float2 q4 = __ldg(plane + 8 * Vh + jj);
+    const float4 q3 = ld_link<COH>(reinterpret_cast<const float4 *>(plane) + 3 * Vh + jj);
+    const float2 q4 = ld_link<COH>(plane + 8 * Vh + jj);
     m.e[2][0] = {q3.x, q3.y};
     m.e[2][1] = {q3.z, q3.w};
     m.e[2][2] = {q4.x, q4.y};
@@ -463,12 +477,13 @@ struct StoreF32x18 {
     float4 *d4 = reinterpret_cast<float4 *>(dst);
     const float4 *s4 = reinterpret_cast<const float4 *>(src);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) d4[(size_t)k * dVh + dj] = s4[(size_t)k * sVh + sj];
-    dst[(size_t)8 * dVh + dj] = src[(size_t)8 * sVh + sj];
+    for (int k = 0; k < 4; ++k) d4[(size_t)k * dVh + dj] = ld_link<COH>(s4 + (size_t)k * sVh + sj);
+    dst[(size_t)8 * dVh + dj] = ld_link<COH>(src + (size_t)8 * sVh + sj);
   }
 };
 
-struct StoreF64x18 {
+template <bool COH>
+struct StoreF64x18T {
   using R = double;
   using Vec = double2;
   static constexpr int NQ = 9;  // one complex number per 128-bit vector
@@ -479,7 +494,7 @@ struct StoreF64x18 {
     M3<double> m;
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
-      const double2 v = __ldg(p + q * Vh);
+      const double2 v = ld_link<COH>(p + q * Vh);
       m.e[q / 3][q % 3] = {v.x, v.y};
     }
     return m;
@@ -490,7 +505,7 @@ struct StoreF64x18 {
     M3<double> m;
 #pragma unroll
     for (int q = 0; q < 6; ++q) {
-      const double2 v = __ldg(p + q * Vh);
+      const double2 v = ld_link<COH>(p + q * Vh);
       m.e[q / 3][q % 3] = {v.x, v.y};
     }
     return m;
@@ -504,9 +519,13 @@ struct StoreF64x18 {
   __device__ static __forceinline__ void copy(Vec *dst, int dVh, int dj, const Vec *src, int sVh, int sj) {
     if (!(in_bounds(dj, dVh, kBoundsIndex) && in_bounds(sj, sVh, kBoundsIndex))) return;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) dst[(size_t)q * dVh + dj] = src[(size_t)q * sVh + sj];
+    for (int q = 0; q < NQ; ++q) dst[(size_t)q * dVh + dj] = ld_link<COH>(src + (size_t)q * sVh + sj);
   }
 };
+
+using StoreF32x12 = StoreF32x12T<false>;
+using StoreF32x18 = StoreF32x18T<false>;
+using StoreF64x18 = StoreF64x18T<false>;
 
 // The (layer, colour, mu) plane of a chain's links.  Offsets stay in 32 bits
 // (the host rejects chains with 2^31 vectors or more).
@@ -798,8 +817,7 @@ struct DrawPre {
   float L, u4sq, costh, sinth, cphi, sphi;
 };
 
-__device__ __forceinline__ void proposal_pre_f(DrawPre &p, uint2 key, uint32_t c0, uint32_t c1, uint32_t tag) {
-  const uint4 w = philox4x32_10(make_uint4(c0, c1, tag, kPurposeHeatbath), key);
+__device__ __forceinline__ void proposal_pre_words(DrawPre &p, const uint4 &w) {
   const float ang = __fmaf_rn(unif_f(w.y), 6.28318530717958648f, -3.14159265358979324f);
   const float cs = __cosf(ang);
   const float l1 = __logf(unif_f(w.x));
@@ -807,6 +825,10 @@ __device__ __forceinline__ void proposal_pre_f(DrawPre &p, uint2 key, uint32_t c
   p.L = l1 + cs * cs * l3;
   const float u4 = unif_f(w.w);
   p.u4sq = u4 * u4;
+}
+
+__device__ __forceinline__ void proposal_pre_f(DrawPre &p, uint2 key, uint32_t c0, uint32_t c1, uint32_t tag) {
+  proposal_pre_words(p, philox4x32_10(make_uint4(c0, c1, tag, kPurposeHeatbath), key));
 }
 
 // The direction from its two words (those direction_words returns).
@@ -819,10 +841,36 @@ __device__ __forceinline__ void direction_pre_f(DrawPre &p, uint32_t wx, uint32_
   p.cphi = -cphi;
 }
 
+// The draw of a float link in the rare alpha ranges, out of line.
+struct DrawF {
+  float x[4];
+  uint32_t nprop;
+  bool accepted;
+};
+static __device__ __noinline__ DrawF su2_draw_rare(float alpha, int hits, uint2 key, uint32_t c0, uint32_t c1,
+                                                   uint32_t tag) {
+  DrawF r;
+  r.nprop = 0;
+  r.accepted = su2_draw(alpha, hits, key, c0, c1, tag, r.x, r.nprop);
+  return r;
+}
+
 // The float draw of one subgroup from its precomputed first proposal.
+// CALL: the rare alpha ranges as a call (short code; in the one-thread forms
+// the call's registers cost more than the code saves).
+template <bool CALL = false>
 __device__ __forceinline__ bool su2_draw_pre(float alpha, int hits, uint2 key, uint32_t c0, uint32_t c1, uint32_t tag,
                                              const DrawPre &p, float x[4], uint32_t &nprop) {
-  if (alpha >= kAlphaFp64 || alpha < kAlphaAccurateLog) return su2_draw(alpha, hits, key, c0, c1, tag, x, nprop);
+  if (alpha >= kAlphaFp64 || alpha < kAlphaAccurateLog) {
+    if constexpr (CALL) {
+      const DrawF r = su2_draw_rare(alpha, hits, key, c0, c1, tag);
+      nprop += r.nprop;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) x[q] = r.x[q];
+      return r.accepted;
+    }
+    return su2_draw(alpha, hits, key, c0, c1, tag, x, nprop);
+  }
   const float ia = rcp_sfu(alpha);
   ++nprop;
   float X = -p.L * ia;
@@ -847,6 +895,29 @@ __device__ __forceinline__ bool su2_draw_pre(float alpha, int hits, uint2 key, u
   return true;
 }
 
+// One subgroup (rows i, j) of the update of a float link.
+template <bool CALL = false>
+__device__ __forceinline__ void cm_subgroup_f(M3<float> &U, const M3<float> &A, int i, int j, float ca, int hits,
+                                              uint2 key, uint32_t c0, uint32_t c1, uint32_t tag, const DrawPre &pre,
+                                              uint32_t &nprop, uint32_t &nacc, float &dretr) {
+  float a0, a1, a2, a3;
+  block_projection(U, A, i, j, a0, a1, a2, a3);
+  float k, ik;
+  norm_and_inverse(a0 * a0 + a1 * a1 + a2 * a2 + a3 * a3, k, ik);
+  if (!(k > 1e-30f)) return;
+  const float alpha = ca * k;
+  float x[4];
+  if (!su2_draw_pre<CALL>(alpha, hits, key, c0, c1, tag, pre, x, nprop)) return;
+  ++nacc;
+  dretr += 2.0f * (k * x[0] - a0);
+  const float v0 = a0 * ik, v1 = a1 * ik, v2 = a2 * ik, v3 = a3 * ik;
+  const float r0 = x[0] * v0 + x[1] * v1 + x[2] * v2 + x[3] * v3;
+  const float r1 = -x[0] * v1 + v0 * x[1] + (x[2] * v3 - x[3] * v2);
+  const float r2 = -x[0] * v2 + v0 * x[2] + (x[3] * v1 - x[1] * v3);
+  const float r3 = -x[0] * v3 + v0 * x[3] + (x[1] * v2 - x[2] * v1);
+  rotate_rows(U, i, j, r0, r1, r2, r3);
+}
+
 // cm_update for float links with the draws' counter-only parts first.
 __device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, float beta, int hits, uint2 key,
                                             uint32_t c0, uint32_t c1, int colour, int mu, uint32_t &nprop,
@@ -866,22 +937,7 @@ __device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, fl
   for (int sg = 0; sg < 3; ++sg) {
     const int i = (sg == 2) ? 1 : 0;
     const int j = (sg == 0) ? 1 : 2;
-    float a0, a1, a2, a3;
-    block_projection(U, A, i, j, a0, a1, a2, a3);
-    float k, ik;
-    norm_and_inverse(a0 * a0 + a1 * a1 + a2 * a2 + a3 * a3, k, ik);
-    if (!(k > 1e-30f)) continue;
-    const float alpha = ca * k;
-    float x[4];
-    if (!su2_draw_pre(alpha, hits, key, c0, c1, heatbath_tag(colour, mu, sg), pre[sg], x, nprop)) continue;
-    ++nacc;
-    dretr += 2.0f * (k * x[0] - a0);
-    const float v0 = a0 * ik, v1 = a1 * ik, v2 = a2 * ik, v3 = a3 * ik;
-    const float r0 = x[0] * v0 + x[1] * v1 + x[2] * v2 + x[3] * v3;
-    const float r1 = -x[0] * v1 + v0 * x[1] + (x[2] * v3 - x[3] * v2);
-    const float r2 = -x[0] * v2 + v0 * x[2] + (x[3] * v1 - x[1] * v3);
-    const float r3 = -x[0] * v3 + v0 * x[3] + (x[1] * v2 - x[2] * v1);
-    rotate_rows(U, i, j, r0, r1, r2, r3);
+    cm_subgroup_f(U, A, i, j, ca, hits, key, c0, c1, heatbath_tag(colour, mu, sg), pre[sg], nprop, nacc, dretr);
   }
 }
 

@@ -46,6 +46,19 @@ constexpr float kAlphaAccurateLog = 2.0f;
 constexpr int kCoopLanes = 8;
 constexpr int kCoopSites = 8192;
 
+// Float chains of one coupling with at most kLanesLinks links per phase take
+// eight lanes per link too (update_site_lanes; the launchers' variant
+// kFloatLanes).  Per phase, one thread per link and eight lanes: 8^3 x 4 5.8
+// and 4.3 us, 8^4 5.9 and 4.4, 16^2 x 8 x 4 (4096 links) 6.0 and 5.4, 16^3 x 4
+// (8192) 6.4 and 7.4.  (Four lanes of two staples each: 4.8, 4.8, 5.1, 5.8.)
+constexpr int kLanesLinks = 4096, kFloatLanes = 16;
+// Chains of one coupling with at most kClusterLinks links per phase run whole
+// sweeps in one launch of a cluster of CTAs (k_sweeps), eight lanes per link:
+// float 4^4 3.3 us per phase (4.2 with a launch per phase), FP64 12.2 (12.5).
+// More links share the cluster's 16 SMs too long: 8^3 x 4 6.3 us against 4.3.
+constexpr int kClusterCtas = 16, kClusterThreads = 128;
+constexpr int kClusterLinks = kClusterCtas * kClusterThreads / kCoopLanes;
+
 // Pairs of FHKP counters per chain (their sums are the totals).
 constexpr int kCounterSlots = 32;
 // A measurement's partial sums: at most this many CTAs per layer (one wave: 5

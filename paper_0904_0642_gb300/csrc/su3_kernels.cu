@@ -463,57 +463,15 @@ __global__ void k_convert(const __grid_constant__ ChainDesc d, double *canon, in
 // double-layered torus lands in the other layer).  Halo sites are never
 // sources, so the copies do not race.
 
-// Refresh the halos of a divided chain: all links (stage < 0: after a start,
-// set_links or re-unitarisation) or, after an update phase, only its (colour,
-// direction).  Threads run over the box's list of halo sites of that colour
-// (blockIdx.y = box): the owner is the same padded site of the neighbouring
-// box given by the entry's offset code, whose box coordinate wraps
-// periodically; a wrap across a glued boundary of the double-layered torus
-// lands in the other layer.
+// Refresh every halo of a divided chain.  Threads run over the box's list of
+// halo sites (blockIdx.y = box).
 template <class S>
-__global__ void k_halo(const __grid_constant__ ChainDesc d, int stage) {
+__global__ void k_halo(const __grid_constant__ ChainDesc d) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  int c0 = 0, c1 = 2, m0 = 0, m1 = d.D;
-  if (stage >= 0) {
-    c0 = stage / d.D;
-    c1 = c0 + 1;
-    m0 = stage - c0 * d.D;
-    m1 = m0 + 1;
-  }
-  const int vl = blockIdx.y;
-  const int L = vl / d.nb;
-  int bc[kMaxD], rest = vl - L * d.nb;
-#pragma unroll
-  for (int k = 0; k < kMaxD; ++k) {
-    bc[k] = 0;
-    if (k < d.D) {
-      bc[k] = rest % d.bdiv[k];
-      rest /= d.bdiv[k];
-    }
-  }
-  const int first = c0 == 0 ? 0 : d.halo_n[0];
-  const int count = (c0 == 0 ? d.halo_n[0] : 0) + (c1 == 2 ? d.halo_n[1] : 0);
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x) {
-    const int4 h = d.halo[first + e];
-    const int colour = (first + e) < d.halo_n[0] ? 0 : 1;
-    int bsrc = 0, bmul = 1, flip = 0;
-#pragma unroll
-    for (int k = 0; k < kMaxD; ++k)
-      if (k < d.D) {
-        const int code = (h.z >> (2 * k)) & 3;
-        int o = bc[k] + (code == 1 ? -1 : (code == 2 ? 1 : 0));
-        if (o < 0 || o >= d.bdiv[k]) {
-          o = o < 0 ? o + d.bdiv[k] : o - d.bdiv[k];
-          if (d.nlayers == 2) flip ^= (d.glue_mask >> k) & 1;
-        }
-        bsrc += o * bmul;
-        bmul *= d.bdiv[k];
-      }
-    const int vsrc = (L ^ flip) * d.nb + bsrc;
-    for (int mu = m0; mu < m1; ++mu)
-      S::copy(plane_ptr<S>(d, vl, colour, mu), d.Vh, h.x >> 1, plane_ptr<S>(d, vsrc, colour, mu), d.Vh, h.y >> 1);
-  }
+  const int count = d.halo_n[0] + d.halo_n[1];
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < count; e += gridDim.x * blockDim.x)
+    halo_copy<S>(d, blockIdx.y, e);
 }
 
 // Copy links between the undivided layout (plain) and the sublattice boxes
@@ -733,7 +691,7 @@ struct TickOccupancy {
 
 int tick_max_threads(int storage, int variant) {
   if (storage == 0) return TickBounds<10>::kThreads;
-  if (storage == 2) return TickBounds<0>::kThreads;
+  if (storage == 2 || variant == kFloatLanes) return TickBounds<0>::kThreads;
   switch (variant) {
     case 0: return TickBounds<0>::kThreads;
     case 1: return TickBounds<1>::kThreads;
@@ -772,11 +730,11 @@ cudaError_t launch_tick(int storage, int variant, bool weighted, bool torus, con
                   : tick_dispatch<TickLaunch, false>(storage, variant, torus, pa, grid, block, st, pdl);
 }
 
-cudaError_t launch_halo(int storage, const ChainDesc &d, int stage, int halo_sites, cudaStream_t st, bool pdl) {
+cudaError_t launch_halo(int storage, const ChainDesc &d, int halo_sites, cudaStream_t st, bool pdl) {
   const int block = 256;
   const dim3 grid((unsigned)((halo_sites + block - 1) / block > 0 ? (halo_sites + block - 1) / block : 1),
                   (unsigned)(d.nlayers * d.nb));
-  return by_storage(storage, [&](auto s) { return launch_ex(k_halo<decltype(s)>, grid, block, st, pdl, d, stage); });
+  return by_storage(storage, [&](auto s) { return launch_ex(k_halo<decltype(s)>, grid, block, st, pdl, d); });
 }
 
 static int copy_grid(size_t nlinks, int block) {

@@ -28,15 +28,21 @@ cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, boo
                           ChainCtl *ctl, const UpdateStep &step, int grid, int block, cudaStream_t st, bool pdl);
 cudaError_t update_occupancy(int storage, int variant, bool weighted, bool sub, bool torus, int block,
                              int *ctas_per_sm);
+// Whole sweeps of a small one-coupling chain in one launch (at most
+// kClusterLinks links per phase).
+bool sweeps_supported(int storage, bool sub);
+cudaError_t launch_sweeps(int storage, bool sub, const ChainDesc &d, ChainCtl *ctl, int sweeps, cudaStream_t st,
+                          bool pdl);
 cudaError_t launch_reunit(int storage, bool sub, const ChainDesc &d, cudaStream_t st, bool pdl);
 cudaError_t launch_measure(int storage, bool sub, const ChainDesc &d, double *out, ChainCtl *ctl, cudaStream_t st,
                            bool pdl);
 cudaError_t launch_set_ctl(ChainCtl *ctl, uint32_t sweep, uint32_t n_meas, int anchor, cudaStream_t st);
 
-// Halo refresh of a divided chain (stage: the update phase colour D + mu, or
-// -1 for all links), and the copies between its sublattice boxes and the
-// undivided layout.  halo_sites: halo sites of one box (both colours).
-cudaError_t launch_halo(int storage, const ChainDesc &d, int stage, int halo_sites, cudaStream_t st, bool pdl = false);
+// Refresh every halo of a divided chain (after a start, new links or a
+// re-unitarisation; update phases write the copies of their links
+// themselves), and the copies between its sublattice boxes and the undivided
+// layout.  halo_sites: halo sites of one box (both colours).
+cudaError_t launch_halo(int storage, const ChainDesc &d, int halo_sites, cudaStream_t st, bool pdl = false);
 cudaError_t launch_sub_copy(int storage, const ChainDesc *sub_dev, const ChainDesc *plain_dev, size_t nlinks,
                             int to_sub, cudaStream_t st);
 cudaError_t launch_start(int storage, const ChainDesc &d, size_t nlinks, int hot, cudaStream_t st);

@@ -128,6 +128,51 @@ __device__ __forceinline__ int in_layer1(const ChainDesc &d, int l) {
     return l;
 }
 
+// The places where a site's links are stored: f(box, checkerboard index) for
+// the site itself (m = 0) and, SUB, for its copies in the halos of the
+// neighbouring boxes (one per nonempty set m of divided directions in which
+// it lies on a face).  m runs from `first` in steps of `step`, so that lanes
+// can share the stores.  An update phase writes the copies of its own links
+// itself: no link of the phase's colour and direction is read in it.  A site
+// on the high (low) face of direction k appears in the low (high) halo of the
+// next (previous) box; a step across a glued boundary of the double-layered
+// torus lands in the other layer.
+template <bool SUB, class F>
+__device__ __forceinline__ void for_replicas(const ChainDesc &d, const SiteGeo &g, int first, int step, F &&f) {
+  if constexpr (!SUB) {
+    if (first == 0) f(g.layer, g.s >> 1);
+  } else {
+    int on = 0;  // directions in which the site lies on a face
+#pragma unroll
+    for (int k = 0; k < kMaxD; ++k)
+      if (k < d.D && d.hpad[k] && (g.x[k] == 1 || g.x[k] == d.idims[k])) on |= 1 << k;
+    const int L = g.layer / d.nb, b = g.layer - L * d.nb;
+#pragma unroll 1
+    for (int m = first; m < (1 << kMaxD); m += step) {
+      if (m & ~on) continue;
+      int s = g.s, flip = 0, box = 0, mul = 1, rest = b;
+#pragma unroll
+      for (int k = 0; k < kMaxD; ++k)
+        if (k < d.D) {
+          int bc = rest % d.bdiv[k];
+          rest /= d.bdiv[k];
+          if ((m >> k) & 1) {
+            const bool low = g.x[k] == 1;
+            s += (low ? d.idims[k] : -d.idims[k]) * d.stride[k];  // 1 -> n + 1, n -> 0
+            bc += low ? -1 : 1;
+            if (bc < 0 || bc >= d.bdiv[k]) {
+              bc = bc < 0 ? d.bdiv[k] - 1 : 0;
+              if (d.nlayers == 2) flip ^= (d.glue_mask >> k) & 1;
+            }
+          }
+          box += bc * mul;
+          mul *= d.bdiv[k];
+        }
+      f((L ^ flip) * d.nb + box, s >> 1);
+    }
+  }
+}
+
 // Random-number site key: layer * V + i_s - 1, or the site number of
 // (x mod period) on the period lattice (identical numbers on sublattices).
 // SUB: from the coordinates in the undivided lattice, so that a divided
@@ -357,15 +402,115 @@ __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, 
     cm_update_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
   else
     cm_update(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
-  S::store(pu, Vh, ju, U);
+  for_replicas<SUB>(d, g, 0, 1, [&](int vl, int j) { S::store(plane_ptr<S>(d, vl, colour, mu), Vh, j, U); });
 }
 
+
+// ------------------------------------------------------------------ float link update, eight lanes per link
+// For lattices whose updates are bound by one thread's chain of ~2900
+// dependent instructions.  Lane l forms the l-th staple product (rows 0, 1);
+// the draws' counter-only parts of the three subgroups take one pass over the
+// lanes; then every lane sums the staples in the order of update_site and
+// runs the subgroups.  Same operations in the same order per element: the
+// links are bitwise those of the other forms.  Called by whole warps; lanes
+// without a link (valid false) run along on a repeated one.
+template <class S, bool SUB>
+__device__ __forceinline__ void update_site_lanes(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
+                                                  int jj, bool valid, uint32_t &nprop, uint32_t &nacc, float &dr) {
+  const int Vh = d.Vh, oc = colour ^ 1;
+  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
+  const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
+  const int js = g.s >> 1;
+  int offp, flp;
+  step_fwd(d, sel(g.x, mu), mu, offp, flp);
+  const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
+  const uint32_t c0 = site_key<SUB>(d, g);
+  const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
+
+  // this lane's links: issued before the draws
+  const int ns = 2 * (d.D - 1), t = l8 < ns ? l8 : 0;
+  const bool up = (t & 1) == 0;
+  int nu = t >> 1;
+  nu += nu >= mu ? 1 : 0;
+  int offn, fln, offm, flm;
+  const int xnu = sel(g.x, nu);
+  step_fwd(d, xnu, nu, offn, fln);
+  step_bwd(d, xnu, nu, offm, flm);
+  const int sn = g.s + offn, ln = lflip<SUB>(d, layer, fln);  // x + nu
+  const int sm = g.s + offm, lm = lflip<SUB>(d, layer, flm);  // x - nu
+  const int spm = sp + offm, lpm = lflip<SUB>(d, lp, flm);    // x + mu - nu
+  // upper: X = U_nu(x), Y = U_mu(x+nu), G = U_nu(x+mu); lower: X = U_mu(x-nu),
+  // Y = U_nu(x+mu-nu), G = U_nu(x-nu)
+  const M3<float> Y = S::load(up ? plane_ptr<S>(d, ln, oc, mu) : plane_ptr<S>(d, lpm, colour, nu), Vh, (up ? sn : spm) >> 1);
+  const M3<float> X = S::load2(up ? plane_ptr<S>(d, layer, colour, nu) : plane_ptr<S>(d, lm, oc, mu), Vh, (up ? g.s : sm) >> 1);
+  const M3<float> G = S::load(up ? plane_ptr<S>(d, lp, oc, nu) : plane_ptr<S>(d, lm, oc, nu), Vh, (up ? sp : sm) >> 1);
+  M3<float> U = S::load(plane_ptr<S>(d, layer, colour, mu), Vh, js);
+
+  // draws: lanes 0..2 the first proposals, lanes 3, 4 the direction blocks;
+  // then lanes 3..5 the directions
+  const int sub = l8 < 3 ? l8 : (l8 < 6 ? l8 - 3 : 0);
+  const uint32_t btag = heatbath_tag(colour, mu, l8 < 3 ? l8 : (l8 == 4 ? 2 : 0)) | (l8 < 3 ? 0u : kHitDirection);
+  const uint4 w = philox4x32_10(make_uint4(c0, sweep, btag, kPurposeHeatbath), key);
+  const int dl = base + (sub == 2 ? 4 : 3);
+  const uint32_t d0 = __shfl_sync(0xffffffffu, w.x, dl), d1 = __shfl_sync(0xffffffffu, w.y, dl);
+  const uint32_t d2 = __shfl_sync(0xffffffffu, w.z, dl), d3 = __shfl_sync(0xffffffffu, w.w, dl);
+  DrawPre mine;
+  proposal_pre_words(mine, w);
+  direction_pre_f(mine, sub == 1 ? d2 : d0, sub == 1 ? d3 : d1);
+
+  // this lane's staple
+  M3<float> M = mul_nn_2(X, Y);
+  third_row(M);
+  M3<float> P;
+  if (up)
+    P = mul_nd_2(G, M);
+  else
+    P = mul_dn_2(M, G);
+  M3<float> A = m3_zero<float>();
+#pragma unroll
+  for (int l = 0; l < 2 * (kMaxD - 1); ++l) {
+    if (l >= ns) break;
+    M3<float> q;
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+        q.e[i][j] = {__shfl_sync(0xffffffffu, P.e[i][j].re, base + l), __shfl_sync(0xffffffffu, P.e[i][j].im, base + l)};
+    acc_su3_2rows(A, q);
+  }
+
+  uint32_t np = 0, na = 0;
+  float dretr = 0.0f;
+  const float ca = 2.0f * d.beta_f / 3.0f;
+#pragma unroll
+  for (int sg = 0; sg < 3; ++sg) {
+    const int i = (sg == 2) ? 1 : 0;
+    const int j = (sg == 0) ? 1 : 2;
+    DrawPre pre;
+    pre.L = __shfl_sync(0xffffffffu, mine.L, base + sg);
+    pre.u4sq = __shfl_sync(0xffffffffu, mine.u4sq, base + sg);
+    pre.costh = __shfl_sync(0xffffffffu, mine.costh, base + 3 + sg);
+    pre.sinth = __shfl_sync(0xffffffffu, mine.sinth, base + 3 + sg);
+    pre.cphi = __shfl_sync(0xffffffffu, mine.cphi, base + 3 + sg);
+    pre.sphi = __shfl_sync(0xffffffffu, mine.sphi, base + 3 + sg);
+    cm_subgroup_f<true>(U, A, i, j, ca, d.hits, key, c0, sweep, heatbath_tag(colour, mu, sg), pre, np, na, dretr);
+    __syncwarp();
+  }
+  if (!valid) return;
+  if (l8 == 0) {
+    nprop += np;
+    nacc += na;
+    dr = dretr;
+  }
+  for_replicas<SUB>(d, g, l8, 8, [&](int vl, int j) { S::store(plane_ptr<S>(d, vl, colour, mu), Vh, j, U); });
+}
 
 // ------------------------------------------------------------------ FP64 link update in fixed point
 // The one-coupling FP64 update with its linear algebra (staples, projections,
 // rotations) in the integers of su3_fixed.cuh.
 
 // Row `row` of a stored FP64 link in fixed point.
+template <bool COH = false>
 __device__ __forceinline__ void load_row_f(const StoreF64x18::Vec *plane, int Vh, int jj, int row, Fc (&r)[3],
                                            FxRange &rg) {
   if (!in_bounds(jj, Vh, kBoundsIndex)) {
@@ -373,15 +518,16 @@ __device__ __forceinline__ void load_row_f(const StoreF64x18::Vec *plane, int Vh
     return;
   }
   const double2 *p = plane + jj + 3 * row * Vh;
-  const double2 q0 = __ldg(p), q1 = __ldg(p + Vh), q2 = __ldg(p + 2 * Vh);
+  const double2 q0 = ld_link<COH>(p), q1 = ld_link<COH>(p + Vh), q2 = ld_link<COH>(p + 2 * Vh);
   r[0] = fc_of(q0.x, q0.y, rg);
   r[1] = fc_of(q1.x, q1.y, rg);
   r[2] = fc_of(q2.x, q2.y, rg);
 }
 
+template <bool COH = false>
 __device__ __forceinline__ void load_f(const StoreF64x18::Vec *plane, int Vh, int jj, FM3 &m, FxRange &rg) {
 #pragma unroll
-  for (int i = 0; i < 3; ++i) load_row_f(plane, Vh, jj, i, m.e[i], rg);
+  for (int i = 0; i < 3; ++i) load_row_f<COH>(plane, Vh, jj, i, m.e[i], rg);
 }
 
 // The draw of one subgroup in double, out of line: proposals with too few
@@ -402,7 +548,7 @@ static __device__ __noinline__ DrawD su2_draw_general(double alpha, int hits, ui
 // The three links of one staple (staple_f): rows 0, 1 of X, all of Y and G.
 // t counts the 2 (D - 1) staples: the upper ones of the other directions in
 // order, then the lower ones.
-template <bool SUB>
+template <bool SUB, bool COH>
 __device__ __forceinline__ void staple_fixed(const ChainDesc &d, const SiteGeo &g, int colour, int mu, int t, int sp,
                                              int lp, FSum &A, FxRange &rg) {
   using S = StoreF64x18;
@@ -423,10 +569,10 @@ __device__ __forceinline__ void staple_fixed(const ChainDesc &d, const SiteGeo &
   const int jy = (up ? sn : spm) >> 1, jx = (up ? g.s : sm) >> 1, jg = (up ? sp : sm) >> 1;
   FM3 Y, G;
   Fc X[2][3];
-  load_f(py, Vh, jy, Y, rg);
-  load_row_f(px, Vh, jx, 0, X[0], rg);
-  load_row_f(px, Vh, jx, 1, X[1], rg);
-  load_f(pg, Vh, jg, G, rg);
+  load_f<COH>(py, Vh, jy, Y, rg);
+  load_row_f<COH>(px, Vh, jx, 0, X[0], rg);
+  load_row_f<COH>(px, Vh, jx, 1, X[1], rg);
+  load_f<COH>(pg, Vh, jg, G, rg);
   staple_f(A, X, Y, G, up, rg);
 }
 
@@ -540,14 +686,14 @@ struct UpdateCount {
 
 // The double-precision update of one site, out of line: links outside the
 // fixed-point range only.
-template <bool SUB>
+template <bool SUB, bool COH>
 __device__ __noinline__ UpdateCount update_site_f64_general(const ChainDesc *d, uint32_t sweep, int colour, int mu,
                                                             int layer, int jj) {
   UpdateCount u = {0, 0, 0.0};
   if constexpr (SUB)
-    update_site<StoreF64x18, false, false, true>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
+    update_site<StoreF64x18T<COH>, false, false, true>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
   else
-    update_site_lean<StoreF64x18, false>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
+    update_site_lean<StoreF64x18T<COH>, false>(*d, sweep, colour, mu, layer, jj, u.nprop, u.nacc, u.dretr);
   return u;
 }
 
@@ -574,12 +720,12 @@ __device__ __forceinline__ void update_site_fixed(const ChainDesc &d, uint32_t s
   // one staple at a time: its instructions once, not six times, in the
   // instruction cache
 #pragma unroll 1
-  for (int t = 0; t < 2 * (d.D - 1); ++t) staple_fixed<SUB>(d, g, colour, mu, t, sp, lp, A, rg);
+  for (int t = 0; t < 2 * (d.D - 1); ++t) staple_fixed<SUB, false>(d, g, colour, mu, t, sp, lp, A, rg);
   S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
   FM3 U;
   load_f(pu, Vh, js, U, rg);
   if (!rg.ok()) {
-    const UpdateCount u = update_site_f64_general<SUB>(&d, sweep, colour, mu, layer, jj);
+    const UpdateCount u = update_site_f64_general<SUB, false>(&d, sweep, colour, mu, layer, jj);
     nprop += u.nprop;
     nacc += u.nacc;
     dr.general = u.dretr;
@@ -592,12 +738,17 @@ __device__ __forceinline__ void update_site_fixed(const ChainDesc &d, uint32_t s
   // a link none of whose subgroups accepted keeps its bits
   if (nacc != before && in_bounds(js, Vh, kBoundsIndex)) {
     // the rows lie in the order 1, 2, 0 after the last subgroup
-    S::Vec *p = pu + js;
+    double2 v[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) {
       const Fc e = U.e[(q / 3 + 2) % 3][q % 3];
-      p[q * Vh] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
+      v[q] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
     }
+    for_replicas<SUB>(d, g, 0, 1, [&](int vl, int j) {
+      S::Vec *p = plane_ptr<S>(d, vl, colour, mu) + j;
+#pragma unroll
+      for (int q = 0; q < 9; ++q) p[q * Vh] = v[q];
+    });
   }
 }
 
@@ -617,7 +768,7 @@ __device__ __forceinline__ int64_t shfl_xor_ll(int64_t a, int m) {
 // column of U each in the projections and rotations.  Results are bitwise
 // those of update_site_fixed.  Called by whole warps; lanes without a link
 // (valid false) run along on a repeated one.
-template <bool SUB>
+template <bool SUB, bool COH = false>
 __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
                                                  int jj, bool valid, uint32_t &nprop, uint32_t &nacc,
                                                  ActionChange &dr) {
@@ -657,7 +808,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
   FSum A = {};
   FxRange rg;
   const int ns = 2 * (d.D - 1);
-  staple_fixed<SUB>(d, g, colour, mu, l8 < ns ? l8 : 0, sp, lp, A, rg);
+  staple_fixed<SUB, COH>(d, g, colour, mu, l8 < ns ? l8 : 0, sp, lp, A, rg);
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -678,7 +829,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
 #pragma unroll
   for (int r = 0; r < 3; ++r) {
     double2 q = make_double2(0.0, 0.0);
-    if (in_bounds(js, Vh, kBoundsIndex)) q = __ldg(pu + js + (3 * r + cc) * Vh);
+    if (in_bounds(js, Vh, kBoundsIndex)) q = ld_link<COH>(pu + js + (3 * r + cc) * Vh);
     u[r] = fc_of(q.x, q.y, rg);
     const int64_t re = cc == 0 ? A.re[0][r] : (cc == 1 ? A.re[1][r] : A.re[2][r]);
     const int64_t im = cc == 0 ? A.im[0][r] : (cc == 1 ? A.im[1][r] : A.im[2][r]);
@@ -755,7 +906,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
   if (!valid) return;
   if (bad) {
     if (l8 == 0) {
-      const UpdateCount uc = update_site_f64_general<SUB>(&d, sweep, colour, mu, layer, jj);
+      const UpdateCount uc = update_site_f64_general<SUB, COH>(&d, sweep, colour, mu, layer, jj);
       nprop += uc.nprop;
       nacc += uc.nacc;
       dr.general = uc.dretr;
@@ -769,11 +920,17 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
   }
   // after the last swap the rows lie in the order 0, 2, 1
   if (l8 < 3 && na && in_bounds(js, Vh, kBoundsIndex)) {
+    double2 v[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
       const Fc e = u[r == 0 ? 0 : 3 - r];
-      pu[js + (3 * r + c) * Vh] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
+      v[r] = make_double2(dbl_of(fx_val(e.re), 60), dbl_of(fx_val(e.im), 60));
     }
+    for_replicas<SUB>(d, g, 0, 1, [&](int vl, int j) {
+      S::Vec *p = plane_ptr<S>(d, vl, colour, mu) + j + c * Vh;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) p[3 * r * Vh] = v[r];
+    });
   }
 }
 
@@ -1274,6 +1431,36 @@ __device__ __forceinline__ void restart_bookkeeping(const ChainDesc &d, const do
   for (int i = lane; i < d.n_action_slots; i += 32) d.action_slots[i] = 0.0;
 }
 
+// ------------------------------------------------------------------ halos
+
+// Entry `e` of the halo list: the links of one halo site of box vl, copied from the site that owns them (the same padded site of
+// the neighbouring box given by the entry's offset code, whose box coordinate
+// wraps periodically; a wrap across a glued boundary of the double-layered
+// torus lands in the other layer).  Halo sites are never sources, so the
+// copies do not race.
+template <class S>
+__device__ __forceinline__ void halo_copy(const ChainDesc &d, int vl, int e) {
+  const int4 h = d.halo[e];
+  const int colour = e < d.halo_n[0] ? 0 : 1, L = vl / d.nb;
+  int bsrc = 0, bmul = 1, flip = 0, rest = vl - L * d.nb;
+#pragma unroll
+  for (int k = 0; k < kMaxD; ++k)
+    if (k < d.D) {
+      const int code = (h.z >> (2 * k)) & 3, bc = rest % d.bdiv[k];
+      rest /= d.bdiv[k];
+      int o = bc + (code == 1 ? -1 : (code == 2 ? 1 : 0));
+      if (o < 0 || o >= d.bdiv[k]) {
+        o = o < 0 ? o + d.bdiv[k] : o - d.bdiv[k];
+        if (d.nlayers == 2) flip ^= (d.glue_mask >> k) & 1;
+      }
+      bsrc += o * bmul;
+      bmul *= d.bdiv[k];
+    }
+  const int vsrc = (L ^ flip) * d.nb + bsrc;
+  for (int mu = 0; mu < d.D; ++mu)
+    S::copy(plane_ptr<S>(d, vl, colour, mu), d.Vh, h.x >> 1, plane_ptr<S>(d, vsrc, colour, mu), d.Vh, h.y >> 1);
+}
+
 // Warp-sum the FHKP counters and add them to the chain's totals (one of
 // kCounterSlots pairs: warps that end together meet on different addresses).
 __device__ __forceinline__ void flush_counters(const ChainDesc &d, uint32_t &np, uint32_t &na) {
@@ -1301,7 +1488,7 @@ __device__ __forceinline__ void flush_counters(const ChainDesc &d, uint32_t &np,
 // measuring: a split into a staple kernel and a heatbath kernel (30 %
 // slower), an L1 prefetch of the next staple direction's links (8 %).
 template <int V> struct TickBounds;
-constexpr int kCoopVariant = 11;
+constexpr int kCoopVariant = 11, kLanesVariant = 12;
 template <> struct TickBounds<0> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };   // FP32, 128 regs
 template <> struct TickBounds<1> { static constexpr int kThreads = 128, kMinBlocks = 5; static constexpr bool kRolled = false; };   // FP32, 96 regs
 template <> struct TickBounds<2> { static constexpr int kThreads = 128, kMinBlocks = 5; static constexpr bool kRolled = true; };    // FP32, rolled, 96 regs
@@ -1310,59 +1497,87 @@ template <> struct TickBounds<4> { static constexpr int kThreads = 256, kMinBloc
 template <> struct TickBounds<10> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64
 template <> struct TickBounds<kCoopVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64, eight lanes per link
 
+template <> struct TickBounds<kLanesVariant> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };  // FP32, eight lanes per link
+
 // ------------------------------------------------------------------ one tile of an update phase
 
-// The updates of one CTA's tile lt of a chain's phase (colour, mu), with the
-// booking of the action change: each warp owns the slot of its links, so the
-// one fire-and-forget add per warp meets no other add in this launch and the
-// order of adds is fixed.
+// Book a warp's change of Re Tr(U A): each warp owns the slot of its links, so
+// the one fire-and-forget add per warp meets no other add in this launch and
+// the order of adds is fixed.
+__device__ __forceinline__ void book_action(const ChainDesc &d, int slot, double sum) {
+  if ((threadIdx.x & 31) == 0 && d.action_slots && in_bounds(slot, d.n_action_slots, kBoundsSlot))
+    atomicAdd(d.action_slots + slot, d.action_factor * sum);
+}
+__device__ __forceinline__ double warp_sum(ActionChange dr) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) dr.v += __shfl_down_sync(0xffffffffu, (long long)dr.v, o);
+  double sum = dbl_of(dr.v, 49);
+  if (__any_sync(0xffffffffu, dr.general != 0.0)) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dr.general += __shfl_down_sync(0xffffffffu, dr.general, o);
+    sum += dr.general;
+  }
+  return sum;
+}
+
+// The links j0.. of one warp with eight lanes per link (slot: the warp's).
+template <class S, bool SUB, bool COH>
+__device__ __forceinline__ void update_warp(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer, int j0,
+                                            int slot, uint32_t &np, uint32_t &na) {
+  if (j0 >= d.Vn) return;
+  const int jj = j0 + (int)(threadIdx.x & 31) / kCoopLanes, jc = min(jj, d.Vn - 1);
+  if constexpr (sizeof(typename S::R) == 8) {
+    ActionChange dr = {0, 0.0};
+    update_site_coop<SUB, COH>(d, sweep, colour, mu, layer, jc, jj < d.Vn, np, na, dr);
+    __syncwarp();
+    book_action(d, slot, warp_sum(dr));
+  } else {
+    float dr = 0.0f;
+    update_site_lanes<S, SUB>(d, sweep, colour, mu, layer, jc, jj < d.Vn, np, na, dr);
+    __syncwarp();
+#pragma unroll
+    for (int o = 16; o >= kCoopLanes; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
+    book_action(d, slot, (double)dr);
+  }
+}
+
+// The updates of one CTA's tile lt of a chain's phase (colour, mu).
 template <class S, int V, bool WT, bool SUB, bool TOR>
 __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, int colour, int mu, int lt,
                                             uint32_t &np, uint32_t &na) {
-  // the one-coupling FP64 update runs in fixed point, with kLanes lanes per link
-  constexpr bool kFixed = std::is_same<S, StoreF64x18>::value && !WT;
-  constexpr int kLanes = V == kCoopVariant ? kCoopLanes : 1;
+  constexpr int kLanes = V == kCoopVariant || V == kLanesVariant ? kCoopLanes : 1, kPerWarp = 32 / kLanes;
   const int layer = lt / d.tiles_per_vl;  // a layer, or a sublattice box of one
   const int j0 = (lt - layer * d.tiles_per_vl) * ((int)blockDim.x / kLanes);
-  const int jj = j0 + (int)threadIdx.x / kLanes;
-  const bool valid = jj < d.Vn;
   const int jw = j0 + (int)(threadIdx.x & ~31u) / kLanes;  // the first link of the warp
-  constexpr int kPerWarp = 32 / kLanes;
-  double sum;  // lane 0: the change of Re Tr(U A) over the warp's links
-  if constexpr (kFixed) {
-    ActionChange dr = {0, 0.0};
-    if constexpr (kLanes > 1) {
-      if (jw < d.Vn) update_site_coop<SUB>(d, sweep, colour, mu, layer, min(jj, d.Vn - 1), valid, np, na, dr);
-    } else {
-      if (valid) update_site_fixed<SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dr.v += __shfl_down_sync(0xffffffffu, (long long)dr.v, o);
-    sum = dbl_of(dr.v, 49);
-    if (__any_sync(0xffffffffu, dr.general != 0.0)) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) dr.general += __shfl_down_sync(0xffffffffu, dr.general, o);
-      sum += dr.general;
-    }
+  const int slot = layer * ((d.Vn + kPerWarp - 1) / kPerWarp) + jw / kPerWarp;
+  if constexpr (kLanes > 1) {
+    update_warp<S, SUB, false>(d, sweep, colour, mu, layer, jw, slot, np, na);
   } else {
-    typename S::R dr = 0;  // in the kernel's precision
-    if (valid) {
-      if constexpr (TOR)
-        update_site_lean<S, false, 4>(d, sweep, colour, mu, layer, jj, np, na, dr);
-      else if constexpr (!TickBounds<V>::kRolled && !SUB)
-        update_site_lean<S, WT>(d, sweep, colour, mu, layer, jj, np, na, dr);
-      else
-        update_site<S, TickBounds<V>::kRolled, WT, SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
-    }
+    const int jj = j0 + (int)threadIdx.x;
+    const bool valid = jj < d.Vn;
+    double sum;
+    // the one-coupling FP64 update runs in fixed point
+    if constexpr (std::is_same<S, StoreF64x18>::value && !WT) {
+      ActionChange dr = {0, 0.0};
+      if (valid) update_site_fixed<SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
+      __syncwarp();
+      sum = warp_sum(dr);
+    } else {
+      typename S::R dr = 0;  // in the kernel's precision
+      if (valid) {
+        if constexpr (TOR)
+          update_site_lean<S, false, 4>(d, sweep, colour, mu, layer, jj, np, na, dr);
+        else if constexpr (!TickBounds<V>::kRolled && !SUB)
+          update_site_lean<S, WT>(d, sweep, colour, mu, layer, jj, np, na, dr);
+        else
+          update_site<S, TickBounds<V>::kRolled, WT, SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
+      }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
-    sum = (double)dr;
-  }
-  // (a warp of the ragged last tile with no link has no slot)
-  if ((threadIdx.x & 31) == 0 && jw < d.Vn && d.action_slots) {
-    const int slot = layer * ((d.Vn + kPerWarp - 1) / kPerWarp) + jw / kPerWarp;
-    if (in_bounds(slot, d.n_action_slots, kBoundsSlot)) atomicAdd(d.action_slots + slot, d.action_factor * sum);
+      for (int o = 16; o > 0; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
+      sum = (double)dr;
+    }
+    // (a warp of the ragged last tile with no link has no slot)
+    if (jw < d.Vn) book_action(d, slot, sum);
   }
 }
 

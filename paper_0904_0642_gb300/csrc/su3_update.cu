@@ -31,6 +31,40 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
   flush_counters(d, np, na);
 }
 
+// Whole sweeps of a small lattice in one launch of one thread-block cluster
+// (eight lanes per link): the phases are separated by the cluster's hardware
+// barrier instead of a kernel boundary, and the code stays in the instruction
+// caches.  Links are read through L2 (COH): other CTAs have written them.
+__device__ __forceinline__ void cluster_barrier() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <class S, bool SUB>
+__global__ void __launch_bounds__(kClusterThreads, 1)
+    k_sweeps(const __grid_constant__ ChainDesc d, ChainCtl *ctl, int sweeps) {
+  wait_previous();
+  const uint32_t base = __ldcg(&ctl->nxt);
+  constexpr int kPerWarp = 32 / kCoopLanes;
+  const int per_vl = (d.Vn + kPerWarp - 1) / kPerWarp, warps = d.nlayers * d.nb * per_vl;
+  const int w0 = (int)(blockIdx.x * blockDim.x + threadIdx.x) / 32, nw = (int)(gridDim.x * blockDim.x) / 32;
+  uint32_t np = 0, na = 0;
+#pragma unroll 1
+  for (int i = 0; i < sweeps * 2 * d.D; ++i) {
+    const int s = i / (2 * d.D), st = i - s * 2 * d.D;
+    const int colour = st >= d.D ? 1 : 0, mu = st - colour * d.D;
+#pragma unroll 1
+    for (int w = w0; w < warps; w += nw) {
+      const int vl = w / per_vl, j0 = (w - vl * per_vl) * kPerWarp;
+      update_warp<S, SUB, true>(d, base + (uint32_t)s, colour, mu, vl, j0, w, np, na);
+    }
+    cluster_barrier();
+  }
+  flush_counters(d, np, na);
+  if (blockIdx.x == 0 && threadIdx.x == 0) ctl->nxt = base + (uint32_t)sweeps;
+}
+
 // One thread per link: blockIdx.z = colour D + mu, blockIdx.y a (virtual) layer.
 template <class S, bool SUB>
 __global__ void __launch_bounds__(128) k_reunit(const __grid_constant__ ChainDesc d) {
@@ -179,6 +213,13 @@ static cudaError_t update_dispatch(int storage, int variant, bool sub, bool toru
                  : OP<StoreF64x18, kCoopVariant, false, false, false>::run(a...);
     return sub ? OP<StoreF64x18, 10, WT, true, false>::run(a...) : OP<StoreF64x18, 10, WT, false, false>::run(a...);
   }
+  if (variant == kFloatLanes && !WT) {
+    if (storage == 2)
+      return sub ? OP<StoreF32x18, kLanesVariant, false, true, false>::run(a...)
+                 : OP<StoreF32x18, kLanesVariant, false, false, false>::run(a...);
+    return sub ? OP<StoreF32x12, kLanesVariant, false, true, false>::run(a...)
+               : OP<StoreF32x12, kLanesVariant, false, false, false>::run(a...);
+  }
   if (storage == 2) {
     if (sub) return OP<StoreF32x18, kSubVariant, WT, true, false>::run(a...);
     return tor ? OP<StoreF32x18, 0, false, false, kT>::run(a...) : OP<StoreF32x18, 0, WT, false, false>::run(a...);
@@ -195,7 +236,7 @@ static cudaError_t update_dispatch(int storage, int variant, bool sub, bool toru
 
 cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, bool torus, const ChainDesc &d,
                           ChainCtl *ctl, const UpdateStep &step, int grid, int block, cudaStream_t st, bool pdl) {
-  if (sub && storage != 0) variant = kSubVariant;
+  if (sub && storage != 0 && variant != kFloatLanes) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaErrorInvalidConfiguration;
   const ChainDesc *pd = &d;
   const UpdateStep *pu = &step;
@@ -206,10 +247,65 @@ cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, boo
 cudaError_t update_occupancy(int storage, int variant, bool weighted, bool sub, bool torus, int block,
                              int *ctas_per_sm) {
   *ctas_per_sm = 0;
-  if (sub && storage != 0) variant = kSubVariant;
+  if (sub && storage != 0 && variant != kFloatLanes) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaSuccess;
   return weighted ? update_dispatch<UpdateOccupancy, true>(storage, variant, sub, torus, block, ctas_per_sm)
                   : update_dispatch<UpdateOccupancy, false>(storage, variant, sub, torus, block, ctas_per_sm);
+}
+
+// The largest cluster the device takes for k_sweeps (0: none).
+template <class K>
+static int cluster_ctas(K *kernel, int threads) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kClusterCtas);
+  cfg.blockDim = dim3((unsigned)threads);
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {kClusterCtas, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n > 0 ? kClusterCtas : 0;
+}
+
+// f(kernel) with the k_sweeps form of a storage.
+template <class F>
+static auto by_sweeps(int storage, bool sub, F &&f) {
+  if (storage == 0) return sub ? f(k_sweeps<StoreF64x18T<true>, true>) : f(k_sweeps<StoreF64x18T<true>, false>);
+  if (storage == 2) return sub ? f(k_sweeps<StoreF32x18T<true>, true>) : f(k_sweeps<StoreF32x18T<true>, false>);
+  return sub ? f(k_sweeps<StoreF32x12T<true>, true>) : f(k_sweeps<StoreF32x12T<true>, false>);
+}
+
+bool sweeps_supported(int storage, bool sub) {
+  return by_sweeps(storage, sub, [](auto *k) { return cluster_ctas(k, kClusterThreads); }) > 0;
+}
+
+cudaError_t launch_sweeps(int storage, bool sub, const ChainDesc &d, ChainCtl *ctl, int sweeps, cudaStream_t st,
+                          bool pdl) {
+  // as many threads as the links need lanes (whole warps), up to the limit
+  const int warps = d.nlayers * d.nb * ((d.Vn + 3) / 4);
+  const int per = (warps + kClusterCtas - 1) / kClusterCtas;
+  const int threads = 32 * (per < kClusterThreads / 32 ? per : kClusterThreads / 32);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kClusterCtas);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim = {kClusterCtas, 1, 1};
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return by_sweeps(storage, sub, [&](auto *k) { return cudaLaunchKernelEx(&cfg, k, d, ctl, sweeps); });
 }
 
 cudaError_t launch_reunit(int storage, bool sub, const ChainDesc &d, cudaStream_t st, bool pdl) {
