@@ -419,6 +419,11 @@ static void fill_desc(Chain &ch, int tile) {
     d.tiles_per_layer = nb * d.tiles_per_vl;
     d.pow2 = 0;
   }
+  for (int i = 0; i < kMaxD; ++i) {
+    d.idiv[i] = fast_div_of((uint32_t)d.idims[i]);
+    d.bdivf[i] = fast_div_of((uint32_t)d.bdiv[i]);
+  }
+  d.tdiv = fast_div_of((uint32_t)d.tiles_per_vl);
 
   d.beta_f = (float)c.beta;
   d.beta_d = c.beta;

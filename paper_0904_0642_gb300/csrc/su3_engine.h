@@ -73,6 +73,17 @@ constexpr int kMeasVals = 5;
 // Partial sums per tile in a measurement: [space, time, poly_re, poly_im].
 constexpr int kPartVals = 4;
 
+// Division of 0 <= r < 2^31 by a number fixed on the host: (hi(m r) + r) >> s
+// (Granlund and Montgomery; three instructions instead of about twenty).
+struct FastDiv {
+  uint32_t m, s;
+};
+inline FastDiv fast_div_of(uint32_t n) {
+  uint32_t s = 0;
+  while (s < 31 && (1u << s) < n) ++s;
+  return {(uint32_t)((((1ull << s) - n) << 32) / n + 1), s};
+}
+
 struct ChainDesc {
   void *links;               // storage base (Vec units, see su3_device.cuh)
   double *results;           // [result_cap][nlayers + 1][kMeasVals]
@@ -111,6 +122,8 @@ struct ChainDesc {
   int32_t hpad[kMaxD];       // 1: divided direction, one halo layer on each side
   int32_t bdiv[kMaxD];       // sublattices per direction
   int32_t gstride[kMaxD];    // strides of the undivided layer
+  FastDiv idiv[kMaxD], bdivf[kMaxD];  // division by idims, bdiv
+  FastDiv tdiv;              // division by tiles_per_vl
   // Halo sites of a box (the same for every box), colour 0 first then
   // colour 1: {padded index, owner's padded index, owner box offset code
   // (2 bits per direction: 0 same box, 1 previous, 2 next), 0}.

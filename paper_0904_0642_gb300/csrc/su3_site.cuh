@@ -18,6 +18,10 @@ struct SiteGeo {
   int layer;
 };
 
+__device__ __forceinline__ int fast_div(int r, const FastDiv &f) {
+  return (int)((__umulhi(f.m, (uint32_t)r) + (uint32_t)r) >> f.s);
+}
+
 // Coordinates of the site of colour `colour` at checkerboard index jj
 // (eqs. xD, x^i, i_c): the even lexicographic index 2 jj shares its row
 // with the odd one, and the colour fixes which of the two it is.
@@ -33,7 +37,7 @@ __device__ __forceinline__ SiteGeo site_of(const ChainDesc &d, int layer, int co
     for (int i = 0; i < kMaxD; ++i) {
       if (i < d.D) {
         const int n = d.idims[i];
-        const int q = r / n;
+        const int q = fast_div(r, d.idiv[i]);
         g.x[i] = r - q * n;
         r = q;
         if (i > 0) par += g.x[i];
@@ -71,7 +75,7 @@ __device__ __forceinline__ SiteGeo site_of(const ChainDesc &d, int layer, int co
     for (int i = 0; i < kMaxD; ++i) {
       if (i < d.D) {
         const int n = d.dims[i];
-        const int q = r / n;
+        const int q = fast_div(r, d.idiv[i]);
         g.x[i] = r - q * n;
         r = q;
         if (i > 0) par += g.x[i];
@@ -154,8 +158,9 @@ __device__ __forceinline__ void for_replicas(const ChainDesc &d, const SiteGeo &
 #pragma unroll
       for (int k = 0; k < kMaxD; ++k)
         if (k < d.D) {
-          int bc = rest % d.bdiv[k];
-          rest /= d.bdiv[k];
+          const int rq = fast_div(rest, d.bdivf[k]);
+          int bc = rest - rq * d.bdiv[k];
+          rest = rq;
           if ((m >> k) & 1) {
             const bool low = g.x[k] == 1;
             s += (low ? d.idims[k] : -d.idims[k]) * d.stride[k];  // 1 -> n + 1, n -> 0
@@ -187,8 +192,8 @@ __device__ __forceinline__ uint32_t site_key(const ChainDesc &d, const SiteGeo &
 #pragma unroll
     for (int i = 0; i < kMaxD; ++i)
       if (i < d.D) {
-        const int bc = b % d.bdiv[i];
-        b /= d.bdiv[i];
+        const int q = fast_div(b, d.bdivf[i]), bc = b - q * d.bdiv[i];
+        b = q;
         const int gx = bc * d.idims[i] + g.x[i] - d.hpad[i];
         key += d.custom_period ? (gx % d.period[i]) * d.pstride[i] : gx * d.gstride[i];
       }
@@ -1546,7 +1551,7 @@ template <class S, int V, bool WT, bool SUB, bool TOR>
 __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, int colour, int mu, int lt,
                                             uint32_t &np, uint32_t &na) {
   constexpr int kLanes = V == kCoopVariant || V == kLanesVariant ? kCoopLanes : 1, kPerWarp = 32 / kLanes;
-  const int layer = lt / d.tiles_per_vl;  // a layer, or a sublattice box of one
+  const int layer = fast_div(lt, d.tdiv);  // a layer, or a sublattice box of one
   const int j0 = (lt - layer * d.tiles_per_vl) * ((int)blockDim.x / kLanes);
   const int jw = j0 + (int)(threadIdx.x & ~31u) / kLanes;  // the first link of the warp
   const int slot = layer * ((d.Vn + kPerWarp - 1) / kPerWarp) + jw / kPerWarp;
