@@ -167,8 +167,7 @@ SU3_HD int clz32(uint32_t x) {
 // floor(x 2^60) by integer operations, for |x| < 2 (a range check rejects
 // others): the mantissa with its leading bit at bit 63, shifted right by
 // 1026 - e (zero and subnormals shift out), negative values as the ones'
-// complement.  The conversion instruction is emulated on this GPU in about
-// four times as many instructions.
+// complement.
 SU3_HD Fx fx_of_mantissa(uint32_t H, uint32_t L, int q, uint32_t s) {
   const int q2 = q > 32 ? q - 32 : 0;
   const uint32_t vh = shr0(H, (uint32_t)q) ^ s;
@@ -208,6 +207,23 @@ SU3_HD double dbl_of(int64_t v, int e) {
   const uint32_t carry = (uint32_t)(m >> 63) ^ 1u;
   const uint32_t hi = s | (((uint32_t)(1023 + 62 - lz - e + (int)carry) << 20) + ((uint32_t)(m >> 43) | (carry << 20)));
   return v == 0 ? 0.0 : dbl_make(hi, (uint32_t)(m >> 11));
+}
+
+// Both by the conversion instructions, which run on the FP64 pipe (16 clocks
+// of the SM per warp) beside the integer pipes: faster where many warps wait
+// on little else (re-unitarisation of 24^4 FP64 links: 101 -> 81 us), slower
+// in the update (225 -> 272 us) and the measurement (296 -> 380 us), whose
+// few warps wait for them.
+SU3_HD Fx fx_of_pipe(double x) {
+#ifdef __CUDA_ARCH__
+  return fx_split(__double2ll_rz(dbl_make((uint32_t)dbl_hi(x) + (60u << 20), dbl_lo(x))));
+#else
+  return fx_of(x);
+#endif
+}
+SU3_HD double dbl_of_pipe(int64_t v, int e) {
+  const double d = (double)v;
+  return v == 0 ? 0.0 : dbl_make((uint32_t)dbl_hi(d) - ((uint32_t)e << 20), dbl_lo(d));
 }
 
 SU3_HD Fc fc_of(double re, double im, FxRange &rg) {
@@ -501,9 +517,9 @@ SU3_HD int64_t neg_log_fx(uint32_t w) {
   const int32_t w5 = 1431655765 - (int32_t)(((int64_t)r * 19173961) >> 32);  // 2^-33
   const int32_t w4 = 1717986918 - (int32_t)(((int64_t)r * w5) >> 38);        // 2^-33
   const int32_t w3 = (1 << 30) - (int32_t)(((int64_t)r * w4) >> 39);         // 2^-32
-  const int64_t w2 = 384307168202282325ll - (((int64_t)r * w3) >> 10);       // 2^-60
+  const int32_t w2 = 1431655765 - (int32_t)(((int64_t)r * w3) >> 38);        // 2^-32
   const Fx rf = fx_split(r60);
-  const int64_t q = (1ll << 59) - fx_mul(rf, fx_split(w2));
+  const int64_t q = (1ll << 59) - (((int64_t)r * w2) >> 10);                 // 2^-60
   const int64_t ln1p = r60 - fx_mul(rf, fx_split(fx_mul(rf, fx_split(q))));
   return z * kLn2_57 + ((t.b - ln1p + 4) >> 3);
 }

@@ -636,9 +636,11 @@ __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, cons
     a2[k] = A.e[k][2];
   }
   dretr2 = 0;
+  uint4 dir = {};  // the direction block: subgroups 0 and 1 share one (direction_words)
 #pragma unroll 1
   for (int sg = 0; sg < 3; ++sg) {
     const uint32_t tag = heatbath_tag(colour, mu, sg);
+    if (sg != 1) dir = philox4x32_10(make_uint4(c0, c1, tag | kHitDirection, kPurposeHeatbath), key);
     FxAcc s[4] = {{0, kHalf60}, {0, kHalf60}, {0, kHalf60}, {0, kHalf60}};
 #pragma unroll
     for (int k = 0; k < 3; ++k) project_k_f(s, u0[k], u1[k], a0[k], a1[k]);
@@ -651,7 +653,7 @@ __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, cons
       Fx x[4];
       bool accepted = st == kAccepted;
       if (accepted) {
-        direction_fx(p, direction_of(direction_words(key, c0, c1, tag)), x);
+        direction_fx(p, direction_of(sg == 1 ? make_uint2(dir.z, dir.w) : make_uint2(dir.x, dir.y)), x);
       } else if (st == kInDouble) {
         const DrawD r = su2_draw_general(2.0 * d.beta_d / 3.0 * dbl_of(n.kappa, 57 + n.s), hits, key, c0, c1, tag);
         h = (int)r.nprop;
@@ -1054,7 +1056,8 @@ __device__ __forceinline__ void reunit_link(typename S::Vec *p, int Vh, int js) 
         rg.doubles(__float_as_int(m.e[i][k].re), __float_as_int(m.e[i][k].im));
         f.e[i][k] = {fx_of(m.e[i][k].re), fx_of(m.e[i][k].im)};
       } else {
-        f.e[i][k] = fc_of(m.e[i][k].re, m.e[i][k].im, rg);
+        rg.doubles(dbl_hi(m.e[i][k].re), dbl_hi(m.e[i][k].im));
+        f.e[i][k] = {fx_of_pipe(m.e[i][k].re), fx_of_pipe(m.e[i][k].im)};
       }
     }
   const bool in = rg.ok(sizeof(R) == 4 ? kElemMaxFloat : kElemMaxHi);
@@ -1075,7 +1078,7 @@ __device__ __forceinline__ void reunit_link(typename S::Vec *p, int Vh, int js) 
         if constexpr (sizeof(R) == 4)
           m.e[i][k] = {flt_of(re), flt_of(im)};
         else
-          m.e[i][k] = {dbl_of(re, 60), dbl_of(im, 60)};
+          m.e[i][k] = {dbl_of_pipe(re, 60), dbl_of_pipe(im, 60)};
       }
     S::store(p, Vh, js, m);
     return;

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(128) k_reunit(const __grid_constant__ ChainDes
 // per site (SPLIT: lattices that do not fill the GPU with a site per thread).
 // The last CTA to finish sums the CTAs' partial sums in a fixed order.
 template <class S, bool SUB, bool SPLIT>
-__global__ void __launch_bounds__(128) k_measure(const __grid_constant__ ChainDesc d, double *out, ChainCtl *ctl,
+__global__ void __launch_bounds__(128, sizeof(typename S::R) == 8 ? 3 : 5) k_measure(const __grid_constant__ ChainDesc d, double *out, ChainCtl *ctl,
                                                  int record) {
   __shared__ double s_red[32];
   __shared__ double s_sum[3][kPartVals];
