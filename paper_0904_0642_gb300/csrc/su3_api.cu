@@ -456,6 +456,8 @@ struct Engine {
   bool weighted_any = false;  // some chain has two couplings: the update's weighted form
   bool sub_any = false;       // the (only) chain is divided into sublattice boxes
   bool torus_all = false;     // every chain is an undivided periodic 4-D torus, one coupling, default key
+  static constexpr int kAutoCtas = -1;  // until set_launch: by the rule in grid_size
+  int resident = 0;           // CTAs of the update kernel that fit the GPU (0: not known)
   bool cluster = false;       // fixed, fewest links: whole sweeps per launch (k_sweeps)
   bool coop = false;          // too few links to fill the GPU: eight lanes per link
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
@@ -485,7 +487,7 @@ struct Engine {
   double *d_meas_out = nullptr;  // stand-alone measurement results
   double *h_pinned = nullptr;    // small pinned staging (results, counters)
   int block = 128;
-  int ctas_per_sm = 0;
+  int ctas_per_sm = kAutoCtas;
   int variant = 0;  // register variant of the tick kernel (launch_tick)
   int total_tiles = 0;
   bool use_graph = true;
@@ -842,6 +844,7 @@ struct Engine {
       torus_all = tor;
       drop_graph();
     }
+    if (ctas_per_sm == kAutoCtas) TRY(count_resident());
     if (chains.size() > chain_cap) {
       cudaFree(d_desc);
       cudaFree(d_state);
@@ -938,14 +941,37 @@ struct Engine {
 
   // ctas_per_sm = 0: one CTA per tile (the hardware balances the tail);
   // > 0: a persistent grid of SMs x ctas_per_sm CTAs looping over tiles.
+  // Not chosen by the caller: float engines take a persistent grid of the
+  // resident CTAs when that saves more launches of CTAs than its last, uneven
+  // round costs.  Several chains: from one full round on (256 x 8^4: 74.7 us
+  // per tick, one CTA per tile 84.2; 40 x 12^4 62.6 and 70.2), as every CTA
+  // loads its chain's descriptor.  One chain: from five rounds on (32^4, 6.7
+  // rounds: 64.0 and 66.9 us; 24^4, 2.1 rounds: 24.0 and 23.2).
   su3_status grid_size(int *grid) {
-    if (ctas_per_sm <= 0) {
-      *grid = std::max(1, total_tiles);
+    *grid = std::max(1, total_tiles);
+    if (ctas_per_sm == 0) return SU3_OK;
+    if (ctas_per_sm == kAutoCtas) {
+      if (storage == SU3_FP64_18 || total_tiles <= (fixed ? 5 : 1) * resident) return SU3_OK;
+      if (resident > 0) *grid = resident;
       return SU3_OK;
     }
     int nsm = 0;
     TRY(device_sm_count(&nsm));
     *grid = std::max(1, std::min(total_tiles, nsm * ctas_per_sm));
+    return SU3_OK;
+  }
+
+  // The CTAs of the update kernel that fit the GPU (rebuild).
+  su3_status count_resident() {
+    int nsm = 0, occ = 0;
+    TRY(device_sm_count(&nsm));
+    const cudaError_t e = fixed ? update_occupancy(storage, kernel_variant(), weighted_any, sub_any, torus_all, block, &occ)
+                                : tick_occupancy(storage, kernel_variant(), weighted_any, torus_all, block, &occ);
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      occ = 0;
+    }
+    resident = nsm * occ;
     return SU3_OK;
   }
 
@@ -1765,7 +1791,7 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
   CU(cudaEventCreate(&a));
   CU(cudaEventCreate(&b));
   double best = 1e30;
-  int best_v = saved_var, best_t = saved_block, best_c = saved_ctas;
+  int best_v = saved_var, best_t = saved_block, best_c = std::max(saved_ctas, 0);
   const int cand_t[] = {64, 128, 256};
   su3_status st = SU3_OK;
   const int nvar = e.sub_any ? 1 : tick_variants(e.storage);  // a divided chain has one kernel form
