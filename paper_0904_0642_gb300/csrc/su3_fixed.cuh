@@ -164,6 +164,11 @@ SU3_HD int clz32(uint32_t x) {
 #endif
 }
 
+SU3_HD int clz64(uint64_t x) {
+  const uint32_t h = (uint32_t)(x >> 32);
+  return h ? clz32(h) : 32 + clz32((uint32_t)x);
+}
+
 // floor(x 2^60) by integer operations, for |x| < 2 (a range check rejects
 // others): the mantissa with its leading bit at bit 63, shifted right by
 // 1026 - e (zero and subnormals shift out), negative values as the ones'
@@ -195,6 +200,24 @@ SU3_HD Fx fx_of(float x) {
 }
 // v 2^-60 as a float, rounded to nearest even.
 SU3_HD float flt_of(int64_t v) { return (float)v * 0x1p-60f; }
+// The same (halves away from zero; zero is not handled), and whether every
+// value within 2^12 units (3.6e-15) rounds to it.
+SU3_HD float flt_of_sure(int64_t v, bool &sure) {
+  const uint64_t m = v < 0 ? 0 - (uint64_t)v : (uint64_t)v;
+  const int lz = clz64(m);
+  const uint64_t n = m << (lz & 63);               // leading bit at 63
+  const uint32_t H = (uint32_t)(n >> 32), R = (uint32_t)(n >> 8);  // R: the dropped bits, 2^32 per ulp
+  const uint32_t thr = 16u << (lz & 31);
+  sure = sure && lz < 27 && R - 0x80000000u + thr > 2u * thr;
+  const uint32_t b = (v < 0 ? 0x80000000u : 0u) + ((uint32_t)(127 + 2 - lz) << 23) + (H >> 8) + (R >> 31);
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float f;
+  std::memcpy(&f, &b, 4);
+  return f;
+#endif
+}
 
 // v 2^-e as a double, rounded to nearest (halves away from zero).
 SU3_HD double dbl_of(int64_t v, int e) {
@@ -572,11 +595,6 @@ SU3_HD int64_t rsqrt_fx(const Fx &n) {
   const int32_t es = (int32_t)(e >> 12);  // 2^-48
   const int64_t g = (e >> 1) + ((3 * (((int64_t)es * es) >> 36)) >> 3);
   return ((int64_t)Y << 34) + mulY(fx_split(g));
-}
-
-SU3_HD int clz64(uint64_t x) {
-  const uint32_t h = (uint32_t)(x >> 32);
-  return h ? clz32(h) : 32 + clz32((uint32_t)x);
 }
 
 // sqrt(p), p > 0 in units 2^-64: the result times 2^e, in [1/2, 1) and in

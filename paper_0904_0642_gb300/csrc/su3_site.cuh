@@ -1022,8 +1022,36 @@ __device__ __forceinline__ void reunit_rows2_f(M3<float> &m) {
   reunit_apply_f(m, d2f_bits(s1 - 1.0), d2f_bits(pdr), d2f_bits(pdi), d2f_bits(s2 - 1.0));
 }
 
+// reunit_apply_f, and whether its floats are sure to be those of the
+// double-precision factors too: those differ from the factors given here
+// (exact to 2^-57) by up to 1e-15, so each result must not change when its
+// correction moves by that and by two ulps.
+__device__ __forceinline__ bool reunit_apply_sure(M3<float> &m, float e1, float pr, float pi, float e2) {
+  constexpr float kAbs = 4e-15f, kRel = 0x1p-22f;
+  C<float> *r1 = m.e[0], *r2 = m.e[1];
+  const float eta1 = fm(fabsf(e1), kRel, kAbs), lo = e1 - eta1, hi = e1 + eta1;
+  bool sure = true;
+  const auto first = [&](float a) {
+    sure = sure && fm(a, lo, a) == fm(a, hi, a);
+    return fm(a, e1, a);
+  };
+  const auto second = [&](float b, float c) {
+    const float corr = fm(b, e2, fm(c, e2, c)), eta = fm(fabsf(corr), kRel, kAbs);
+    sure = sure && b + (corr - eta) == b + (corr + eta);
+    return b + corr;
+  };
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r1[k] = {first(r1[k].re), first(r1[k].im)};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const C<float> a = r1[k];
+    r2[k] = {second(r2[k].re, fm(pi, a.im, -pr * a.re)), second(r2[k].im, fm(-pi, a.re, -pr * a.im))};
+  }
+  return sure;
+}
+
 // One stored link in double precision, out of line: links whose rows are far
-// from orthonormal (reunit_link) only.
+// from orthonormal, or whose float rounding is not sure (reunit_link).
 template <class S>
 static __device__ __noinline__ void reunit_link_general(typename S::Vec *p, int Vh, int js) {
   if constexpr (S::kTwoRows) {
@@ -1041,7 +1069,10 @@ static __device__ __noinline__ void reunit_link_general(typename S::Vec *p, int 
 // Re-unitarise one stored link: the sums, products and reciprocal square roots
 // in fixed point (errors below 2^-57, absolute; the double-precision pipe ran
 // at 90 % of its rate here), the result rounded to the storage precision, or
-// applied to two-row float storage as in reunit_rows2_f.
+// applied to two-row float storage as in reunit_rows2_f.  Float links that
+// might round differently from the double-precision form (one warp in
+// several hundred holds such a link; links with zeros always) take that form:
+// the stored floats are its floats.
 template <class S>
 __device__ __forceinline__ void reunit_link(typename S::Vec *p, int Vh, int js) {
   using R = typename S::R;
@@ -1065,23 +1096,28 @@ __device__ __forceinline__ void reunit_link(typename S::Vec *p, int Vh, int js) 
   if constexpr (S::kTwoRows) {
     float e1, pr, pi, e2;
     if (in && reunit_factors_f(f.e[0], f.e[1], e1, pr, pi, e2)) {
-      reunit_apply_f(m, e1, pr, pi, e2);
-      S::store(p, Vh, js, m);
-      return;
+      if (reunit_apply_sure(m, e1, pr, pi, e2)) {
+        S::store(p, Vh, js, m);
+        return;
+      }
     }
   } else if (in && reunit_f<sizeof(R) == 4>(f, rr) && rr.ok()) {
+    bool sure = true;
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         const int64_t re = fx_val(f.e[i][k].re), im = fx_val(f.e[i][k].im);
-        if constexpr (sizeof(R) == 4)
-          m.e[i][k] = {flt_of(re), flt_of(im)};
-        else
+        if constexpr (sizeof(R) == 4) {
+          m.e[i][k].re = flt_of_sure(re, sure);
+          m.e[i][k].im = flt_of_sure(im, sure);
+        } else
           m.e[i][k] = {dbl_of_pipe(re, 60), dbl_of_pipe(im, 60)};
       }
-    S::store(p, Vh, js, m);
-    return;
+    if (sure) {
+      S::store(p, Vh, js, m);
+      return;
+    }
   }
   reunit_link_general<S>(p, Vh, js);
 }
