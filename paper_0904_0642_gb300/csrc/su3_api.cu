@@ -461,7 +461,23 @@ struct Engine {
   bool cluster = false;       // fixed, fewest links: whole sweeps per launch (k_sweeps)
   bool coop = false;          // too few links to fill the GPU: eight lanes per link
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
-  int kernel_variant() const { return !coop ? variant : (storage == SU3_FP64_18 ? 1 : kFloatLanes); }
+  int kernel_variant() const {
+    if (coop) return storage == SU3_FP64_18 ? 1 : kFloatLanes;
+    return ctas_per_sm == kAutoCtas ? auto_variant : variant;
+  }
+  // The register variant of a two-row float chain until set_launch, from the
+  // warps of its update phase (rebuild).  One warp per scheduler or fewer: the
+  // rolled variant 3, whose short code is fetched sooner (DLT 2 x 16^3 x 4 6.0
+  // us per phase, variant 0 6.7; 12^4 5.9 and 6.4; from 1.7 warps on variant 0
+  // is faster, 16^4 7.0 and 7.2).  Otherwise variant 1 (20 warps per SM, each
+  // round about 1.2 times as long as with 16) where it saves enough rounds
+  // (20^4 12.4 and 14.1 us, 24^4 22.0 and 23.1).
+  int auto_variant = 0;
+  static int variant_for(long long warps, int nsm) {
+    const auto rounds = [&](long long per_sm) { return (warps + per_sm * nsm - 1) / (per_sm * nsm); };
+    if (warps <= 4ll * nsm) return 3;
+    return 6 * rounds(20) < 5 * rounds(16) ? 1 : 0;
+  }
   // The links of one update phase of an FP64 chain that may take eight lanes
   // per link (others: more than any limit).
   long long coop_sites(const Chain &ch) const {
@@ -844,7 +860,12 @@ struct Engine {
       torus_all = tor;
       drop_graph();
     }
-    if (ctas_per_sm == kAutoCtas) TRY(count_resident());
+    if (ctas_per_sm == kAutoCtas) {
+      int nsm = 0;
+      TRY(device_sm_count(&nsm));
+      auto_variant = fixed && !coop && !sb && storage == SU3_FP32_12 ? variant_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
+      TRY(count_resident());
+    }
     if (chains.size() > chain_cap) {
       cudaFree(d_desc);
       cudaFree(d_state);
