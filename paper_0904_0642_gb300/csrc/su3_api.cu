@@ -1133,6 +1133,7 @@ struct Engine {
         u.mu = st % d.D;
         u.offset = (uint32_t)i;
         u.first = i == 0 && st == 0;
+        u.early = i > 0 || st >= 2;
         u.advance = i == c.m - 1 && st == 2 * d.D - 1 ? (uint32_t)c.m : 0u;
         u.tiles = total_tiles;
         TRY(each(0, [&] {
@@ -2092,13 +2093,6 @@ extern "C" su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, 
     hbm_budget_bytes = (size_t)(0.8 * (double)fr);
   }
   srv->budget = hbm_budget_bytes;
-  if (srv->eng.make_pool(hbm_budget_bytes) != SU3_OK) {
-    const std::string msg = g_err;
-    srv->eng.release();
-    cudaStreamDestroy(st);
-    delete srv;
-    return fail(SU3_ECUDA, "%s", msg.c_str());
-  }
   srv->max_slots = max_slots;
   {
     // persistent grid: its size does not depend on the resident jobs, so the
@@ -2242,6 +2236,10 @@ void su3_server::loop() {
     // Bring admitted jobs on the device (outside the lock).
     bool changed = false;
     std::vector<std::pair<uint64_t, const double *>> starts;  // jobs with a given start configuration
+    if (!admitted.empty() && !eng.pool && eng.make_pool(budget) != SU3_OK) {
+      die(g_err);
+      break;
+    }
     for (auto &j : admitted) {
       Chain ch;
       su3_config c = j.job.cfg;

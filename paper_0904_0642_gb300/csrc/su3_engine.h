@@ -173,6 +173,7 @@ struct UpdateStep {
   uint32_t offset;         // sweeps completed since the schedule's first launch
   uint32_t advance;        // last launch: sweeps to add to the counter (0: not the last)
   int32_t first;           // 1: the schedule's first launch
+  int32_t early;           // 1: its third or a later one: `cur` may be read before the previous launch has ended
   int32_t tiles;
 };
 

@@ -419,20 +419,36 @@ __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, 
 // runs the subgroups.  Same operations in the same order per element: the
 // links are bitwise those of the other forms.  Called by whole warps; lanes
 // without a link (valid false) run along on a repeated one.
-template <class S, bool SUB>
-__device__ __forceinline__ void update_site_lanes(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
-                                                  int jj, bool valid, uint32_t &nprop, uint32_t &nacc, float &dr) {
-  const int Vh = d.Vh, oc = colour ^ 1;
+
+// Lane l's part of the draws (no link is read): lanes 0..2 the first
+// proposals, lanes 3, 4 the direction blocks; then lanes 3..5 the directions.
+__device__ __forceinline__ DrawPre lanes_draws_f(uint2 key, uint32_t c0, uint32_t sweep, int colour, int mu) {
   const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
-  const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
+  const int sub = l8 < 3 ? l8 : (l8 < 6 ? l8 - 3 : 0);
+  const uint32_t btag = heatbath_tag(colour, mu, l8 < 3 ? l8 : (l8 == 4 ? 2 : 0)) | (l8 < 3 ? 0u : kHitDirection);
+  const uint4 w = philox4x32_10(make_uint4(c0, sweep, btag, kPurposeHeatbath), key);
+  const int dl = base + (sub == 2 ? 4 : 3);
+  const uint32_t d0 = __shfl_sync(0xffffffffu, w.x, dl), d1 = __shfl_sync(0xffffffffu, w.y, dl);
+  const uint32_t d2 = __shfl_sync(0xffffffffu, w.z, dl), d3 = __shfl_sync(0xffffffffu, w.w, dl);
+  DrawPre mine;
+  proposal_pre_words(mine, w);
+  direction_pre_f(mine, sub == 1 ? d2 : d0, sub == 1 ? d3 : d1);
+  return mine;
+}
+
+template <class S, bool SUB>
+__device__ __forceinline__ void update_site_lanes(const ChainDesc &d, uint32_t sweep, int colour, int mu,
+                                                  const SiteGeo &g, uint32_t c0, bool valid, const DrawPre &mine,
+                                                  uint32_t &nprop, uint32_t &nacc, float &dr) {
+  const int Vh = d.Vh, oc = colour ^ 1, layer = g.layer;
+  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
   const int js = g.s >> 1;
   int offp, flp;
   step_fwd(d, sel(g.x, mu), mu, offp, flp);
   const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
-  const uint32_t c0 = site_key<SUB>(d, g);
   const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
 
-  // this lane's links: issued before the draws
+  // this lane's links
   const int ns = 2 * (d.D - 1), t = l8 < ns ? l8 : 0;
   const bool up = (t & 1) == 0;
   int nu = t >> 1;
@@ -450,18 +466,6 @@ __device__ __forceinline__ void update_site_lanes(const ChainDesc &d, uint32_t s
   const M3<float> X = S::load2(up ? plane_ptr<S>(d, layer, colour, nu) : plane_ptr<S>(d, lm, oc, mu), Vh, (up ? g.s : sm) >> 1);
   const M3<float> G = S::load(up ? plane_ptr<S>(d, lp, oc, nu) : plane_ptr<S>(d, lm, oc, nu), Vh, (up ? sp : sm) >> 1);
   M3<float> U = S::load(plane_ptr<S>(d, layer, colour, mu), Vh, js);
-
-  // draws: lanes 0..2 the first proposals, lanes 3, 4 the direction blocks;
-  // then lanes 3..5 the directions
-  const int sub = l8 < 3 ? l8 : (l8 < 6 ? l8 - 3 : 0);
-  const uint32_t btag = heatbath_tag(colour, mu, l8 < 3 ? l8 : (l8 == 4 ? 2 : 0)) | (l8 < 3 ? 0u : kHitDirection);
-  const uint4 w = philox4x32_10(make_uint4(c0, sweep, btag, kPurposeHeatbath), key);
-  const int dl = base + (sub == 2 ? 4 : 3);
-  const uint32_t d0 = __shfl_sync(0xffffffffu, w.x, dl), d1 = __shfl_sync(0xffffffffu, w.y, dl);
-  const uint32_t d2 = __shfl_sync(0xffffffffu, w.z, dl), d3 = __shfl_sync(0xffffffffu, w.w, dl);
-  DrawPre mine;
-  proposal_pre_words(mine, w);
-  direction_pre_f(mine, sub == 1 ? d2 : d0, sub == 1 ? d3 : d1);
 
   // this lane's staple
   M3<float> M = mul_nn_2(X, Y);
@@ -775,27 +779,17 @@ __device__ __forceinline__ int64_t shfl_xor_ll(int64_t a, int m) {
 // column of U each in the projections and rotations.  Results are bitwise
 // those of update_site_fixed.  Called by whole warps; lanes without a link
 // (valid false) run along on a repeated one.
-template <bool SUB, bool COH = false>
-__device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
-                                                 int jj, bool valid, uint32_t &nprop, uint32_t &nacc,
-                                                 ActionChange &dr) {
-  using S = StoreF64x18;
-  const int Vh = d.Vh;
-  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
-  const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
-  const int js = g.s >> 1;
-  int offp, flp;
-  step_fwd(d, sel(g.x, mu), mu, offp, flp);
-  const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
-  const uint32_t c0 = site_key<SUB>(d, g);
-  const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
-  const InvBeta ib = {d.inv_beta_m, d.inv_beta_e};
-  const int hits = d.hits;
 
-  // The first proposals and directions: a block of random words per lane
-  // (lanes 0..2: the proposals, 3 and 4: the direction blocks of subgroups 0,
-  // 1 and of subgroup 2), then lanes 0..2 take ln u1 and the proposal's angle,
-  // lanes 3..5 ln u3 and the direction.
+// Lane l's part of the draws (no link is read).  A block of random words per
+// lane (lanes 0..2: the first proposals, 3 and 4: the direction blocks of
+// subgroups 0, 1 and of subgroup 2), then lanes 0..2 take ln u1 and the
+// proposal's angle, lanes 3..5 ln u3 and the direction.
+struct CoopDraws {
+  int64_t L, u4sq;        // lanes 0..2
+  Fx st, ct, cphi, sphi;  // lanes 3..5
+};
+__device__ __forceinline__ CoopDraws coop_draws(uint2 key, uint32_t c0, uint32_t sweep, int colour, int mu) {
+  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
   const int sub = l8 < 3 ? l8 : (l8 < 6 ? l8 - 3 : 0);
   const uint32_t btag = heatbath_tag(colour, mu, l8 < 3 ? l8 : (l8 == 4 ? 2 : 0)) | (l8 < 3 ? 0u : kHitDirection);
   const uint4 w = philox4x32_10(make_uint4(c0, sweep, btag, kPurposeHeatbath), key);
@@ -808,8 +802,31 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
   int64_t cs, sn;
   trig_fx(prop ? 2u * w.y + 1u : wphi, prop ? 0 : 1, cs, sn);
   const int64_t nl = neg_log_fx(prop ? w.x : w3rd);
-  const int64_t L1 = radius_fx(nl, shfl_ll(nl, base + (l8 + 3 & 7)), cs), u41 = square_fx(w.w);
-  const Fx st1 = sin_theta_fx(wth), ct1 = cos_theta_fx(wth), cp1 = fx_split(cs), sp1 = fx_split(sn);
+  CoopDraws r;
+  r.L = radius_fx(nl, shfl_ll(nl, base + ((l8 + 3) & 7)), cs);
+  r.u4sq = square_fx(w.w);
+  r.st = sin_theta_fx(wth);
+  r.ct = cos_theta_fx(wth);
+  r.cphi = fx_split(cs);
+  r.sphi = fx_split(sn);
+  return r;
+}
+
+template <bool SUB, bool COH = false>
+__device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sweep, int colour, int mu,
+                                                 const SiteGeo &g, int jj, uint32_t c0, bool valid,
+                                                 const CoopDraws &mine, uint32_t &nprop, uint32_t &nacc,
+                                                 ActionChange &dr) {
+  using S = StoreF64x18;
+  const int Vh = d.Vh, layer = g.layer;
+  const int lane = threadIdx.x & 31, l8 = lane & 7, base = lane & 24;
+  const int js = g.s >> 1;
+  int offp, flp;
+  step_fwd(d, sel(g.x, mu), mu, offp, flp);
+  const int sp = g.s + offp, lp = lflip<SUB>(d, layer, flp);  // x + mu
+  const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
+  const InvBeta ib = {d.inv_beta_m, d.inv_beta_e};
+  const int hits = d.hits;
 
   // staples
   FSum A = {};
@@ -864,12 +881,12 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
       }
       pa[q] = fold60(s[q]);
     }
-    const int64_t L = shfl_ll(L1, base + sg), u4 = shfl_ll(u41, base + sg);
+    const int64_t L = shfl_ll(mine.L, base + sg), u4 = shfl_ll(mine.u4sq, base + sg);
     Direction dir;
-    dir.st = shfl_fx(st1, base + 3 + sg);
-    dir.ct = shfl_fx(ct1, base + 3 + sg);
-    dir.cphi = shfl_fx(cp1, base + 3 + sg);
-    dir.sphi = shfl_fx(sp1, base + 3 + sg);
+    dir.st = shfl_fx(mine.st, base + 3 + sg);
+    dir.ct = shfl_fx(mine.ct, base + 3 + sg);
+    dir.cphi = shfl_fx(mine.cphi, base + 3 + sg);
+    dir.sphi = shfl_fx(mine.sphi, base + 3 + sg);
     FxNorm n;
     if (norm_fx(pa, n)) {
       const uint32_t tag = heatbath_tag(colour, mu, sg);
@@ -1541,7 +1558,7 @@ template <> struct TickBounds<4> { static constexpr int kThreads = 256, kMinBloc
 template <> struct TickBounds<10> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64
 template <> struct TickBounds<kCoopVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64, eight lanes per link
 
-template <> struct TickBounds<kLanesVariant> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };  // FP32, eight lanes per link
+template <> struct TickBounds<kLanesVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP32, eight lanes per link
 
 // ------------------------------------------------------------------ one tile of an update phase
 
@@ -1564,40 +1581,80 @@ __device__ __forceinline__ double warp_sum(ActionChange dr) {
   return sum;
 }
 
-// The links j0.. of one warp with eight lanes per link (slot: the warp's).
-template <class S, bool SUB, bool COH>
-__device__ __forceinline__ void update_warp(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer, int j0,
-                                            int slot, uint32_t &np, uint32_t &na) {
-  if (j0 >= d.Vn) return;
-  const int jj = j0 + (int)(threadIdx.x & 31) / kCoopLanes, jc = min(jj, d.Vn - 1);
-  if constexpr (sizeof(typename S::R) == 8) {
-    ActionChange dr = {0, 0.0};
-    update_site_coop<SUB, COH>(d, sweep, colour, mu, layer, jc, jj < d.Vn, np, na, dr);
-    __syncwarp();
-    book_action(d, slot, warp_sum(dr));
-  } else {
-    float dr = 0.0f;
-    update_site_lanes<S, SUB>(d, sweep, colour, mu, layer, jc, jj < d.Vn, np, na, dr);
-    __syncwarp();
-#pragma unroll
-    for (int o = 16; o >= kCoopLanes; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
-    book_action(d, slot, (double)dr);
+// The links j0.. of one warp with eight lanes per link, in two parts: what
+// needs no link (the site, the draws), and the update.
+template <class S, bool SUB>
+struct WarpLinks {
+  using Draws = std::conditional_t<sizeof(typename S::R) == 8, CoopDraws, DrawPre>;
+  SiteGeo g;
+  int jj;
+  bool valid;
+  uint32_t c0;
+  Draws draws;
+
+  __device__ __forceinline__ void prepare(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer, int j0) {
+    const int j = j0 + (int)(threadIdx.x & 31) / kCoopLanes;
+    valid = j < d.Vn;
+    jj = min(j, d.Vn - 1);
+    g = site_of<SUB>(d, layer, colour, jj);
+    c0 = site_key<SUB>(d, g);
+    const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
+    if constexpr (sizeof(typename S::R) == 8)
+      draws = coop_draws(key, c0, sweep, colour, mu);
+    else
+      draws = lanes_draws_f(key, c0, sweep, colour, mu);
   }
+
+  // slot: the warp's action slot
+  template <bool COH>
+  __device__ __forceinline__ void update(const ChainDesc &d, uint32_t sweep, int colour, int mu, int slot,
+                                         uint32_t &np, uint32_t &na) {
+    if constexpr (sizeof(typename S::R) == 8) {
+      ActionChange dr = {0, 0.0};
+      update_site_coop<SUB, COH>(d, sweep, colour, mu, g, jj, c0, valid, draws, np, na, dr);
+      __syncwarp();
+      book_action(d, slot, warp_sum(dr));
+    } else {
+      float dr = 0.0f;
+      update_site_lanes<S, SUB>(d, sweep, colour, mu, g, c0, valid, draws, np, na, dr);
+      __syncwarp();
+#pragma unroll
+      for (int o = 16; o >= kCoopLanes; o >>= 1) dr += __shfl_down_sync(0xffffffffu, dr, o);
+      book_action(d, slot, (double)dr);
+    }
+  }
+};
+
+// The lanes of a link and the first link of this warp in tile lt (slot: the
+// warp's action slot).
+template <int V>
+constexpr int kLanesOf = V == kCoopVariant || V == kLanesVariant ? kCoopLanes : 1;
+struct WarpPlace {
+  int layer, jw, slot;
+};
+template <int LANES>
+__device__ __forceinline__ WarpPlace warp_place(const ChainDesc &d, int lt) {
+  constexpr int kPerWarp = 32 / LANES;
+  WarpPlace p;
+  p.layer = fast_div(lt, d.tdiv);  // a layer, or a sublattice box of one
+  p.jw = (lt - p.layer * d.tiles_per_vl) * ((int)blockDim.x / LANES) + (int)(threadIdx.x & ~31u) / LANES;
+  p.slot = p.layer * ((d.Vn + kPerWarp - 1) / kPerWarp) + p.jw / kPerWarp;
+  return p;
 }
 
 // The updates of one CTA's tile lt of a chain's phase (colour, mu).
 template <class S, int V, bool WT, bool SUB, bool TOR>
 __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, int colour, int mu, int lt,
                                             uint32_t &np, uint32_t &na) {
-  constexpr int kLanes = V == kCoopVariant || V == kLanesVariant ? kCoopLanes : 1, kPerWarp = 32 / kLanes;
-  const int layer = fast_div(lt, d.tdiv);  // a layer, or a sublattice box of one
-  const int j0 = (lt - layer * d.tiles_per_vl) * ((int)blockDim.x / kLanes);
-  const int jw = j0 + (int)(threadIdx.x & ~31u) / kLanes;  // the first link of the warp
-  const int slot = layer * ((d.Vn + kPerWarp - 1) / kPerWarp) + jw / kPerWarp;
-  if constexpr (kLanes > 1) {
-    update_warp<S, SUB, false>(d, sweep, colour, mu, layer, jw, slot, np, na);
+  const WarpPlace p = warp_place<kLanesOf<V>>(d, lt);
+  const int layer = p.layer;
+  if constexpr (kLanesOf<V> > 1) {
+    if (p.jw >= d.Vn) return;
+    WarpLinks<S, SUB> w;
+    w.prepare(d, sweep, colour, mu, layer, p.jw);
+    w.template update<false>(d, sweep, colour, mu, p.slot, np, na);
   } else {
-    const int jj = j0 + (int)threadIdx.x;
+    const int jj = p.jw + (int)(threadIdx.x & 31);
     const bool valid = jj < d.Vn;
     double sum;
     // the one-coupling FP64 update runs in fixed point
@@ -1621,7 +1678,7 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
       sum = (double)dr;
     }
     // (a warp of the ragged last tile with no link has no slot)
-    if (jw < d.Vn) book_action(d, slot, sum);
+    if (p.jw < d.Vn) book_action(d, p.slot, sum);
   }
 }
 

@@ -16,18 +16,46 @@ __device__ __forceinline__ void wait_previous() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// The sweep counter of a schedule's launch (its first one copies it).
+__device__ __forceinline__ uint32_t next_base(ChainCtl *ctl, const UpdateStep &u) {
+  const uint32_t base = __ldcg(u.first ? &ctl->nxt : &ctl->cur);
+  if (u.first && blockIdx.x == 0 && threadIdx.x == 0) ctl->cur = base;
+  return base;
+}
+
 template <class S, int V, bool WT, bool SUB, bool TOR>
 __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBlocks)
     k_update(const __grid_constant__ ChainDesc d, ChainCtl *ctl, const UpdateStep u) {
-  wait_previous();
-  const uint32_t base = __ldcg(u.first ? &ctl->nxt : &ctl->cur);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    if (u.first) ctl->cur = base;
-    if (u.advance) ctl->nxt = base + u.advance;
-  }
   uint32_t np = 0, na = 0;
-  for (int lt = blockIdx.x; lt < u.tiles; lt += gridDim.x)
-    update_tile<S, V, WT, SUB, TOR>(d, base + u.offset, u.colour, u.mu, lt, np, na);
+  if constexpr (kLanesOf<V> > 1) {
+    // The site and the draws need no link: they run before the wait, while the
+    // previous phase ends - except in a schedule's first two launches, whose
+    // predecessors may still be writing the sweep counter.
+    uint32_t base = 0;
+    const bool early = u.early != 0;
+    if (early) base = __ldcg(&ctl->cur);
+    WarpLinks<S, SUB> w;
+    int lt = blockIdx.x;
+    WarpPlace p = warp_place<kCoopLanes>(d, lt);
+    if (early && p.jw < d.Vn) w.prepare(d, base + u.offset, u.colour, u.mu, p.layer, p.jw);
+    wait_previous();
+    if (!early) base = next_base(ctl, u);
+    if (u.advance && blockIdx.x == 0 && threadIdx.x == 0) ctl->nxt = base + u.advance;
+    if (!early && p.jw < d.Vn) w.prepare(d, base + u.offset, u.colour, u.mu, p.layer, p.jw);
+    while (true) {
+      if (p.jw < d.Vn) w.template update<false>(d, base + u.offset, u.colour, u.mu, p.slot, np, na);
+      lt += gridDim.x;
+      if (lt >= u.tiles) break;
+      p = warp_place<kCoopLanes>(d, lt);
+      if (p.jw < d.Vn) w.prepare(d, base + u.offset, u.colour, u.mu, p.layer, p.jw);
+    }
+  } else {
+    wait_previous();
+    const uint32_t base = next_base(ctl, u);
+    if (u.advance && blockIdx.x == 0 && threadIdx.x == 0) ctl->nxt = base + u.advance;
+    for (int lt = blockIdx.x; lt < u.tiles; lt += gridDim.x)
+      update_tile<S, V, WT, SUB, TOR>(d, base + u.offset, u.colour, u.mu, lt, np, na);
+  }
   flush_counters(d, np, na);
 }
 
@@ -57,7 +85,9 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
 #pragma unroll 1
     for (int w = w0; w < warps; w += nw) {
       const int vl = w / per_vl, j0 = (w - vl * per_vl) * kPerWarp;
-      update_warp<S, SUB, true>(d, base + (uint32_t)s, colour, mu, vl, j0, w, np, na);
+      WarpLinks<S, SUB> links;
+      links.prepare(d, base + (uint32_t)s, colour, mu, vl, j0);
+      links.template update<true>(d, base + (uint32_t)s, colour, mu, w, np, na);
     }
     cluster_barrier();
   }
