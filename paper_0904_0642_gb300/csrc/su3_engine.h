@@ -50,12 +50,15 @@ constexpr int kCoopSites = 8192;
 // eight lanes per link too (update_site_lanes; the launchers' variant
 // kFloatLanes).  Per phase, one thread per link and eight lanes: 8^3 x 4 5.8
 // and 4.3 us, 8^4 5.9 and 4.4, 16^2 x 8 x 4 (4096 links) 6.0 and 5.4, 16^3 x 4
-// (8192) 6.4 and 7.4.  (Four lanes of two staples each: 4.8, 4.8, 5.1, 5.8.)
+// (8192) 6.4 and 7.4; with the draws before the wait (k_update) 8^3 x 4 takes
+// 3.7 and 8^4 3.84.  (Four lanes of two staples each: 4.8, 4.8, 5.1, 5.8.)
 constexpr int kLanesLinks = 4096, kFloatLanes = 16;
 // Chains of one coupling with at most kClusterLinks links per phase run whole
-// sweeps in one launch of a cluster of CTAs (k_sweeps), eight lanes per link:
-// float 4^4 3.3 us per phase (4.2 with a launch per phase), FP64 12.2 (12.5).
-// More links share the cluster's 16 SMs too long: 8^3 x 4 6.3 us against 4.3.
+// sweeps in one launch of a cluster of CTAs (k_sweeps), eight lanes per link.
+// Per phase, against a launch per phase: float 4^4 3.25 us (3.62), 8^3 3.22
+// (3.77), 16^2 3.78 (4.57); FP64 4^4 11.4 (11.6), 8^3 11.6 (12.1).  More links
+// share the cluster's 16 SMs too long: float 8^3 x 4 6.3 us against 4.3, both
+// with the draws after the wait.
 constexpr int kClusterCtas = 16, kClusterThreads = 128;
 constexpr int kClusterLinks = kClusterCtas * kClusterThreads / kCoopLanes;
 

@@ -63,9 +63,12 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
 // (eight lanes per link): the phases are separated by the cluster's hardware
 // barrier instead of a kernel boundary, and the code stays in the instruction
 // caches.  Links are read through L2 (COH): other CTAs have written them.
-__device__ __forceinline__ void cluster_barrier() {
+__device__ __forceinline__ void cluster_arrive() {
   __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
@@ -82,15 +85,21 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
   for (int i = 0; i < sweeps * 2 * d.D; ++i) {
     const int s = i / (2 * d.D), st = i - s * 2 * d.D;
     const int colour = st >= d.D ? 1 : 0, mu = st - colour * d.D;
+    int w = w0;
 #pragma unroll 1
-    for (int w = w0; w < warps; w += nw) {
+    do {
       const int vl = w / per_vl, j0 = (w - vl * per_vl) * kPerWarp;
       WarpLinks<S, SUB> links;
-      links.prepare(d, base + (uint32_t)s, colour, mu, vl, j0);
-      links.template update<true>(d, base + (uint32_t)s, colour, mu, w, np, na);
-    }
-    cluster_barrier();
+      // the site and the draws need no link: the first of a phase before the
+      // wait for the previous phase's links
+      if (w < warps) links.prepare(d, base + (uint32_t)s, colour, mu, vl, j0);
+      if (i > 0 && w == w0) cluster_wait();
+      if (w < warps) links.template update<true>(d, base + (uint32_t)s, colour, mu, w, np, na);
+      w += nw;
+    } while (w < warps);
+    cluster_arrive();
   }
+  cluster_wait();
   flush_counters(d, np, na);
   if (blockIdx.x == 0 && threadIdx.x == 0) ctl->nxt = base + (uint32_t)sweeps;
 }
