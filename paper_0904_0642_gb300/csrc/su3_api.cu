@@ -460,23 +460,32 @@ struct Engine {
   int resident = 0;           // CTAs of the update kernel that fit the GPU (0: not known)
   bool cluster = false;       // fixed, fewest links: whole sweeps per launch (k_sweeps)
   bool coop = false;          // too few links to fill the GPU: eight lanes per link
+  int early = 0;              // the form of an update begun before the previous launch has ended (0: none)
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
   int kernel_variant() const {
     if (coop) return storage == SU3_FP64_18 ? 1 : kFloatLanes;
+    if (early) return early;
     return ctas_per_sm == kAutoCtas ? auto_variant : variant;
   }
-  // The register variant of a two-row float chain until set_launch, from the
-  // warps of its update phase (rebuild).  One warp per scheduler or fewer: the
-  // rolled variant 3, whose short code is fetched sooner (DLT 2 x 16^3 x 4 6.0
-  // us per phase, variant 0 6.7; 12^4 5.9 and 6.4; from 1.7 warps on variant 0
-  // is faster, 16^4 7.0 and 7.2).  Otherwise variant 1 (20 warps per SM, each
-  // round about 1.2 times as long as with 16) where it saves enough rounds
-  // (20^4 12.4 and 14.1 us, 24^4 22.0 and 23.1).
+  // The register variant of a two-row float chain without another form, until
+  // set_launch, from the warps of its update phase (rebuild): variant 1 (20
+  // warps per SM, each round about 1.2 times as long as with 16) where it
+  // saves enough rounds (20^4 12.4 and 14.1 us, 24^4 22.0 and 23.1).
   int auto_variant = 0;
   static int variant_for(long long warps, int nsm) {
     const auto rounds = [&](long long per_sm) { return (warps + per_sm * nsm - 1) / (per_sm * nsm); };
-    if (warps <= 4ll * nsm) return 3;
     return 6 * rounds(20) < 5 * rounds(16) ? 1 : 0;
+  }
+  // The form of a one-coupling float chain's update that begins before the
+  // previous launch has ended, while its warps fit beside that one's (8 per SM
+  // at its registers).  Per phase, without and with it: DLT 2 x 16^3 x 4 6.2
+  // and 4.65 us, 12^4 6.1 and 4.5 (in four boxes 8.2 and 6.3), 16^4 7.2 and
+  // 6.3, 18^3 x 12 7.3 and 6.6 (18 reals 7.9 and 7.0); beyond the line 18^3 x
+  // 14 10.1 and 11.1, 24^4 23.6 and 28.  Rolled at one warp per scheduler: its
+  // short code is fetched sooner (12^4 4.5 us, unrolled 4.8; 16^4 6.6 and 6.3).
+  static int early_for(long long warps, int nsm) {
+    if (warps > 8ll * nsm) return 0;
+    return warps <= 4ll * nsm ? kFloatEarlyRolled : kFloatEarly;
   }
   // The links of one update phase of an FP64 chain that may take eight lanes
   // per link (others: more than any limit).
@@ -860,10 +869,13 @@ struct Engine {
       torus_all = tor;
       drop_graph();
     }
+    int nsm = 0;
+    TRY(device_sm_count(&nsm));
+    const int ef = fixed && !coop && !w && storage != SU3_FP64_18 ? early_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
+    if (ef != early) drop_graph();
+    early = ef;
     if (ctas_per_sm == kAutoCtas) {
-      int nsm = 0;
-      TRY(device_sm_count(&nsm));
-      auto_variant = fixed && !coop && !sb && storage == SU3_FP32_12 ? variant_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
+      auto_variant = fixed && !sb && storage == SU3_FP32_12 ? variant_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
       TRY(count_resident());
     }
     if (chains.size() > chain_cap) {
@@ -1821,7 +1833,7 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
     for (int t : cand_t) {
       if (t > tick_max_threads(e.storage, v)) continue;
       int occ = 0;
-      const int kv = e.coop ? e.kernel_variant() : v;
+      const int kv = e.coop || e.early ? e.kernel_variant() : v;
       const cudaError_t oe = e.fixed ? update_occupancy(e.storage, kv, e.weighted_any, e.sub_any, e.torus_all, t, &occ)
                                      : tick_occupancy(e.storage, kv, e.weighted_any, e.torus_all, t, &occ);
       if (oe != cudaSuccess || occ < 1) continue;

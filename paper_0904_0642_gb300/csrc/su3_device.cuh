@@ -918,11 +918,9 @@ __device__ __forceinline__ void cm_subgroup_f(M3<float> &U, const M3<float> &A, 
   rotate_rows(U, i, j, r0, r1, r2, r3);
 }
 
-// cm_update for float links with the draws' counter-only parts first.
-__device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, float beta, int hits, uint2 key,
-                                            uint32_t c0, uint32_t c1, int colour, int mu, uint32_t &nprop,
-                                            uint32_t &nacc, float &dretr) {
-  DrawPre pre[3];
+// cm_update for float links in two parts: what the three draws need of no link
+// (pre), and the update.
+__device__ __forceinline__ void cm_draws_f(DrawPre (&pre)[3], uint2 key, uint32_t c0, uint32_t c1, int colour, int mu) {
 #pragma unroll
   for (int sg = 0; sg < 3; ++sg) proposal_pre_f(pre[sg], key, c0, c1, heatbath_tag(colour, mu, sg));
   // the two direction blocks, split as direction_words splits them
@@ -931,6 +929,10 @@ __device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, fl
   direction_pre_f(pre[0], d01.x, d01.y);
   direction_pre_f(pre[1], d01.z, d01.w);
   direction_pre_f(pre[2], d2.x, d2.y);
+}
+__device__ __forceinline__ void cm_apply_f(M3<float> &U, const M3<float> &A, float beta, int hits, uint2 key,
+                                           uint32_t c0, uint32_t c1, int colour, int mu, const DrawPre (&pre)[3],
+                                           uint32_t &nprop, uint32_t &nacc, float &dretr) {
   dretr = 0.0f;
   const float ca = 2.0f * beta / 3.0f;
 #pragma unroll
@@ -939,6 +941,13 @@ __device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, fl
     const int j = (sg == 0) ? 1 : 2;
     cm_subgroup_f(U, A, i, j, ca, hits, key, c0, c1, heatbath_tag(colour, mu, sg), pre[sg], nprop, nacc, dretr);
   }
+}
+__device__ __forceinline__ void cm_update_f(M3<float> &U, const M3<float> &A, float beta, int hits, uint2 key,
+                                            uint32_t c0, uint32_t c1, int colour, int mu, uint32_t &nprop,
+                                            uint32_t &nacc, float &dretr) {
+  DrawPre pre[3];
+  cm_draws_f(pre, key, c0, c1, colour, mu);
+  cm_apply_f(U, A, beta, hits, key, c0, c1, colour, mu, pre, nprop, nacc, dretr);
 }
 
 }  // namespace su3g

@@ -48,11 +48,15 @@ constexpr int kCoopSites = 8192;
 
 // Float chains of one coupling with at most kLanesLinks links per phase take
 // eight lanes per link too (update_site_lanes; the launchers' variant
-// kFloatLanes).  Per phase, one thread per link and eight lanes: 8^3 x 4 5.8
-// and 4.3 us, 8^4 5.9 and 4.4, 16^2 x 8 x 4 (4096 links) 6.0 and 5.4, 16^3 x 4
-// (8192) 6.4 and 7.4; with the draws before the wait (k_update) 8^3 x 4 takes
-// 3.7 and 8^4 3.84.  (Four lanes of two staples each: 4.8, 4.8, 5.1, 5.8.)
-constexpr int kLanesLinks = 4096, kFloatLanes = 16;
+// kFloatLanes): one warp per scheduler.  Per phase, against one thread per
+// link (kFloatEarly below): 12^2 x 8 x 4 (2304 links) 4.05 us and 4.20, 8^4 in
+// four boxes 4.6 and 5.6; 12^3 x 4 (3456) 4.68 and 4.16, 16^2 x 8 x 4 (4096)
+// 5.7 and 4.2.
+constexpr int kLanesLinks = 2432, kFloatLanes = 16;
+// The launchers' variants of the float updates that begin before the previous
+// launch has ended, one thread per link: the second is rolled, and the first
+// too unless the chain is an undivided 4-D torus with the default keys.
+constexpr int kFloatEarly = 17, kFloatEarlyRolled = 18;
 // Chains of one coupling with at most kClusterLinks links per phase run whole
 // sweeps in one launch of a cluster of CTAs (k_sweeps), eight lanes per link.
 // Per phase, against a launch per phase: float 4^4 3.25 us (3.62), 8^3 3.22

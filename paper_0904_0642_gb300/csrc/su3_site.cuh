@@ -271,7 +271,7 @@ __device__ __forceinline__ M3<typename S::R> load_at(const ChainDesc &d, const t
                                                      int j, bool rows2) {
   // the plane offset lies within the (virtual) layers' planes
   if (!in_bounds(p, (long long)d.nlayers * d.nb * 2 * d.D * S::NQ * Vh, kBoundsLink)) return m3_zero<typename S::R>();
-  if constexpr (std::is_same<S, StoreF32x18>::value)
+  if constexpr (sizeof(typename S::Vec) == 8)  // the 18-real float forms
     return rows2 ? S::load2(base + p, Vh, j) : S::load(base + p, Vh, j);
   else
   {
@@ -311,9 +311,14 @@ __device__ __forceinline__ void add_staples_idx(const ChainDesc &d, const typena
 // once per site: forward and backward site offsets and layer flips in every
 // direction, and the plane offsets as multiples of one plane stride.  Same
 // arithmetic, same order as update_site.
-template <class S, bool WT, int DF = 0>
+// EARLY (float): the draws come first, and ready(nu) before the staples of a direction.
+struct NotEarly {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+template <class S, bool WT, int DF = 0, bool EARLY = false, class Ready = NotEarly>
 __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
-                                                 int jj, uint32_t &nprop, uint32_t &nacc, typename S::R &dretr) {
+                                                 int jj, uint32_t &nprop, uint32_t &nacc, typename S::R &dretr,
+                                                 Ready &&ready = Ready()) {
   using R = typename S::R;
   using Vec = typename S::Vec;
   // DF > 0: every chain of the launch is a periodic torus (one layer) of
@@ -349,10 +354,13 @@ __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sw
   const int pmu_oc = oc * CS + mu * PS;  // plane (oc, mu) within a layer
   const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
   const uint32_t skey = kTorus ? (uint32_t)s : site_key<false>(d, g);  // the torus form has the default key
+  [[maybe_unused]] DrawPre pre[3];
+  if constexpr (EARLY) cm_draws_f(pre, key, skey, sweep, colour, mu);
   M3<R> A = m3_zero<R>();
 #pragma unroll
   for (int nu = 0; nu < kMaxD; ++nu) {
     if (nu < D && nu != mu) {
+      ready(nu);
       const int lb = layer ^ ff[nu], lm = layer ^ fb[nu], lf = lp ^ fb[nu];
       const int sm = s + ob[nu];
       add_staples_idx<S, WT>(d, base, Vh,
@@ -368,7 +376,9 @@ __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sw
   typename S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
   M3<R> U = S::load(pu, Vh, jj);
   const R beta = (WT && d.weighted) ? R(1) : (sizeof(R) == 4 ? (R)d.beta_f : (R)d.beta_d);
-  if constexpr (sizeof(R) == 4)
+  if constexpr (EARLY)
+    cm_apply_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, pre, nprop, nacc, dretr);
+  else if constexpr (sizeof(R) == 4)
     cm_update_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
   else
     cm_update(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
@@ -377,9 +387,10 @@ __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sw
 
 // ROLLED: the loop over staple directions stays a loop (no unrolling), so the
 // compiler cannot hoist later directions' loads; fewer registers, less code.
-template <class S, bool ROLLED, bool WT, bool SUB>
+template <class S, bool ROLLED, bool WT, bool SUB, bool EARLY = false, class Ready = NotEarly>
 __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer, int jj,
-                                            uint32_t &nprop, uint32_t &nacc, typename S::R &dretr) {
+                                            uint32_t &nprop, uint32_t &nacc, typename S::R &dretr,
+                                            Ready &&ready = Ready()) {
   using R = typename S::R;
   const int Vh = d.Vh;
   const SiteGeo g = site_of<SUB>(d, layer, colour, jj);
@@ -389,11 +400,16 @@ __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, 
   const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
   const uint32_t skey = site_key<SUB>(d, g);
 
+  [[maybe_unused]] DrawPre pre[3];
+  if constexpr (EARLY) cm_draws_f(pre, key, skey, sweep, colour, mu);
   M3<R> A = m3_zero<R>();
   if constexpr (ROLLED) {
 #pragma unroll 1
     for (int nu = 0; nu < d.D; ++nu)
-      if (nu != mu) add_staples<S, WT, SUB>(d, g, colour, mu, nu, sel(g.x, nu), sp, lp, A);
+      if (nu != mu) {
+        ready(nu);
+        add_staples<S, WT, SUB>(d, g, colour, mu, nu, sel(g.x, nu), sp, lp, A);
+      }
   } else {
 #pragma unroll
     for (int nu = 0; nu < kMaxD; ++nu)
@@ -403,7 +419,9 @@ __device__ __forceinline__ void update_site(const ChainDesc &d, uint32_t sweep, 
   const int ju = g.s >> 1;  // jj itself unless the site sits in a padded box
   M3<R> U = S::load(pu, Vh, ju);
   const R beta = (WT && d.weighted) ? R(1) : (sizeof(R) == 4 ? (R)d.beta_f : (R)d.beta_d);
-  if constexpr (sizeof(R) == 4)
+  if constexpr (EARLY)
+    cm_apply_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, pre, nprop, nacc, dretr);
+  else if constexpr (sizeof(R) == 4)
     cm_update_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
   else
     cm_update(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
@@ -1559,6 +1577,14 @@ template <> struct TickBounds<10> { static constexpr int kThreads = 256, kMinBlo
 template <> struct TickBounds<kCoopVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP64, eight lanes per link
 
 template <> struct TickBounds<kLanesVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };  // FP32, eight lanes per link
+// FP32, one thread per link, begun before the previous launch has ended
+// (k_update): all registers (at most 8 warps per SM), unrolled for 4-D tori
+// and rolled.
+constexpr int kEarlyVariant = 13, kEarlyRolled = 14;
+template <int V>
+constexpr bool kIsEarly = V == kEarlyVariant || V == kEarlyRolled;
+template <> struct TickBounds<kEarlyVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };
+template <> struct TickBounds<kEarlyRolled> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = true; };
 
 // ------------------------------------------------------------------ one tile of an update phase
 
@@ -1643,9 +1669,9 @@ __device__ __forceinline__ WarpPlace warp_place(const ChainDesc &d, int lt) {
 }
 
 // The updates of one CTA's tile lt of a chain's phase (colour, mu).
-template <class S, int V, bool WT, bool SUB, bool TOR>
+template <class S, int V, bool WT, bool SUB, bool TOR, class Ready = NotEarly>
 __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, int colour, int mu, int lt,
-                                            uint32_t &np, uint32_t &na) {
+                                            uint32_t &np, uint32_t &na, Ready &&ready = Ready()) {
   const WarpPlace p = warp_place<kLanesOf<V>>(d, lt);
   const int layer = p.layer;
   if constexpr (kLanesOf<V> > 1) {
@@ -1666,7 +1692,11 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
     } else {
       typename S::R dr = 0;  // in the kernel's precision
       if (valid) {
-        if constexpr (TOR)
+        if constexpr (kIsEarly<V> && TickBounds<V>::kRolled)
+          update_site<S, true, WT, SUB, true>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
+        else if constexpr (kIsEarly<V>)
+          update_site_lean<S, false, 4, true>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
+        else if constexpr (TOR)
           update_site_lean<S, false, 4>(d, sweep, colour, mu, layer, jj, np, na, dr);
         else if constexpr (!TickBounds<V>::kRolled && !SUB)
           update_site_lean<S, WT>(d, sweep, colour, mu, layer, jj, np, na, dr);

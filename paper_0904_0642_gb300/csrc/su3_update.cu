@@ -49,6 +49,34 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
       p = warp_place<kCoopLanes>(d, lt);
       if (p.jw < d.Vn) w.prepare(d, base + u.offset, u.colour, u.mu, p.layer, p.jw);
     }
+  } else if constexpr (kIsEarly<V>) {
+    // A launch that leaves room on the GPU runs beside its predecessor: all
+    // but what depends on that one comes before the wait.  The previous
+    // launch writes links of direction prev only, so the draws, and the sums
+    // over the staples up to those of direction prev, do not wait (in the
+    // sums' order: three of the four directions of a 4-D sweep gain).  The
+    // launch before that has ended: every CTA of the previous one waited for
+    // it.  Links come from L2: only the wait makes L1 forget what this SM
+    // read before earlier launches wrote.
+    bool waited = u.early == 0;
+    uint32_t base;
+    if (waited) {
+      wait_previous();
+      base = next_base(ctl, u);
+    } else {
+      base = __ldcg(&ctl->cur);
+    }
+    const int prev = u.mu == 0 ? d.D - 1 : u.mu - 1;
+    const auto ready = [&](int nu) {
+      if (!waited && nu == prev) {
+        wait_previous();
+        waited = true;
+      }
+    };
+    for (int lt = blockIdx.x; lt < u.tiles; lt += gridDim.x)
+      update_tile<S, V, WT, SUB, TOR>(d, base + u.offset, u.colour, u.mu, lt, np, na, ready);
+    ready(prev);  // a thread without a link
+    if (u.advance && blockIdx.x == 0 && threadIdx.x == 0) ctl->nxt = base + u.advance;
   } else {
     wait_previous();
     const uint32_t base = next_base(ctl, u);
@@ -259,6 +287,17 @@ static cudaError_t update_dispatch(int storage, int variant, bool sub, bool toru
     return sub ? OP<StoreF32x12, kLanesVariant, false, true, false>::run(a...)
                : OP<StoreF32x12, kLanesVariant, false, false, false>::run(a...);
   }
+  // (links read before the wait come from L2: the coherent store forms)
+  if (variant == kFloatEarly && tor)
+    return storage == 2 ? OP<StoreF32x18T<true>, kEarlyVariant, false, false, kT>::run(a...)
+                        : OP<StoreF32x12T<true>, kEarlyVariant, false, false, kT>::run(a...);
+  if (variant >= kFloatEarly && !WT) {
+    if (storage == 2)
+      return sub ? OP<StoreF32x18T<true>, kEarlyRolled, false, true, false>::run(a...)
+                 : OP<StoreF32x18T<true>, kEarlyRolled, false, false, false>::run(a...);
+    return sub ? OP<StoreF32x12T<true>, kEarlyRolled, false, true, false>::run(a...)
+               : OP<StoreF32x12T<true>, kEarlyRolled, false, false, false>::run(a...);
+  }
   if (storage == 2) {
     if (sub) return OP<StoreF32x18, kSubVariant, WT, true, false>::run(a...);
     return tor ? OP<StoreF32x18, 0, false, false, kT>::run(a...) : OP<StoreF32x18, 0, WT, false, false>::run(a...);
@@ -275,7 +314,7 @@ static cudaError_t update_dispatch(int storage, int variant, bool sub, bool toru
 
 cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, bool torus, const ChainDesc &d,
                           ChainCtl *ctl, const UpdateStep &step, int grid, int block, cudaStream_t st, bool pdl) {
-  if (sub && storage != 0 && variant != kFloatLanes) variant = kSubVariant;
+  if (sub && storage != 0 && variant < kFloatLanes) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaErrorInvalidConfiguration;
   const ChainDesc *pd = &d;
   const UpdateStep *pu = &step;
@@ -286,7 +325,7 @@ cudaError_t launch_update(int storage, int variant, bool weighted, bool sub, boo
 cudaError_t update_occupancy(int storage, int variant, bool weighted, bool sub, bool torus, int block,
                              int *ctas_per_sm) {
   *ctas_per_sm = 0;
-  if (sub && storage != 0 && variant != kFloatLanes) variant = kSubVariant;
+  if (sub && storage != 0 && variant < kFloatLanes) variant = kSubVariant;
   if (block > tick_max_threads(storage, variant)) return cudaSuccess;
   return weighted ? update_dispatch<UpdateOccupancy, true>(storage, variant, sub, torus, block, ctas_per_sm)
                   : update_dispatch<UpdateOccupancy, false>(storage, variant, sub, torus, block, ctas_per_sm);
