@@ -461,10 +461,12 @@ struct Engine {
   bool cluster = false;       // fixed, fewest links: whole sweeps per launch (k_sweeps)
   bool coop = false;          // too few links to fill the GPU: eight lanes per link
   int early = 0;              // the form of an update begun before the previous launch has ended (0: none)
+  int parked = 0;             // the form of an update with its draws parked in shared memory (0: none)
   int tile() const { return coop ? block / kCoopLanes : block; }  // sites of a CTA's tile
   int kernel_variant() const {
     if (coop) return storage == SU3_FP64_18 ? 1 : kFloatLanes;
     if (early) return early;
+    if (parked) return parked;
     return ctas_per_sm == kAutoCtas ? auto_variant : variant;
   }
   // The register variant of a two-row float chain without another form, until
@@ -486,6 +488,23 @@ struct Engine {
   static int early_for(long long warps, int nsm) {
     if (warps > 8ll * nsm) return 0;
     return warps <= 4ll * nsm ? kFloatEarlyRolled : kFloatEarly;
+  }
+  // The form of an undivided one-coupling float chain whose update fits the GPU
+  // in one round but not in the early form: its draws, computed before the
+  // wait, lie in shared memory until the staples are summed.  kFloatParked1
+  // (20 warps per SM, two-row links) where two launches fit side by side or 16
+  // warps per SM are too few, kFloatParked0 (16 warps) between.  Per phase,
+  // without and with it: 18^3 x 14 10.1 and 8.5 us (18 reals 10.8 and 9.6),
+  // 20^3 x 16 10.4 and 9.5 (11.0 and 10.0), 20^4 12.9 and 11.7, 52^3 9.2 and
+  // 8.6, 400^2 9.9 and 9.0.  Beyond one round the shared memory costs L1 that
+  // the links need (64^3 15.9 and 16.2, 24^4 22.1 and 24.1, 32^4 65 and 81;
+  // 18 reals 20^4 15.5 and 15.9).  Not for persistent grids, which ask for
+  // their rounds (20^4 on 4 CTAs per SM 14.2 and 17.0).
+  int parked_for(long long warps, int nsm) const {
+    if (ctas_per_sm > 0 || warps > 20ll * nsm) return 0;
+    const bool one = storage == SU3_FP32_12 && block <= kParkedThreads1;
+    if (one && (warps <= 10ll * nsm || warps > 16ll * nsm)) return kFloatParked1;
+    return warps <= 16ll * nsm ? kFloatParked0 : 0;
   }
   // The links of one update phase of an FP64 chain that may take eight lanes
   // per link (others: more than any limit).
@@ -872,8 +891,11 @@ struct Engine {
     int nsm = 0;
     TRY(device_sm_count(&nsm));
     const int ef = fixed && !coop && !w && storage != SU3_FP64_18 ? early_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
-    if (ef != early) drop_graph();
+    const int pf = fixed && !coop && !w && !sb && !ef && storage != SU3_FP64_18
+                       ? parked_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
+    if (ef != early || pf != parked) drop_graph();
     early = ef;
+    parked = pf;
     if (ctas_per_sm == kAutoCtas) {
       auto_variant = fixed && !sb && storage == SU3_FP32_12 ? variant_for((phase_links(chains[0]) + 31) / 32, nsm) : 0;
       TRY(count_resident());

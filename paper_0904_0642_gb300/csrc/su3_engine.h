@@ -57,6 +57,9 @@ constexpr int kLanesLinks = 2432, kFloatLanes = 16;
 // launch has ended, one thread per link: the second is rolled, and the first
 // too unless the chain is an undivided 4-D torus with the default keys.
 constexpr int kFloatEarly = 17, kFloatEarlyRolled = 18;
+// The launchers' variants of the float updates whose draws alone come before
+// that wait (128 and 96 registers; the second up to kParkedThreads1 threads).
+constexpr int kFloatParked0 = 19, kFloatParked1 = 20, kParkedThreads1 = 128;
 // Chains of one coupling with at most kClusterLinks links per phase run whole
 // sweeps in one launch of a cluster of CTAs (k_sweeps), eight lanes per link.
 // Per phase, against a launch per phase: float 4^4 3.25 us (3.62), 8^3 3.22

@@ -691,6 +691,7 @@ struct TickOccupancy {
 
 int tick_max_threads(int storage, int variant) {
   if (storage == 0) return TickBounds<10>::kThreads;
+  if (variant == kFloatParked1) return kParkedThreads1;
   if (storage == 2 || variant >= kFloatLanes) return TickBounds<0>::kThreads;
   switch (variant) {
     case 0: return TickBounds<0>::kThreads;

@@ -307,15 +307,41 @@ __device__ __forceinline__ void add_staples_idx(const ChainDesc &d, const typena
     acc_su3_2rows(A, mul_dn_2(ef, h));
 }
 
+// A thread's draws parked in shared memory, in slots of its own (no barrier).
+constexpr int kParkedBytes = 9 * sizeof(float2);  // per thread
+__device__ __forceinline__ float2 *parked_draws() {
+  extern __shared__ float2 s_parked[];
+  return s_parked + threadIdx.x;
+}
+__device__ __forceinline__ void park_draws(const DrawPre (&pre)[3]) {
+  float2 *p = parked_draws();
+#pragma unroll
+  for (int g = 0; g < 3; ++g) {
+    p[(3 * g) * blockDim.x] = make_float2(pre[g].L, pre[g].u4sq);
+    p[(3 * g + 1) * blockDim.x] = make_float2(pre[g].costh, pre[g].sinth);
+    p[(3 * g + 2) * blockDim.x] = make_float2(pre[g].cphi, pre[g].sphi);
+  }
+}
+__device__ __forceinline__ void unpark_draws(DrawPre (&pre)[3]) {
+  const float2 *p = parked_draws();
+#pragma unroll
+  for (int g = 0; g < 3; ++g) {
+    const float2 a = p[(3 * g) * blockDim.x], b = p[(3 * g + 1) * blockDim.x], c = p[(3 * g + 2) * blockDim.x];
+    pre[g] = DrawPre{a.x, a.y, b.x, b.y, c.x, c.y};
+  }
+}
+struct NotEarly {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+
 // update_site for an undivided lattice with the neighbour geometry computed
 // once per site: forward and backward site offsets and layer flips in every
 // direction, and the plane offsets as multiples of one plane stride.  Same
 // arithmetic, same order as update_site.
-// EARLY (float): the draws come first, and ready(nu) before the staples of a direction.
-struct NotEarly {
-  __device__ __forceinline__ void operator()(int) const {}
-};
-template <class S, bool WT, int DF = 0, bool EARLY = false, class Ready = NotEarly>
+// EARLY 1: the draws first, in registers, and ready(nu) before the staples of
+// a direction.  EARLY 2: the draws first, parked in shared memory (a thread's
+// own slots) until the staples are summed, and ready(-1) before the staples.
+template <class S, bool WT, int DF = 0, int EARLY = 0, class Ready = NotEarly>
 __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sweep, int colour, int mu, int layer,
                                                  int jj, uint32_t &nprop, uint32_t &nacc, typename S::R &dretr,
                                                  Ready &&ready = Ready()) {
@@ -355,12 +381,16 @@ __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sw
   const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
   const uint32_t skey = kTorus ? (uint32_t)s : site_key<false>(d, g);  // the torus form has the default key
   [[maybe_unused]] DrawPre pre[3];
-  if constexpr (EARLY) cm_draws_f(pre, key, skey, sweep, colour, mu);
+  if constexpr (EARLY > 0) cm_draws_f(pre, key, skey, sweep, colour, mu);
+  if constexpr (EARLY == 2) {
+    park_draws(pre);
+    ready(-1);
+  }
   M3<R> A = m3_zero<R>();
 #pragma unroll
   for (int nu = 0; nu < kMaxD; ++nu) {
     if (nu < D && nu != mu) {
-      ready(nu);
+      if constexpr (EARLY == 1) ready(nu);
       const int lb = layer ^ ff[nu], lm = layer ^ fb[nu], lf = lp ^ fb[nu];
       const int sm = s + ob[nu];
       add_staples_idx<S, WT>(d, base, Vh,
@@ -376,7 +406,8 @@ __device__ __forceinline__ void update_site_lean(const ChainDesc &d, uint32_t sw
   typename S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
   M3<R> U = S::load(pu, Vh, jj);
   const R beta = (WT && d.weighted) ? R(1) : (sizeof(R) == 4 ? (R)d.beta_f : (R)d.beta_d);
-  if constexpr (EARLY)
+  if constexpr (EARLY == 2) unpark_draws(pre);
+  if constexpr (EARLY > 0)
     cm_apply_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, pre, nprop, nacc, dretr);
   else if constexpr (sizeof(R) == 4)
     cm_update_f(U, A, beta, d.hits, key, skey, sweep, colour, mu, nprop, nacc, dretr);
@@ -1583,6 +1614,12 @@ template <> struct TickBounds<kLanesVariant> { static constexpr int kThreads = 2
 constexpr int kEarlyVariant = 13, kEarlyRolled = 14;
 template <int V>
 constexpr bool kIsEarly = V == kEarlyVariant || V == kEarlyRolled;
+// FP32, draws parked in shared memory: variants 0 and 1 otherwise.
+constexpr int kParked0 = 15, kParked1 = 16;
+template <int V>
+constexpr bool kIsParked = V == kParked0 || V == kParked1;
+template <> struct TickBounds<kParked0> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };
+template <> struct TickBounds<kParked1> { static constexpr int kThreads = kParkedThreads1, kMinBlocks = 5; static constexpr bool kRolled = false; };
 template <> struct TickBounds<kEarlyVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };
 template <> struct TickBounds<kEarlyRolled> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = true; };
 
@@ -1695,7 +1732,9 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
         if constexpr (kIsEarly<V> && TickBounds<V>::kRolled)
           update_site<S, true, WT, SUB, true>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
         else if constexpr (kIsEarly<V>)
-          update_site_lean<S, false, 4, true>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
+          update_site_lean<S, false, 4, 1>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
+        else if constexpr (kIsParked<V>)
+          update_site_lean<S, false, TOR ? 4 : 0, 2>(d, sweep, colour, mu, layer, jj, np, na, dr, ready);
         else if constexpr (TOR)
           update_site_lean<S, false, 4>(d, sweep, colour, mu, layer, jj, np, na, dr);
         else if constexpr (!TickBounds<V>::kRolled && !SUB)
@@ -1718,8 +1757,10 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
 // stream (the kernel waits for that one's completion and memory at its first
 // instruction, so only the launch itself overlaps the previous kernel).
 template <class... P, class... A>
-static cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, int block, cudaStream_t st, bool pdl, A &&...a) {
+static cudaError_t launch_shared(void (*kernel)(P...), dim3 grid, int block, size_t smem, cudaStream_t st, bool pdl,
+                                 A &&...a) {
   cudaLaunchConfig_t cfg = {};
+  cfg.dynamicSmemBytes = smem;
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
   cfg.stream = st;
@@ -1729,6 +1770,10 @@ static cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, int block, cudaStr
   cfg.attrs = attr;
   cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(a)...);
+}
+template <class... P, class... A>
+static cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, int block, cudaStream_t st, bool pdl, A &&...a) {
+  return launch_shared(kernel, grid, block, 0, st, pdl, std::forward<A>(a)...);
 }
 
 // Run f with a value of the storage form of `storage` (0: FP64 18-real,

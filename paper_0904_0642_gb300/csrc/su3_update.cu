@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
       p = warp_place<kCoopLanes>(d, lt);
       if (p.jw < d.Vn) w.prepare(d, base + u.offset, u.colour, u.mu, p.layer, p.jw);
     }
-  } else if constexpr (kIsEarly<V>) {
+  } else if constexpr (kIsEarly<V> || kIsParked<V>) {
     // A launch that leaves room on the GPU runs beside its predecessor: all
     // but what depends on that one comes before the wait.  The previous
     // launch writes links of direction prev only, so the draws, and the sums
@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
     // sums' order: three of the four directions of a 4-D sweep gain).  The
     // launch before that has ended: every CTA of the previous one waited for
     // it.  Links come from L2: only the wait makes L1 forget what this SM
-    // read before earlier launches wrote.
+    // read before earlier launches wrote.  The parked forms have only the
+    // draws before the wait and read links as ever.
     bool waited = u.early == 0;
     uint32_t base;
     if (waited) {
@@ -68,7 +69,7 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
     }
     const int prev = u.mu == 0 ? d.D - 1 : u.mu - 1;
     const auto ready = [&](int nu) {
-      if (!waited && nu == prev) {
+      if (!waited && (kIsParked<V> || nu == prev)) {
         wait_previous();
         waited = true;
       }
@@ -255,17 +256,23 @@ __global__ void k_set_ctl(ChainCtl *ctl, uint32_t sweep, uint32_t n_meas, int an
 
 constexpr int kSubVariant = 3;  // the FP32 variant of a divided chain
 
+// Dynamic shared memory per thread.
+template <int V>
+constexpr int kSharedOf = kIsParked<V> ? kParkedBytes : 0;
+
 template <class S, int V, bool WT, bool SUB, bool TOR>
 struct UpdateLaunch {
   static cudaError_t run(const ChainDesc *d, ChainCtl *ctl, const UpdateStep *u, int grid, int block, cudaStream_t st,
                          bool pdl) {
-    return launch_ex(k_update<S, V, WT, SUB, TOR>, dim3((unsigned)grid), block, st, pdl, *d, ctl, *u);
+    return launch_shared(k_update<S, V, WT, SUB, TOR>, dim3((unsigned)grid), block, kSharedOf<V> * block, st, pdl, *d,
+                         ctl, *u);
   }
 };
 template <class S, int V, bool WT, bool SUB, bool TOR>
 struct UpdateOccupancy {
   static cudaError_t run(int block, int *ctas) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_update<S, V, WT, SUB, TOR>, block, 0);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(ctas, k_update<S, V, WT, SUB, TOR>, block,
+                                                         kSharedOf<V> * block);
   }
 };
 
@@ -291,6 +298,13 @@ static cudaError_t update_dispatch(int storage, int variant, bool sub, bool toru
   if (variant == kFloatEarly && tor)
     return storage == 2 ? OP<StoreF32x18T<true>, kEarlyVariant, false, false, kT>::run(a...)
                         : OP<StoreF32x12T<true>, kEarlyVariant, false, false, kT>::run(a...);
+  if (variant == kFloatParked1 && storage == 1 && !WT && !sub)
+    return tor ? OP<StoreF32x12, kParked1, false, false, kT>::run(a...) : OP<StoreF32x12, kParked1, false, false, false>::run(a...);
+  if (variant == kFloatParked0 && !WT && !sub) {
+    if (storage == 2)
+      return tor ? OP<StoreF32x18, kParked0, false, false, kT>::run(a...) : OP<StoreF32x18, kParked0, false, false, false>::run(a...);
+    return tor ? OP<StoreF32x12, kParked0, false, false, kT>::run(a...) : OP<StoreF32x12, kParked0, false, false, false>::run(a...);
+  }
   if (variant >= kFloatEarly && !WT) {
     if (storage == 2)
       return sub ? OP<StoreF32x18T<true>, kEarlyRolled, false, true, false>::run(a...)

@@ -1,5 +1,5 @@
 """The float update forms of one-chain engines (eight lanes per link, updates
-begun before the previous launch has ended, plain) against the stage machine
+begun before the previous launch has ended, parked draws, plain) against the stage machine
 of a fused launch, bit for bit, on both sides of the lines between them."""
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 F12, F18 = su3.SU3_FP32_12, su3.SU3_FP32_18
 DLT = dict(boundary=su3.SU3_DLT)
 
-CASES = [  # links of a phase, one warp per scheduler and two per scheduler (152 SMs)
+CASES = [  # links of a phase (152 SMs)
     ("lanes-ragged", [6, 6, 10, 2], F12, {}),                    # 360
     ("lanes-D3", [14, 14, 12], F18, {}),                         # 1176
     ("lanes-dlt", [10, 6, 6, 4], F18, DLT),                      # 1440
@@ -24,7 +24,13 @@ CASES = [  # links of a phase, one warp per scheduler and two per scheduler (152
     ("early-torus", [16, 16, 16, 10], F12, {}),                  # 20480: unrolled
     ("early-torus-18", [18, 18, 18, 12], F18, {}),               # 34992
     ("early-D3-two", [64, 32, 34], F12, {}),                     # 34816: rolled, two warps per scheduler
-    ("plain", [18, 18, 18, 14], F12, {}),                        # 40824
+    ("parked-torus", [18, 18, 18, 14], F12, {}),                 # 40824
+    ("parked-18", [20, 20, 20, 16], F18, {}),                    # 64000
+    ("parked-period", [18, 18, 18, 18], F12, dict(rng_period=[18, 18, 18, 6])),  # 52488
+    ("parked-dlt", [20, 20, 20, 10], F12, DLT),                  # 80000
+    ("parked-last", [54, 60, 60], F12, {}),                      # 97200: 20 warps per SM are 97280 links
+    ("plain-first", [56, 60, 60], F12, {}),                      # 100800
+    ("plain-18", [20, 20, 20, 20], F18, {}),                     # 80000
 ]
 
 
