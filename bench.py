@@ -61,7 +61,7 @@ def kernel_hash():
     """Hash of the kernel sources with comments and blank lines removed, so
     that recorded ncu counters stay valid across comment edits."""
     h = hashlib.sha256()
-    for f in ("su3_device.cuh", "su3_kernels.cu", "su3_engine.h"):
+    for f in ("su3_device.cuh", "su3_fixed.cuh", "su3_site.cuh", "su3_update.cu", "su3_kernels.cu", "su3_engine.h"):
         with open(os.path.join(ROOT, "paper_0904_0642_gb300", "csrc", f)) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         for ln in src.splitlines():
@@ -612,8 +612,8 @@ def main():
         alg_bytes = (V // 2) * (2 * len(DIMS) + 1) * 48
         achieved = alg_bytes / (upd_ms * 1e-3) / 1e9
         line["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
-                            "frac": achieved / peaks["hbm_gbs"], "traffic": recorded_traffic("k_tick_fp32_update"),
-                            "peak_source": f"hbm_gbs of {peak_src}", "kernel": "k_tick<StoreF32x12> update phase",
+                            "frac": achieved / peaks["hbm_gbs"], "traffic": recorded_traffic("k_update_fp32"),
+                            "peak_source": f"hbm_gbs of {peak_src}", "kernel": "k_update<StoreF32x12>",
                             "alg_bytes_per_launch": alg_bytes, "avg_launch_us": upd_ms * 1e3,
                             "tick_source": "graph-timed: (T(20 sweeps, re-unitarised every 20) - T(10 sweeps, "
                                            "every 10)) / 80 update ticks",

@@ -114,9 +114,10 @@ su3_status su3_lattice_create(int D, const int *dims, su3_boundary boundary, dou
  * is cut into ndiv[i] sublattices along direction i, each of interior
  * extent n^i / ndiv[i] (even, >= 2, else EINVAL).  Every sublattice keeps
  * its links in its own box with one halo layer on both sides of each cut
- * direction; after every tick that changes links a halo kernel copies the
- * changed links (faces, and the corner links when two or more directions
- * are cut) from the sublattice that owns them.  The random numbers are
+ * direction; an update writes the copies of its links in the halos of the
+ * other boxes too (faces, and the corner links when two or more directions
+ * are cut), and a halo kernel refreshes them all after a re-unitarisation
+ * and when links are replaced.  The random numbers are
  * keyed by the undivided site, so results are bitwise those of the
  * undivided lattice.  Not with a caller-owned link buffer, ensembles or
  * the server, nor with two couplings on a DLT cut along a glued direction
@@ -259,8 +260,13 @@ su3_status su3_lattice_info(su3_lattice *lat, size_t *links, size_t *bytes);
  * only).  threads:
  * CTA width, a multiple of 32 up to the variant's maximum.  ctas_per_sm = 0
  * launches one CTA per tile of `threads` sites; > 0 a persistent grid of
- * (SM count x ctas_per_sm) CTAs that loop over the tiles.  The random
- * numbers do not depend on the shape, so results are identical for every
+ * (SM count x ctas_per_sm) CTAs that loop over the tiles.  Until the first
+ * call, variant and grid follow from the number of tiles (128 threads).
+ * Chains that leave the GPU partly idle (few links, or less than a round of
+ * its warps on a grid of one CTA per tile) run an update of their own form
+ * whatever the variant; threads and ctas_per_sm hold for it too, except that
+ * a chain of at most 256 links per phase runs whole sweeps in one launch of
+ * fixed shape.  The random numbers do not depend on the shape, so results are identical for every
  * choice.  su3_autotune times the candidates on this lattice, each from the
  * same links (links, counters and sweep counter are restored afterwards),
  * and keeps the fastest; outputs may be NULL. */
@@ -273,8 +279,8 @@ su3_status su3_use_graph(su3_lattice *lat, int on);
 
 /* Launch each update tick as a programmatic dependent of the previous one
  * (on by default): the next tick is scheduled while the previous one ends
- * and waits at its first instruction for the previous tick's completion
- * and memory, so results are identical either way.  Where the driver
+ * and waits for the previous tick's completion and memory before it touches
+ * what that one writes, so results are identical either way.  Where the driver
  * refuses such launches the library falls back to ordinary ones. */
 su3_status su3_use_pdl(su3_lattice *lat, int on);
 

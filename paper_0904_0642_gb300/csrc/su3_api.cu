@@ -858,7 +858,9 @@ struct Engine {
       weighted = weighted || ch.desc.weighted;
     }
     // eight lanes per link: FP64, and one-chain float engines, with few links
-    const bool cp = !weighted && (storage == SU3_FP64_18 ? sites <= kCoopSites
+    const int D = fixed ? chains[0].cfg.D : 4;
+    const int most = D > 3 ? kCoopSites : D == 3 ? kCoopSites3 : kCoopSites2;
+    const bool cp = !weighted && (storage == SU3_FP64_18 ? sites <= most
                                                          : fixed && phase_links(chains[0]) <= kLanesLinks);
     if (cp != coop) drop_graph();
     coop = cp;

@@ -40,11 +40,15 @@ constexpr float kAlphaAccurateLog = 2.0f;
 
 // FP64 chains of one coupling with at most kCoopSites links per update phase
 // take eight lanes per link (update_site_coop): a tile then holds an eighth
-// of a CTA's threads.  One thread per link takes 35 us per phase for any
-// lattice below one wave (38912 links at 8 warps per SM); eight lanes take
-// 15 us per wave of 4864 links, so the line lies at two waves, rounded down.
+// of a CTA's threads.  In 4-D one thread per link takes 33 us per phase for
+// any lattice below one wave (38912 links at 8 warps per SM), eight lanes 12
+// us for few links, 16 for a full wave of 4864 and 30.4 for 8192 links.  A
+// one-chain engine of fewer dimensions has fewer staples than lanes and leaves
+// them sooner.  With and without lanes, 3-D: 22^3 (5324 links) 26.2 and 27.3
+// us, 24^2 x 22 (6336) 28.9 and 27.3, 24^3 (6912) 30.1 and 27.7; 2-D: 96 x 100
+// (4800) 17.0 and 21.0, 108 x 100 (5400) 27.7 and 22.3, 128^2 32.7 and 22.0.
 constexpr int kCoopLanes = 8;
-constexpr int kCoopSites = 8192;
+constexpr int kCoopSites = 8192, kCoopSites3 = 5632, kCoopSites2 = 4864;
 
 // Float chains of one coupling with at most kLanesLinks links per phase take
 // eight lanes per link too (update_site_lanes; the launchers' variant

@@ -14,11 +14,12 @@
 // result is read as hh 2^32 + x, rounded to units 2^-60.  Every rounding is
 // thus 2^-57 or less, against 2^-54 to 2^-52 in the double-precision form.
 //
-// Measured, one update phase: 24^4 (165888 links) 900 us in double, 240 us
-// here; 4^4 (128 links) 97 us in double, 35 us here, 15 us with eight lanes
-// per link.  What bounds it: the integer pipes (46 % of the wide
-// multiply-adds' rate, at 8 warps per SM and 255 registers) and instruction
-// fetch; 168 and 128 registers (12 and 16 warps per SM) are 8 and 16 % slower.
+// Measured, one update phase: 24^4 (165888 links) 900 us in double, 218 us
+// here; 4^4 (128 links) 97 us in double, 32 us here, 11.4 us with eight lanes
+// per link.  What bounds it: the integer pipes (53 % of the wide
+// multiply-adds' rate and 42 % of the logic's, which share the dispatch, at 8
+// warps per SM and 255 registers); 168 and 128 registers (12 and 16 warps per
+// SM) are 8 and 16 % slower.
 //
 // Overflow.  The bounds below hold for any inputs with every element at most
 // kElemMax in magnitude (no unitarity assumed), and the results of one stage

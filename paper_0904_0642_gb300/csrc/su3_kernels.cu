@@ -1,15 +1,17 @@
 // su3_kernels.cu -- CUDA kernels of the checkerboard SU(3) heatbath (sm_103a).
 //
-// k_tick: one persistent launch advances every resident chain by one stage
-//   (a (colour, direction) update phase, a re-unitarisation or a
-//   measurement).  One thread per site of the tile (tile = CTA width); tiles
-//   of all chains are spread over a grid of CTAs sized to the SM count.
-//   The chains' stage machines advance at the end of the launch (one
-//   chain: by the last warp to finish; several: by the first, into a second
-//   state slot, with the last one flipping the slot parity), and the last
-//   warp reduces measurement partial sums in a fixed order.
-// k_start, k_convert, k_measure*: start configurations, canonical-layout
-//   conversion and stand-alone measurements.
+// k_tick (engines of several chains, the server's): one persistent launch
+//   advances every resident chain by one stage (a (colour, direction) update
+//   phase, a re-unitarisation or a measurement).  One thread per site of the
+//   tile (tile = CTA width); tiles of all chains are spread over a grid of
+//   CTAs sized to the SM count.  The chains' stage machines advance at the end
+//   of the launch (by the first warp to finish, into a second state slot, with
+//   the last one flipping the slot parity; one resident chain: by the last
+//   warp), and the last warp reduces measurement partial sums in a fixed
+//   order.  An engine of one chain runs the kernels of su3_update.cu.
+// k_start, k_convert, k_halo, k_sub_copy, k_measure_noalloc: start
+//   configurations, canonical-layout conversion, the boxes of a divided
+//   lattice and measurements of links the caller holds.
 #include <cstdio>
 #include <mutex>
 #include <type_traits>

@@ -1,4 +1,4 @@
-"""The float update forms of one-chain engines (eight lanes per link, updates
+"""The update forms of one-chain engines (eight lanes per link, updates
 begun before the previous launch has ended, parked draws, plain) against the stage machine
 of a fused launch, bit for bit, on both sides of the lines between them."""
 import numpy as np
@@ -8,7 +8,7 @@ import paper_0904_0642_gb300 as su3
 
 pytestmark = pytest.mark.gpu
 
-F12, F18 = su3.SU3_FP32_12, su3.SU3_FP32_18
+F12, F18, F64 = su3.SU3_FP32_12, su3.SU3_FP32_18, su3.SU3_FP64_18
 DLT = dict(boundary=su3.SU3_DLT)
 
 CASES = [  # links of a phase (152 SMs)
@@ -31,6 +31,9 @@ CASES = [  # links of a phase (152 SMs)
     ("parked-last", [54, 60, 60], F12, {}),                      # 97200: 20 warps per SM are 97280 links
     ("plain-first", [56, 60, 60], F12, {}),                      # 100800
     ("plain-18", [20, 20, 20, 20], F18, {}),                     # 80000
+    ("lanes-64-D3", [24, 20, 20], F64, {}),                      # 4800: lanes alone, not with a second chain
+    ("plain-64-D2", [128, 78], F64, {}),                         # 4992
+    ("plain-64-D3", [20, 20, 16], F64, DLT),                     # 6400
 ]
 
 
