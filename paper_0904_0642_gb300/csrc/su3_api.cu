@@ -110,13 +110,22 @@ static const char *bounds_site_name(unsigned long long site) {
   }
 }
 
+// The first recorded violation of any translation unit's kernels.
+static cudaError_t first_violation(unsigned long long r[3]) {
+  cudaError_t (*const units[])(unsigned long long *) = {bounds_record, bounds_record_update, bounds_record_update64,
+                                                        bounds_record_stages};
+  cudaError_t e = cudaSuccess;
+  for (auto *unit : units)
+    if ((e = unit(r)) != cudaSuccess || r[0]) break;
+  return e;
+}
+
 // ECUDA with the first recorded device bounds violation (debug-bounds
 // builds; always OK otherwise).
 static su3_status bounds_status() {
   if (!debug_bounds_build()) return SU3_OK;
   unsigned long long r[3];
-  CU(bounds_record(r));
-  if (!r[0]) CU(bounds_record_update(r));
+  CU(first_violation(r));
   if (r[0])
     return fail(SU3_ECUDA, "device bounds check: %s %lld outside [0, %lld)", bounds_site_name(r[0]), (long long)r[1],
                 (long long)r[2]);
@@ -126,8 +135,7 @@ static su3_status bounds_status() {
 extern "C" su3_status su3_bounds_status(uint64_t *site, int64_t *index, int64_t *extent) {
   unsigned long long r[3] = {0, 0, 0};
   if (debug_bounds_build()) {
-    CU(bounds_record(r));
-    if (!r[0]) CU(bounds_record_update(r));
+    CU(first_violation(r));
   }
   if (site) *site = r[0];
   if (index) *index = (int64_t)r[1];

@@ -1,4 +1,4 @@
-// su3_launch.h -- host-side entry points of the kernels in su3_kernels.cu.
+// su3_launch.h -- host-side entry points of the kernels.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -33,6 +33,13 @@ cudaError_t update_occupancy(int storage, int variant, bool weighted, bool sub, 
 bool sweeps_supported(int storage, bool sub);
 cudaError_t launch_sweeps(int storage, bool sub, const ChainDesc &d, ChainCtl *ctl, int sweeps, cudaStream_t st,
                           bool pdl);
+// The same of FP64 chains (su3_update64.cu), to which the above pass them.
+cudaError_t launch_update64(int variant, bool weighted, bool sub, const ChainDesc &d, ChainCtl *ctl,
+                            const UpdateStep &step, int grid, int block, cudaStream_t st, bool pdl);
+cudaError_t update_occupancy64(int variant, bool weighted, bool sub, int block, int *ctas_per_sm);
+bool sweeps_supported64(bool sub);
+cudaError_t launch_sweeps64(bool sub, const ChainDesc &d, ChainCtl *ctl, int sweeps, cudaStream_t st, bool pdl);
+
 cudaError_t launch_reunit(int storage, bool sub, const ChainDesc &d, cudaStream_t st, bool pdl);
 cudaError_t launch_measure(int storage, bool sub, const ChainDesc &d, double *out, ChainCtl *ctl, cudaStream_t st,
                            bool pdl);
@@ -62,8 +69,10 @@ int noalloc_max_tiles();
 // recorded violation (site, index, extent; site 0: none), and a self-test
 // that records a deliberate violation without any memory access.
 bool debug_bounds_build();
-cudaError_t bounds_record(unsigned long long out[3]);
-cudaError_t bounds_record_update(unsigned long long out[3]);  // of su3_update.cu's kernels
+cudaError_t bounds_record(unsigned long long out[3]);  // of su3_kernels.cu, then of the other units
+cudaError_t bounds_record_update(unsigned long long out[3]);
+cudaError_t bounds_record_update64(unsigned long long out[3]);
+cudaError_t bounds_record_stages(unsigned long long out[3]);
 cudaError_t launch_bounds_selftest();
 cudaError_t launch_measure_noalloc(int storage, const ChainDesc &d, int block, double *out, cudaStream_t st);
 

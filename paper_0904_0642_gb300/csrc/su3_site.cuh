@@ -1753,6 +1753,15 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
 
 // ------------------------------------------------------------------ launching
 
+// Every kernel may be scheduled before the previous one of the stream has
+// finished (programmatic launch): wait for its completion and memory before
+// touching anything, then let the next kernel be scheduled.  Both are no-ops
+// for an ordinary launch.
+__device__ __forceinline__ void wait_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // pdl: launch as a programmatic dependent of the previous kernel in the
 // stream (the kernel waits for that one's completion and memory at its first
 // instruction, so only the launch itself overlaps the previous kernel).
