@@ -483,7 +483,7 @@ def serve_fp64_one_at_a_time(su3, torch, jobs):
 
 
 def bench_serving(su3, torch, peaks):
-    """BASELINE config 5: Poisson arrivals of mixed jobs into the
+    """Poisson arrivals of mixed jobs into the
     continuous-batching server (FP32 12-real links, FP64 re-unitarisation
     and reductions), against a plain FP64 one-job-at-a-time loop under the
     same arrivals."""
