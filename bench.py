@@ -62,7 +62,7 @@ def kernel_hash():
     that recorded ncu counters stay valid across comment edits."""
     h = hashlib.sha256()
     for f in ("su3_device.cuh", "su3_fixed.cuh", "su3_site.cuh", "su3_phase.cuh", "su3_update.cu", "su3_update64.cu",
-              "su3_stages.cu", "su3_kernels.cu", "su3_engine.h"):
+              "su3_stages.cu", "su3_tick.cu", "su3_kernels.cu", "su3_engine.h"):
         with open(os.path.join(ROOT, "paper_0904_0642_gb300", "csrc", f)) as fh:
             src = re.sub(r"/\*.*?\*/", "", fh.read(), flags=re.S)
         for ln in src.splitlines():

@@ -13,7 +13,8 @@ LIB = os.path.join(HERE, "libsu3gb300.so")
 # the same sources with device bounds checks (SU3_DEBUG_BOUNDS)
 BUILD_DBG = os.path.join(HERE, "_build_dbg")
 LIB_DBG = os.path.join(HERE, "libsu3gb300_dbg.so")
-SOURCES = ["su3_update.cu", "su3_update64.cu", "su3_stages.cu", "su3_kernels.cu", "su3_api.cu"]
+SOURCES = ["su3_update.cu", "su3_update64.cu", "su3_tick.cu", "su3_stages.cu", "su3_kernels.cu",
+           "su3_api.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-Wall"]
 

@@ -112,8 +112,8 @@ static const char *bounds_site_name(unsigned long long site) {
 
 // The first recorded violation of any translation unit's kernels.
 static cudaError_t first_violation(unsigned long long r[3]) {
-  cudaError_t (*const units[])(unsigned long long *) = {bounds_record, bounds_record_update, bounds_record_update64,
-                                                        bounds_record_stages};
+  cudaError_t (*const units[])(unsigned long long *) = {bounds_record, bounds_record_tick, bounds_record_update,
+                                                        bounds_record_update64, bounds_record_stages};
   cudaError_t e = cudaSuccess;
   for (auto *unit : units)
     if ((e = unit(r)) != cudaSuccess || r[0]) break;

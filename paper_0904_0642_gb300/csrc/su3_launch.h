@@ -70,6 +70,7 @@ int noalloc_max_tiles();
 // that records a deliberate violation without any memory access.
 bool debug_bounds_build();
 cudaError_t bounds_record(unsigned long long out[3]);  // of su3_kernels.cu, then of the other units
+cudaError_t bounds_record_tick(unsigned long long out[3]);
 cudaError_t bounds_record_update(unsigned long long out[3]);
 cudaError_t bounds_record_update64(unsigned long long out[3]);
 cudaError_t bounds_record_stages(unsigned long long out[3]);

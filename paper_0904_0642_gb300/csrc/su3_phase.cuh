@@ -2,9 +2,10 @@
 // the host knows.  The descriptor is a kernel parameter: geometry and pointers
 // are uniform values from the constant bank, nothing is loaded before the
 // links.  The float forms are compiled in su3_update.cu, the FP64 forms in
-// su3_update64.cu, re-unitarisation and measurement in su3_stages.cu: a module
-// is loaded by a process at the first use of one of its kernels, and the
-// update forms together take 25 ms to load.
+// su3_update64.cu, re-unitarisation and measurement in su3_stages.cu, the fused
+// stage machine of many chains in su3_tick.cu: a module is loaded by a process
+// at the first use of one of its kernels, and the update forms together take
+// 25 ms to load.
 #pragma once
 #include "su3_launch.h"
 #include "su3_site.cuh"

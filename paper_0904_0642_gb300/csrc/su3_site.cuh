@@ -1,6 +1,6 @@
 // su3_site.cuh -- device code of one site: geometry and neighbours, the link
 // update in its forms, re-unitarisation and measurement.  Included by the
-// kernels of one chain (su3_update.cu) and of many (su3_kernels.cu).
+// kernels of one chain (su3_phase.cuh) and of many (su3_tick.cu).
 #pragma once
 #include <type_traits>
 #include <utility>
