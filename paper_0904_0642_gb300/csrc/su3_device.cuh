@@ -377,15 +377,21 @@ __device__ __forceinline__ void acc_su3_2rows_w(M3<R> &A, const M3<R> &m, R w) {
 // and copy (one link between two planes, for halo and box copies).
 
 // COH: loads see what other CTAs of the same launch have written and
-// synchronised (through L2); otherwise they take the read-only path, which is
-// right for links that no CTA of the launch writes.
+// synchronised, and what an earlier launch wrote while this SM held the line
+// (through L2).  Otherwise they are cached in L1, and still ordinary loads:
+// the read-only path (ld.global.nc) would need links that nothing writes for
+// the kernel's whole lifetime, and a programmatic launch is resident, before
+// its wait, while its predecessor writes them.  Ordinary loads are ordered by
+// that wait, and not slower: ten sweeps of 256 chains of 8^4 take 5990 us with
+// them and 6080 with read-only ones, of 32^4 5304 and 5313 (ordinary loads kept
+// in program order, __ldca, cost 6190 in the first).
 
 template <bool COH, class T>
 __device__ __forceinline__ T ld_link(const T *p) {
   if constexpr (COH)
     return __ldcg(p);
   else
-    return __ldg(p);
+    return *p;
 }
 
 template <bool COH>

@@ -171,9 +171,9 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
   bool wrote_partials = false;  // this thread wrote data that the last warp reads
   bool staged = false;  // (MC) stg holds the chain of this CTA's next tile
   for (int t = blockIdx.x; t < total; t += gridDim.x) {
-    const int c = __ldg(ea.tile_chain + t);  // the same for every thread of the CTA
+    const int c = ea.tile_chain[t];  // the same for every thread of the CTA
     int cn = -1;  // (MC) the chain of the CTA's next tile
-    if constexpr (MC) cn = t + (int)gridDim.x < total ? __ldg(ea.tile_chain + t + gridDim.x) : -1;
+    if constexpr (MC) cn = t + (int)gridDim.x < total ? ea.tile_chain[t + gridDim.x] : -1;
     if (c != cur) {
       if (cur >= 0) flush_counters(sd, np, na);
       if constexpr (MC)
