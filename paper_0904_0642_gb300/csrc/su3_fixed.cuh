@@ -170,6 +170,9 @@ SU3_HD int clz64(uint64_t x) {
   return h ? clz32(h) : 32 + clz32((uint32_t)x);
 }
 
+// v 2^-n rounded to nearest (halves up), 0 <= n < 62.
+SU3_HD int64_t shift_round(int64_t v, int n) { return (v + ((1ll << n) >> 1)) >> n; }
+
 // floor(x 2^60) by integer operations, for |x| < 2 (a range check rejects
 // others): the mantissa with its leading bit at bit 63, shifted right by
 // 1026 - e (zero and subnormals shift out), negative values as the ones'
@@ -731,6 +734,9 @@ SU3_HD bool norm_fx(const int64_t a[4], FxNorm &n) {
   for (int q = 0; q < 4; ++q) {
     f[q] = fx_split(a[q] << s);
     fmac(sum, f[q], f[q]);
+    // the product that fmac drops has one sign here: without it the norm is
+    // low by 4 units on average, and the booked action drifts
+    sum.x += ((int64_t)f[q].l * f[q].l) >> 32;
   }
   const Fx n2 = fx_split(fold60(sum));
   n.y = fx_split(rsqrt_fx(n2));

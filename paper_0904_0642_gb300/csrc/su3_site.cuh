@@ -718,7 +718,7 @@ __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, cons
       if (accepted) {
         ++nacc;
         // k x0 - a0 with k = kappa 2^(3 - s)
-        dretr2 += (fx_mul(fx_split(n.kappa), x[0]) >> n.s) - a[0];
+        dretr2 += shift_round(fx_mul(fx_split(n.kappa), x[0]), n.s) - a[0];
         Fx r[4], rn[4];
         quat_fx(x, n.v, r);
 #pragma unroll
@@ -757,8 +757,9 @@ __device__ __noinline__ UpdateCount update_site_f64_general(const ChainDesc *d, 
   return u;
 }
 
-// The change of Re Tr(U A) of one update: in units 2^-49 (sums over a warp are
-// exact), and in double where the double-precision form ran.
+// The change of Re Tr(U A) of one update: rounded to units 2^-51, the last
+// place of a double of its size (at most 36 for SU(3) links; sums over a warp
+// are exact), and in double where the double-precision form ran.
 struct ActionChange {
   int64_t v;
   double general;
@@ -794,7 +795,7 @@ __device__ __forceinline__ void update_site_fixed(const ChainDesc &d, uint32_t s
   const uint32_t before = nacc;
   int64_t half;
   cm_update_fixed(d, U, factor56(A), site_key<SUB>(d, g), sweep, colour, mu, nprop, nacc, half);
-  dr.v = half >> 7;
+  dr.v = shift_round(half, 5);
   // a link none of whose subgroups accepted keeps its bits
   if (nacc != before && in_bounds(js, Vh, kBoundsIndex)) {
     // the rows lie in the order 1, 2, 0 after the last subgroup
@@ -957,7 +958,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
       np += (uint32_t)h;
       if (accepted) {
         ++na;
-        half += (fx_mul(fx_split(n.kappa), x[0]) >> n.s) - pa[0];
+        half += shift_round(fx_mul(fx_split(n.kappa), x[0]), n.s) - pa[0];
         Fx r[4], rn[4];
         quat_fx(x, n.v, r);
 #pragma unroll
@@ -989,7 +990,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
   if (l8 == 0) {
     nprop += np;
     nacc += na;
-    dr.v = half >> 7;
+    dr.v = shift_round(half, 5);
   }
   // after the last swap the rows lie in the order 0, 2, 1
   if (l8 < 3 && na && in_bounds(js, Vh, kBoundsIndex)) {
@@ -1635,7 +1636,7 @@ __device__ __forceinline__ void book_action(const ChainDesc &d, int slot, double
 __device__ __forceinline__ double warp_sum(ActionChange dr) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) dr.v += __shfl_down_sync(0xffffffffu, (long long)dr.v, o);
-  double sum = dbl_of(dr.v, 49);
+  double sum = dbl_of(dr.v, 51);
   if (__any_sync(0xffffffffu, dr.general != 0.0)) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dr.general += __shfl_down_sync(0xffffffffu, dr.general, o);
