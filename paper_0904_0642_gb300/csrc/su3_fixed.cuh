@@ -28,8 +28,16 @@
 //     |x| <= 6 x 2 x 1.0625 x 2^59 = 6.4 2^60 < 2^63;
 //   the staple sum: six matrices, 6 x 1.0625 x 2^60 < 2^63;
 //   the projection (twelve products of a link and the staple sum, the latter
-//     in units 2^-56) folds x into hh after every four:
-//     |x| <= 4 (1.0625 2^59 + 6.4 2^55) + 2^32 < 2^63.
+//     in units 2^-56) folds x into hh after every four.  The rotations of
+//     earlier subgroups mix the link's rows and keep their squares' sum, at
+//     most 18 x 1.0625^2 = 4.51^2, so that the four elements of a fold add up
+//     to 9.02 at most: |x| <= 9.02 2^59 + 4 x 6.4 x 2^55 + 2^32 < 2^63, and
+//     |a| <= 4.51 sqrt(2) 15.7 / 2 = 50 (15.7: the norm of a staple column),
+//     2^62.7 in units 2^-57;
+//   from there on |a| must be below 8 (SU(3) links: at most 6).  norm_fx marks
+//     others: they may have no leading zeros left to shift into, and the change
+//     of Re Tr(U A) / 2 over the three subgroups, 3 (8 + 8) 2^57 < 2^63, needs
+//     the bound too.
 // A site that fails a check (links far from SU(3), infinities, NaN) is updated
 // by the double-precision form instead.
 #pragma once
@@ -713,7 +721,7 @@ struct InvBeta {
 };
 
 // |a| of a projection: a[q] (units 2^-57) = v[q] k with v a unit quaternion.
-// k = kappa 2^(3 - s), kappa and its inverse y in units 2^-60.
+// k = kappa 2^(3 - s), kappa and its inverse y in units 2^-60, s >= 0.
 struct FxNorm {
   Fx v[4];
   Fx y;
@@ -721,13 +729,20 @@ struct FxNorm {
   int s;
 };
 
-// false when a vanishes.
-SU3_HD bool norm_fx(const int64_t a[4], FxNorm &n) {
+// false when a vanishes or has a component of 8 or more; large becomes negative
+// when the norm is 8 or more.  The callers read it once, after the three
+// subgroups: no branch waits for kappa (one that did cost 1 %).  KEEP: only
+// the sign changes, and a count of proposals can carry it (a register of its
+// own costs the one-thread update 1 %, the masks the eight-lane one).
+template <bool KEEP>
+SU3_HD bool norm_fx(const int64_t a[4], FxNorm &n, int32_t &large) {
+  constexpr int32_t kMask = KEEP ? INT32_MIN : -1;
   uint64_t top = 0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) top |= (uint64_t)(a[q] ^ (a[q] >> 63));
-  if (top == 0) return false;
   const int s = clz64(top) - 4;  // the largest |a| to [1/2, 1)
+  large |= s & kMask;
+  if ((uint32_t)s > 59u) return false;  // a = 0: s = 60
   FxAcc sum = {0, kHalf60};
   Fx f[4];
 #pragma unroll
@@ -744,6 +759,7 @@ SU3_HD bool norm_fx(const int64_t a[4], FxNorm &n) {
 #pragma unroll
   for (int q = 0; q < 4; ++q) n.v[q] = fx_split(fx_mul(f[q], n.y));
   n.s = s;
+  if (s == 0) large |= (int32_t)((uint32_t)((uint64_t)n.kappa >> 32) << 3) & kMask;  // kappa < 2: 1 is the sign bit
   return true;
 }
 

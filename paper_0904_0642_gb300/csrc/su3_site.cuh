@@ -673,9 +673,10 @@ __device__ __forceinline__ void swap_rows(Fc (&a)[3], Fc (&b)[3]) {
 // fixed point.  The loop over the subgroups stays a loop (its body once in
 // the instruction cache): the rows of U and the columns of A of the current
 // subgroup are swapped into places 0 and 1.
-// dretr2: the change of Re Tr(U A) / 2 in units 2^-57.
+// dretr2: the change of Re Tr(U A) / 2 in units 2^-57.  nprop negative: a
+// norm out of range (norm_fx), nothing of the update is to be used.
 __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, const FM3 &A, uint32_t c0, uint32_t c1,
-                                                int colour, int mu, uint32_t &nprop, uint32_t &nacc,
+                                                int colour, int mu, int32_t &nprop, uint32_t &nacc,
                                                 int64_t &dretr2) {
   const uint2 key = make_uint2(d.seed_lo, d.seed_hi);
   const InvBeta ib = {d.inv_beta_m, d.inv_beta_e};
@@ -699,7 +700,7 @@ __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, cons
     for (int k = 0; k < 3; ++k) project_k_f(s, u0[k], u1[k], a0[k], a1[k]);
     const int64_t a[4] = {fold60(s[0]), fold60(s[1]), fold60(s[2]), fold60(s[3])};  // 2^-56, and the factor 1/2
     FxNorm n;
-    if (norm_fx(a, n)) {
+    if (norm_fx<true>(a, n, nprop)) {
       Proposal p;
       int h = 0;
       const ProposalStatus st = propose_until(h, hits, key, c0, c1, tag, n, ib, p);
@@ -714,7 +715,7 @@ __device__ __forceinline__ void cm_update_fixed(const ChainDesc &d, FM3 &U, cons
 #pragma unroll
         for (int q = 0; q < 4; ++q) x[q] = fx_of(r.x[q]);
       }
-      nprop += (uint32_t)h;
+      nprop += h;
       if (accepted) {
         ++nacc;
         // k x0 - a0 with k = kappa 2^(3 - s)
@@ -785,19 +786,25 @@ __device__ __forceinline__ void update_site_fixed(const ChainDesc &d, uint32_t s
   S::Vec *pu = plane_ptr<S>(d, layer, colour, mu);
   FM3 U;
   load_f(pu, Vh, js, U, rg);
-  if (!rg.ok()) {
+  int32_t np = -1;
+  uint32_t na = 0;
+  int64_t half;
+  if (rg.ok()) {
+    np = 0;
+    cm_update_fixed(d, U, factor56(A), site_key<SUB>(d, g), sweep, colour, mu, np, na, half);
+  }
+  if (np < 0) {
     const UpdateCount u = update_site_f64_general<SUB, false>(&d, sweep, colour, mu, layer, jj);
     nprop += u.nprop;
     nacc += u.nacc;
     dr.general = u.dretr;
     return;
   }
-  const uint32_t before = nacc;
-  int64_t half;
-  cm_update_fixed(d, U, factor56(A), site_key<SUB>(d, g), sweep, colour, mu, nprop, nacc, half);
+  nprop += (uint32_t)np;
+  nacc += na;
   dr.v = shift_round(half, 5);
   // a link none of whose subgroups accepted keeps its bits
-  if (nacc != before && in_bounds(js, Vh, kBoundsIndex)) {
+  if (na && in_bounds(js, Vh, kBoundsIndex)) {
     // the rows lie in the order 1, 2, 0 after the last subgroup
     double2 v[9];
 #pragma unroll
@@ -914,6 +921,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
 
   uint32_t np = 0, na = 0;
   int64_t half = 0;
+  int32_t large = 0;
 #pragma unroll 1
   for (int sg = 0; sg < 3; ++sg) {
     // the projection: this lane's k, then the sum over the lanes (the rounding
@@ -938,7 +946,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
     dir.cphi = shfl_fx(mine.cphi, base + 3 + sg);
     dir.sphi = shfl_fx(mine.sphi, base + 3 + sg);
     FxNorm n;
-    if (norm_fx(pa, n)) {
+    if (norm_fx<false>(pa, n, large)) {
       const uint32_t tag = heatbath_tag(colour, mu, sg);
       Proposal p;
       int h = 1;
@@ -978,7 +986,7 @@ __device__ __forceinline__ void update_site_coop(const ChainDesc &d, uint32_t sw
     a[1] = fc_sel(keep == 0, ta, a[1]);
   }
   if (!valid) return;
-  if (bad) {
+  if (bad || large < 0) {  // the same in a link's lanes
     if (l8 == 0) {
       const UpdateCount uc = update_site_f64_general<SUB, COH>(&d, sweep, colour, mu, layer, jj);
       nprop += uc.nprop;
