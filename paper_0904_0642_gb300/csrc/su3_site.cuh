@@ -1288,12 +1288,13 @@ static __device__ __noinline__ double plaquette_general(const ChainDesc *d, int 
                               S::load2(plane_ptr<S>(*d, layer, colour, mu), d->Vh, g.s >> 1));
 }
 
-// Sums of plaquettes: integers in units 2^-48 (at most 2^11 plaquettes per
-// sum), and in double those of links out of range.
+// Sums of plaquettes: integers in units 2^-56 (a site's planes: six at most, of
+// magnitude below 7 for links in range), read as one double; and in double
+// those of links out of range.
 struct PlaquetteSum {
   int64_t v = 0;
   double general = 0.0;
-  __device__ __forceinline__ double value() const { return dbl_of(v, 48) + general; }
+  __device__ __forceinline__ double value() const { return dbl_of(v, 56) + general; }
 };
 
 template <bool SUB>
@@ -1301,7 +1302,7 @@ __device__ __forceinline__ void add_plaquette(const ChainDesc &d, const SiteGeo 
                                               PlaquetteSum &s) {
   int64_t tr;
   if (plaquette_fixed<SUB>(d, g, colour, mu, nu, tr))
-    s.v += (tr + (1 << 11)) >> 12;
+    s.v += shift_round(tr, 4);
   else
     s.general += plaquette_general<SUB>(&d, g.layer, colour, jj, mu, nu);
 }
