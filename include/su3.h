@@ -439,7 +439,9 @@ void su3_server_destroy(su3_server *srv);
  *                   would (that job is done with SU3_ENOMEM; the worker
  *                   carries on);
  *   "server_round"  the worker's next round of ticks fails as a failed
- *                   launch would (the worker stops; see su3_server_poll).
+ *                   launch would (the worker stops; see su3_server_poll);
+ *   "programmatic"  the next programmatic launch outside a graph is refused
+ *                   (the handle goes over to ordinary launches).
  * EINVAL for an unknown site or a negative count. */
 su3_status su3_inject_fault(const char *site, int count);
 

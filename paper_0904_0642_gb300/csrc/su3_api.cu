@@ -70,7 +70,7 @@ extern "C" const char *su3_last_error(void) { return g_err.c_str(); }
 
 // ------------------------------------------------------------------ fault injection (host side)
 
-enum FaultSite { kFaultServerAdmit = 0, kFaultServerRound = 1, kFaultSites = 2 };
+enum FaultSite { kFaultServerAdmit = 0, kFaultServerRound = 1, kFaultProgrammatic = 2, kFaultSites = 3 };
 static std::atomic<int> g_fault[kFaultSites];
 
 // True (and one armed pass used up) when the site is armed.
@@ -88,6 +88,8 @@ extern "C" su3_status su3_inject_fault(const char *site, int count) {
     g_fault[kFaultServerAdmit] = count;
   else if (!std::strcmp(site, "server_round"))
     g_fault[kFaultServerRound] = count;
+  else if (!std::strcmp(site, "programmatic"))
+    g_fault[kFaultProgrammatic] = count;
   else
     return fail(SU3_EINVAL, "unknown fault site '%s'", site);
   return SU3_OK;
@@ -1048,16 +1050,25 @@ struct Engine {
     return launch_halo(storage, ch.desc, ch.halo_n[0] + ch.halo_n[1], stream, programmatic);
   }
 
-  su3_status one_tick(int grid) {
-    cudaError_t e = launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, pdl);
-    if (e != cudaSuccess && pdl) {  // not offered here: plain launches from now on
+  // Run launch(), which launches programmatically while `pdl` is set; where
+  // the driver refuses that, ordinary launches from now on.
+  template <class F>
+  su3_status launched(F &&launch) {
+    cudaError_t e = pdl && consume_fault(kFaultProgrammatic) ? cudaErrorNotSupported : launch();
+    if (e != cudaSuccess && pdl) {
       cudaGetLastError();
       pdl = false;
       drop_graph();
-      e = launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, false);
+      e = launch();
     }
     CU(e);
     return SU3_OK;
+  }
+
+  su3_status one_tick(int grid) {
+    return launched([&] {
+      return launch_tick(storage, kernel_variant(), weighted_any, torus_all, args(), grid, block, stream, pdl);
+    });
   }
 
   // Divided chains: undivided layout <-> boxes (to_sub = 1: scatter and
@@ -1226,17 +1237,7 @@ struct Engine {
       return SU3_OK;
     }
     return launch_chunk(c, grid, [&](int kind, auto &&launch) -> su3_status {
-      auto once = [&]() -> su3_status {
-        cudaError_t e = launch();
-        if (e != cudaSuccess && pdl) {  // not offered here: plain launches from now on
-          cudaGetLastError();
-          pdl = false;
-          drop_graph();
-          e = launch();
-        }
-        CU(e);
-        return SU3_OK;
-      };
+      auto once = [&] { return launched(launch); };
       return profiling ? profiled(kind, once) : once();
     });
   }
@@ -1579,8 +1580,7 @@ extern "C" su3_status su3_reunitarize(su3_lattice *lat) {
   LAT_CHECK(lat);
   Engine &e = lat->eng;
   if (e.tiles_dirty) TRY(e.rebuild());
-  CU(e.reunit_all());
-  return SU3_OK;
+  return e.launched([&] { return e.reunit_all(); });
 }
 
 extern "C" su3_status su3_plaquette(su3_lattice *lat, int layer, double *total, double *space, double *time) {
