@@ -284,11 +284,13 @@ su3_status su3_use_graph(su3_lattice *lat, int on);
  * refuses such launches the library falls back to ordinary ones. */
 su3_status su3_use_pdl(su3_lattice *lat, int on);
 
-/* Kernel timing.  With profiling on, su3_sweep launches its ticks one by
- * one (no graph) with a CUDA event pair around each on the handle's stream,
- * and su3_get_profile sums the device time per stage kind: update phases,
- * re-unitarisations, measurements (synchronises; reset = 1 clears).  The
- * results do not change. */
+/* Kernel timing.  With profiling on, su3_sweep launches its stages one by
+ * one (no graph) with a CUDA event pair around each launch on the handle's
+ * stream, and su3_get_profile sums the device time per stage kind: update
+ * phases, re-unitarisations, measurements (synchronises; reset = 1 clears).
+ * update_launches counts phases, 2 D per sweep, also for a chain of at most
+ * 256 links per phase, which runs whole sweeps in a launch: update_ms /
+ * update_launches is the time of a phase.  The results do not change. */
 typedef struct su3_profile {
   double update_ms;
   int64_t update_launches;

@@ -557,7 +557,7 @@ struct Engine {
   bool profiling = false;
   struct EvPair {
     cudaEvent_t a, b;
-    int kind;
+    int kind, phases;
   };
   std::vector<EvPair> prof_pending;
   double prof_ms[3] = {0, 0, 0};
@@ -574,11 +574,12 @@ struct Engine {
   }
 
   // A launch between two events, of kind 0 (update), 1 (re-unitarisation) or
-  // 2 (measurement).
+  // 2 (measurement), that runs `phases` of its kind.
   template <class F>
-  su3_status profiled(int kind, F &&launch) {
+  su3_status profiled(int kind, F &&launch, int phases = 1) {
     EvPair p;
     p.kind = kind;
+    p.phases = phases;
     CU(cudaEventCreate(&p.a));
     CU(cudaEventCreate(&p.b));
     CU(cudaEventRecord(p.a, stream));
@@ -611,7 +612,7 @@ struct Engine {
       float ms = 0;
       CU(cudaEventElapsedTime(&ms, p.a, p.b));
       prof_ms[p.kind] += ms;
-      prof_n[p.kind] += 1;
+      prof_n[p.kind] += p.phases;
     }
     drop_events();
     if (out) {
@@ -1176,11 +1177,12 @@ struct Engine {
     return e;
   }
 
-  // The launches of a chunk; each(kind, launch) runs one.
+  // The launches of a chunk; each(kind, launch, phases) runs one.
   template <class F>
   su3_status launch_chunk(const Chunk &c, int grid, F &&each) {
     const ChainDesc &d = chains[0].desc;
-    if (cluster) TRY(each(0, [&] { return launch_sweeps(storage, sub_any, d, d_ctl, c.m, stream, pdl); }));
+    if (cluster)
+      TRY(each(0, [&] { return launch_sweeps(storage, sub_any, d, d_ctl, c.m, stream, pdl); }, 2 * d.D * c.m));
     for (int i = 0; i < (cluster ? 0 : c.m); ++i)
       for (int st = 0; st < 2 * d.D; ++st) {
         UpdateStep u{};
@@ -1207,7 +1209,7 @@ struct Engine {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal), le = cudaSuccess;
     if (e != cudaSuccess) return e;
-    launch_chunk(c, grid, [&](int, auto &&launch) -> su3_status {
+    launch_chunk(c, grid, [&](int, auto &&launch, int = 1) -> su3_status {
       if (le == cudaSuccess) le = launch();
       return SU3_OK;
     });
@@ -1236,9 +1238,9 @@ struct Engine {
       CU(cudaGraphLaunch(g, stream));
       return SU3_OK;
     }
-    return launch_chunk(c, grid, [&](int kind, auto &&launch) -> su3_status {
+    return launch_chunk(c, grid, [&](int kind, auto &&launch, int phases = 1) -> su3_status {
       auto once = [&] { return launched(launch); };
-      return profiling ? profiled(kind, once) : once();
+      return profiling ? profiled(kind, once, phases) : once();
     });
   }
 
