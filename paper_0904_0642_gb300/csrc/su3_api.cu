@@ -1862,18 +1862,23 @@ static su3_status autotune_engine(Engine &e, int *variant, int *threads, int *ct
   int best_v = saved_var, best_t = saved_block, best_c = std::max(saved_ctas, 0);
   const int cand_t[] = {64, 128, 256};
   su3_status st = SU3_OK;
-  const int nvar = e.sub_any ? 1 : tick_variants(e.storage);  // a divided chain has one kernel form
+  // a divided chain, eight lanes per link and the early form have one kernel
+  // whatever the variant; whole sweeps per launch also have one shape
+  const bool one_kernel = e.sub_any || e.coop || e.early, one_shape = e.fixed && e.cluster;
+  const int nvar = one_kernel ? 1 : tick_variants(e.storage);
   for (int v = 0; v < nvar && st == SU3_OK; ++v)
     for (int t : cand_t) {
-      if (t > tick_max_threads(e.storage, v)) continue;
+      if (t > tick_max_threads(e.storage, v) || (one_shape && t != 128)) continue;
       int occ = 0;
       const int kv = e.coop || e.early ? e.kernel_variant() : v;
       const cudaError_t oe = e.fixed ? update_occupancy(e.storage, kv, e.weighted_any, e.sub_any, e.torus_all, t, &occ)
                                      : tick_occupancy(e.storage, kv, e.weighted_any, e.torus_all, t, &occ);
       if (oe != cudaSuccess || occ < 1) continue;
       // 0 = one CTA per tile, then persistent grids of 1, 2, 4, ..., occ CTAs per SM
+      if (one_shape) occ = 0;
       for (int c = 0; c <= occ && st == SU3_OK; c = (c == 0) ? 1 : ((c < occ && 2 * c > occ) ? occ : 2 * c)) {
-        if ((st = e.set_launch(v, t, c)) != SU3_OK) break;
+        if ((st = e.set_launch(v, t, c)) != SU3_OK || (st = e.rebuild()) != SU3_OK) break;
+        if (v > 0 && e.parked) continue;  // the same kernel as with variant 0
         // every candidate starts from the same links: without re-unitarisation
         // FP32 links leave SU(3) within ~60 sweeps and the timings with them
         for (size_t k = 0; k < e.chains.size(); ++k)
