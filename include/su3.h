@@ -442,6 +442,8 @@ void su3_server_destroy(su3_server *srv);
  *                   carries on);
  *   "server_round"  the worker's next round of ticks fails as a failed
  *                   launch would (the worker stops; see su3_server_poll);
+ *   "server_pool"   a new server's memory pool cannot be made (its jobs'
+ *                   memory comes from plain allocations);
  *   "programmatic"  the next programmatic launch outside a graph is refused
  *                   (the handle goes over to ordinary launches).
  * EINVAL for an unknown site or a negative count. */

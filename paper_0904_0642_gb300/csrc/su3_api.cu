@@ -70,7 +70,7 @@ extern "C" const char *su3_last_error(void) { return g_err.c_str(); }
 
 // ------------------------------------------------------------------ fault injection (host side)
 
-enum FaultSite { kFaultServerAdmit = 0, kFaultServerRound = 1, kFaultProgrammatic = 2, kFaultSites = 3 };
+enum FaultSite { kFaultServerAdmit = 0, kFaultServerRound = 1, kFaultProgrammatic = 2, kFaultServerPool = 3, kFaultSites = 4 };
 static std::atomic<int> g_fault[kFaultSites];
 
 // True (and one armed pass used up) when the site is armed.
@@ -90,6 +90,8 @@ extern "C" su3_status su3_inject_fault(const char *site, int count) {
     g_fault[kFaultServerRound] = count;
   else if (!std::strcmp(site, "programmatic"))
     g_fault[kFaultProgrammatic] = count;
+  else if (!std::strcmp(site, "server_pool"))
+    g_fault[kFaultServerPool] = count;
   else
     return fail(SU3_EINVAL, "unknown fault site '%s'", site);
   return SU3_OK;
@@ -681,21 +683,33 @@ struct Engine {
 
   // A server's chains come and go: their memory comes from a pool of its own
   // (allocations and frees in stream order, no device-wide waits), which
-  // keeps at most `kPoolKept` bytes and is destroyed with the server.
+  // keeps at most `kPoolKept` bytes and is destroyed with the server.  Where
+  // no pool can be made it comes from plain allocations.
   cudaMemPool_t pool = nullptr;
+  bool pool_tried = false;
   static constexpr uint64_t kPoolKept = 1ull << 30;
 
-  su3_status make_pool(size_t most) {
+  void make_pool(size_t most) {
+    if (pool_tried) return;
+    pool_tried = true;
     int dev = 0;
-    CU(cudaGetDevice(&dev));
-    cudaMemPoolProps props = {};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = dev;
-    CU(cudaMemPoolCreate(&pool, &props));
-    uint64_t keep = std::min<uint64_t>(kPoolKept, most);
-    CU(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
-    return SU3_OK;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) {
+      cudaMemPoolProps props = {};
+      props.allocType = cudaMemAllocationTypePinned;
+      props.location.type = cudaMemLocationTypeDevice;
+      props.location.id = dev;
+      e = consume_fault(kFaultServerPool) ? cudaErrorNotSupported : cudaMemPoolCreate(&pool, &props);
+    }
+    if (e == cudaSuccess) {
+      uint64_t keep = std::min<uint64_t>(kPoolKept, most);
+      e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+      if (e != cudaSuccess) cudaMemPoolDestroy(pool);
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      pool = nullptr;
+    }
   }
 
   template <class T>
@@ -2287,10 +2301,7 @@ void su3_server::loop() {
     // Bring admitted jobs on the device (outside the lock).
     bool changed = false;
     std::vector<std::pair<uint64_t, const double *>> starts;  // jobs with a given start configuration
-    if (!admitted.empty() && !eng.pool && eng.make_pool(budget) != SU3_OK) {
-      die(g_err);
-      break;
-    }
+    if (!admitted.empty()) eng.make_pool(budget);
     for (auto &j : admitted) {
       Chain ch;
       su3_config c = j.job.cfg;

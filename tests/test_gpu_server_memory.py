@@ -1,0 +1,38 @@
+"""The job server's device memory."""
+import numpy as np
+import pytest
+
+import paper_0904_0642_gb300 as su3
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture
+def disarm():
+    yield
+    su3.su3_inject_fault("server_pool", 0)
+
+
+def config(dims, seed=3, **kw):
+    return su3.make_config(dims, beta=5.7, seed=seed, storage=su3.SU3_FP32_12, start=su3.SU3_START_HOT, hits=2,
+                           reunit_every=10, **kw)
+
+
+def test_jobs_run_without_a_pool(disarm):
+    """Where no memory pool can be made the jobs' memory comes from plain
+    allocations, and links go in and out as ever."""
+    dims, links = [8, 8, 8, 4], []
+    su3.su3_inject_fault("server_pool", 1)
+    srv = su3.Server(max_slots=2)
+    for n in (5, 7):  # the second job starts from the first one's links
+        out = np.zeros((1, 8 * 8 * 8 * 4, 4, 3, 3, 2))
+        job = srv.submit(config(dims), n, links_in=links[-1] if links else None, links_out=out)
+        assert srv.wait(job, timeout_s=60).status == su3.SU3_OK
+        links.append(out)
+    srv.close()
+    with su3.Lattice(dims, beta=5.7, seed=3, storage=su3.SU3_FP32_12, start=su3.SU3_START_HOT, hits=2,
+                     reunit_every=10) as lat:
+        for n, out in zip((5, 7), links):
+            lat.set_sweep_counter(0)
+            lat.sweep(n)
+            assert np.array_equal(lat.get_links(), out)
