@@ -409,7 +409,10 @@ typedef struct su3_result {
  * The worker thread runs the resident chains in rounds of 16 fused ticks
  * (one captured graph) and reads their stage machines back after each
  * round (one host synchronisation per round): admission and retirement
- * happen between rounds, which sets the granularity of job latency. */
+ * happen between rounds, which sets the granularity of job latency.
+ * The memory of retired jobs is kept for the next ones, 1 GiB (or the budget,
+ * if smaller) at most, and 32 MiB once the server has been idle for five
+ * seconds. */
 su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, su3_server **out);
 /* Queue a job; never blocks.  EINVAL for a bad job, ENOMEM when the job
  * alone exceeds the budget, ECUDA (with the worker's message) once the

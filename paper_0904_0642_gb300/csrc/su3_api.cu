@@ -683,11 +683,13 @@ struct Engine {
 
   // A server's chains come and go: their memory comes from a pool of its own
   // (allocations and frees in stream order, no device-wide waits), which
-  // keeps at most `kPoolKept` bytes and is destroyed with the server.  Where
-  // no pool can be made it comes from plain allocations.
+  // keeps at most `kPoolKept` bytes between jobs, kPoolIdle once the server has
+  // been idle for kIdleSeconds (the next job does not notice: 32^4, 20 sweeps,
+  // 16.5 ms after seven idle seconds with and without), and is destroyed with
+  // the server.  Where no pool can be made it comes from plain allocations.
   cudaMemPool_t pool = nullptr;
   bool pool_tried = false;
-  static constexpr uint64_t kPoolKept = 1ull << 30;
+  static constexpr uint64_t kPoolKept = 1ull << 30, kPoolIdle = 32ull << 20;
 
   void make_pool(size_t most) {
     if (pool_tried) return;
@@ -712,6 +714,12 @@ struct Engine {
     }
   }
 
+  // Give back what the pool keeps beside the chains' memory, down to `keep`.
+  void trim_pool(uint64_t keep) {
+    cudaStreamSynchronize(stream);
+    cudaMemPoolTrimTo(pool, keep);
+  }
+
   template <class T>
   cudaError_t chain_alloc(T **p, size_t bytes) {
     void *v = nullptr;
@@ -722,8 +730,7 @@ struct Engine {
       e = cudaMallocFromPoolAsync(&v, bytes, pool, stream);
       if (e == cudaErrorMemoryAllocation) {  // what the pool keeps in pieces may be enough in one
         cudaGetLastError();
-        cudaStreamSynchronize(stream);
-        cudaMemPoolTrimTo(pool, 0);
+        trim_pool(0);
         e = cudaMallocFromPoolAsync(&v, bytes, pool, stream);
       }
     }
@@ -2111,6 +2118,7 @@ struct su3_server {
   cudaEvent_t round_ev[2] = {nullptr, nullptr};  // around each round of ticks
   uint64_t rounds = 0;       // rounds run (under mu)
   double device_ms = 0.0;    // their device time (under mu)
+  static constexpr int kIdleSeconds = 5;
   bool dead = false;         // the worker stopped after an error (under mu)
   std::string worker_error;  // its message (under mu)
   std::map<uint64_t, double *> links_out;  // jobs whose final links go to a host buffer
@@ -2294,7 +2302,19 @@ void su3_server::loop() {
     std::vector<ServerJob> admitted;
     {
       std::unique_lock<std::mutex> lk(mu);
-      while (!stop && queue.empty() && eng.chains.empty()) cv.wait(lk);
+      bool kept = eng.pool != nullptr;  // the pool may hold memory
+      while (!stop && queue.empty() && eng.chains.empty()) {
+        if (!kept) {
+          cv.wait(lk);
+          continue;
+        }
+        kept = cv.wait_for(lk, std::chrono::seconds(kIdleSeconds)) != std::cv_status::timeout;
+        if (!kept && !stop && queue.empty()) {
+          lk.unlock();
+          eng.trim_pool(Engine::kPoolIdle);
+          lk.lock();
+        }
+      }
       if (stop) break;
       admit_locked(admitted);
     }

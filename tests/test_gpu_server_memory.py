@@ -1,6 +1,9 @@
 """The job server's device memory."""
+import time
+
 import numpy as np
 import pytest
+import torch
 
 import paper_0904_0642_gb300 as su3
 
@@ -36,3 +39,22 @@ def test_jobs_run_without_a_pool(disarm):
             lat.set_sweep_counter(0)
             lat.sweep(n)
             assert np.array_equal(lat.get_links(), out)
+
+
+def test_idle_server_gives_its_memory_back():
+    """A 32^4 job holds 201 MB of links; a server that has been idle for a
+    while keeps 32 MiB at most."""
+    dims = [32, 32, 32, 32]
+    size = su3.su3_link_bytes(config(dims))
+    srv = su3.Server(max_slots=2)
+    # what the first job brings once: the context, modules, the worker's buffers
+    assert srv.wait(srv.submit(config([4, 4, 4, 4]), 1), timeout_s=60).status == su3.SU3_OK
+    before = torch.cuda.mem_get_info()[0]
+    assert srv.wait(srv.submit(config(dims), 1), timeout_s=60).status == su3.SU3_OK
+    deadline = time.time() + 10
+    while torch.cuda.mem_get_info()[0] < before - size // 4 and time.time() < deadline:
+        time.sleep(0.05)
+    assert torch.cuda.mem_get_info()[0] >= before - size // 4
+    # and takes jobs as before
+    assert srv.wait(srv.submit(config(dims), 1), timeout_s=60).status == su3.SU3_OK
+    srv.close()
