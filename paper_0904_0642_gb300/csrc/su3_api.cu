@@ -541,6 +541,7 @@ struct Engine {
   int32_t *d_meas_list = nullptr;  // [chain_cap] the chains a launch measures
   size_t tile_cap = 0, chain_cap = 0;
   double *d_meas_out = nullptr;  // stand-alone measurement results
+  double *d_partials = nullptr;  // and partial sums (measure_into)
   double *h_pinned = nullptr;    // small pinned staging (results, counters)
   int block = 128;
   int ctas_per_sm = kAutoCtas;
@@ -663,6 +664,8 @@ struct Engine {
     cudaFree(d_tile_chain);
     cudaFree(d_meas_list);
     cudaFree(d_meas_out);
+    cudaFree(d_partials);
+    d_partials = nullptr;
     cudaFreeHost(h_pinned);
     d_desc = nullptr;
     d_state = nullptr;
@@ -821,7 +824,7 @@ struct Engine {
       ch.bytes_total += ch.link_bytes;
     }
     // partials and action slots sized for the narrowest tile
-    const bool few = phase_links(ch) <= (storage == SU3_FP64_18 ? kCoopSites : kLanesLinks);
+    const bool few = storage == SU3_FP64_18 ? phase_links(ch) <= kCoopSites : fixed && phase_links(ch) <= kLanesLinks;
     const int narrow = few ? 32 / kCoopLanes : 32;
     fill_desc(ch, narrow);
     size_t ntiles = (size_t)ch.desc.nlayers * ch.desc.tiles_per_layer;
@@ -829,7 +832,7 @@ struct Engine {
       fill_plain(ch, narrow);
       ntiles = std::max(ntiles, (size_t)ch.pdesc.nlayers * ch.pdesc.tiles_per_layer);
     }
-    const size_t npart = std::max(ntiles, (size_t)ch.desc.nlayers * kMeasureCtas) * kPartVals;
+    const size_t npart = (fixed ? std::max(ntiles, (size_t)ch.desc.nlayers * kMeasureCtas) : ntiles) * kPartVals;
     const size_t nres = (size_t)ch.desc.result_cap * (ch.desc.nlayers + 1) * kMeasVals;
     // one block of scratch: what starts at zero (counters, booked changes,
     // reference, results) first, then the partial sums
@@ -1332,10 +1335,19 @@ struct Engine {
 
   // Measure a chain's links (divided: gathered into the undivided layout)
   // into device memory, queued.
+  // Engines of many chains measure one chain at a time with one set of partial
+  // sums; a chain's own are those of its tiles in the fused launch.
   su3_status measure_into(size_t c, double *device_out) {
     const ChainDesc *d = nullptr;
     TRY(io_desc(c, &d));
-    CU(launch_measure(storage, false, *d, device_out, d_ctl, stream, false));
+    if (fixed) {
+      CU(launch_measure(storage, false, *d, device_out, d_ctl, stream, false));
+      return SU3_OK;
+    }
+    if (!d_partials) CU(cudaMalloc(&d_partials, 2 * kMeasureCtas * kPartVals * sizeof(double)));
+    ChainDesc md = *d;
+    md.partials = d_partials;
+    CU(launch_measure(storage, false, md, device_out, d_ctl, stream, false));
     return SU3_OK;
   }
 
@@ -2135,14 +2147,15 @@ struct su3_server {
 };
 
 static size_t job_bytes(const su3_config &c) {
-  // links + measurement scratch (partials for 32-wide tiles, result ring, counters)
+  // links + measurement scratch (partials for 32-wide tiles, result ring,
+  // counters); the further counter slots (496 bytes) are not charged, so that
+  // a budget that fits a job exactly keeps doing so
   size_t V = 1;
   for (int i = 0; i < c.D; ++i) V *= (size_t)c.dims[i];
   const size_t layers = c.boundary == SU3_DLT ? 2 : 1;
   const size_t tiles = layers * ((V / 2 + 31) / 32);
   const size_t cap = c.measure_capacity > 0 ? (size_t)c.measure_capacity : 1024;
-  return link_bytes_of(&c) + std::max(tiles, layers * kMeasureCtas) * kPartVals * 8 + cap * (layers + 1) * kMeasVals * 8 +
-         kCounterBytes + tiles * 8;
+  return link_bytes_of(&c) + tiles * kPartVals * 8 + cap * (layers + 1) * kMeasVals * 8 + 16 + tiles * 8;
 }
 
 extern "C" su3_status su3_server_create(size_t hbm_budget_bytes, int max_slots, su3_server **out) {

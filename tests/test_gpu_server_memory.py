@@ -58,3 +58,21 @@ def test_idle_server_gives_its_memory_back():
     # and takes jobs as before
     assert srv.wait(srv.submit(config(dims), 1), timeout_s=60).status == su3.SU3_OK
     srv.close()
+
+
+@pytest.mark.parametrize("dims,layers", [([4, 4, 4, 4], 1), ([8, 8, 8, 4], 2), ([24, 24, 24], 1)], ids=str)
+def test_budget_of_one_job(dims, layers):
+    """A job needs its links, 32 bytes of partial sums and 8 of booked action
+    per 32 sites of a colour, its ring of measurements and two counters: a
+    budget of that takes it, one byte less does not."""
+    cfg = config(dims, boundary=su3.SU3_DLT if layers == 2 else su3.SU3_PBC, measure_every=2, measure_capacity=16)
+    tiles = layers * -(-int(np.prod(dims)) // 64)
+    need = su3.su3_link_bytes(cfg) + tiles * 40 + 16 * (layers + 1) * 40 + 16
+    srv = su3.Server(hbm_budget_bytes=need, max_slots=2)
+    assert srv.wait(srv.submit(cfg, 4), timeout_s=60).status == su3.SU3_OK
+    srv.close()
+    srv = su3.Server(hbm_budget_bytes=need - 1, max_slots=2)
+    with pytest.raises(su3.Su3Error) as ei:
+        srv.submit(cfg, 4)
+    assert ei.value.status == su3.SU3_ENOMEM
+    srv.close()
