@@ -553,8 +553,32 @@ struct Engine {
   bool pdl = true;
   cudaGraphExec_t graph = nullptr;
   int graph_ticks = 0;
-  // fixed schedule: one graph per kind of chunk (chunk_kind)
-  cudaGraphExec_t chunk_graph[4 * (kMaxChunk + 1)] = {};
+  // Fixed schedule: one graph per kind of chunk (Chunk::kind).  The captured
+  // launches carry the descriptor, and with it the hits of su3_sweep: a set of
+  // graphs for each of the last few, so that a caller may alternate.
+  struct ChunkGraphs {
+    int hits;
+    cudaGraphExec_t of_kind[4 * (kMaxChunk + 1)];
+  };
+  static constexpr size_t kGraphSets = 4;
+  std::vector<ChunkGraphs> chunk_graphs;  // the last used first
+
+  ChunkGraphs &graphs_of(int hits) {
+    auto at = std::find_if(chunk_graphs.begin(), chunk_graphs.end(), [&](const ChunkGraphs &g) { return g.hits == hits; });
+    if (at == chunk_graphs.end()) {
+      if (chunk_graphs.size() == kGraphSets) {
+        drop(chunk_graphs.back());
+        chunk_graphs.pop_back();
+      }
+      at = chunk_graphs.insert(chunk_graphs.end(), ChunkGraphs{hits, {}});
+    }
+    std::rotate(chunk_graphs.begin(), at, at + 1);
+    return chunk_graphs.front();
+  }
+  static void drop(ChunkGraphs &set) {
+    for (auto &g : set.of_kind)
+      if (g) cudaGraphExecDestroy(g);
+  }
   bool tiles_dirty = true;
   // kernel timing (su3_set_profiling)
   bool profiling = false;
@@ -1025,10 +1049,8 @@ struct Engine {
     if (graph) cudaGraphExecDestroy(graph);
     graph = nullptr;
     graph_ticks = 0;
-    for (auto &g : chunk_graph) {
-      if (g) cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
+    for (auto &set : chunk_graphs) drop(set);
+    chunk_graphs.clear();
   }
 
   // ctas_per_sm = 0: one CTA per tile (the hardware balances the tail);
@@ -1249,7 +1271,7 @@ struct Engine {
     int grid = 0;
     TRY(grid_size(&grid));
     if (use_graph && !profiling && !cluster) {
-      cudaGraphExec_t &g = chunk_graph[c.kind()];
+      cudaGraphExec_t &g = graphs_of(chains[0].desc.hits).of_kind[c.kind()];
       if (!g) {
         cudaError_t e = capture_chunk(c, grid, &g);
         if (e != cudaSuccess && pdl) {  // programmatic edges not capturable here: plain ones
@@ -1606,7 +1628,6 @@ extern "C" su3_status su3_sweep(su3_lattice *lat, int n, int hits) {
     ch.cfg.hits = hits;
     ch.desc.hits = hits;
     TRY(lat->eng.upload_desc(0));
-    lat->eng.drop_graph();  // the captured launches carry the descriptor
   }
   return lat->eng.sweep_all(n);
 }
