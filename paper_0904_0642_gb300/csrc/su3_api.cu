@@ -1270,7 +1270,10 @@ struct Engine {
   su3_status run_chunk(const Chunk &c) {
     int grid = 0;
     TRY(grid_size(&grid));
-    if (use_graph && !profiling && !cluster) {
+    // a caller who captures the stream gets the launches themselves
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(stream, &capture));
+    if (use_graph && !profiling && !cluster && capture == cudaStreamCaptureStatusNone) {
       cudaGraphExec_t &g = graphs_of(chains[0].desc.hits).of_kind[c.kind()];
       if (!g) {
         cudaError_t e = capture_chunk(c, grid, &g);
