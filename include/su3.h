@@ -472,7 +472,8 @@ su3_status su3_bounds_selftest(void);
 
 /* Thread-local message of the last error (empty string if none). */
 const char *su3_last_error(void);
-/* Library version string. */
+/* Library version string: version, architecture, and a hash of the sources
+ * and flags it was built from. */
 const char *su3_version(void);
 
 #ifdef __cplusplus

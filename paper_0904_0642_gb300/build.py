@@ -1,6 +1,7 @@
 """Build libsu3gb300.so in-tree with nvcc for sm_103a (no cmake)."""
 from __future__ import annotations
 
+import hashlib
 import os
 import subprocess
 import sys
@@ -31,6 +32,16 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def build_id(csrc: str = CSRC, header: str = os.path.join(HERE, "..", "include", "su3.h")) -> str:
+    """What the kernels are compiled from: a hash of the sources, headers and
+    flags, part of su3_version()."""
+    h = hashlib.sha256(repr((ARCH, FLAGS)).encode())
+    for path in sorted(os.path.join(csrc, f) for f in os.listdir(csrc) if f.endswith((".cu", ".cuh", ".h"))) + [header]:
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + b"\0" + f.read())
+    return h.hexdigest()[:12]
+
+
 def build(force: bool = False, verbose: bool = False, debug: bool = True) -> str:
     """Compile the release library and (debug=True) the debug-bounds library,
     all translation units in parallel; returns the release library's path."""
@@ -38,16 +49,23 @@ def build(force: bool = False, verbose: bool = False, debug: bool = True) -> str
     headers.append(os.path.join(HERE, "..", "include", "su3.h"))
     targets = [(BUILD, LIB, [])] + ([(BUILD_DBG, LIB_DBG, ["-DSU3_DEBUG_BOUNDS"])] if debug else [])
     jobs, links = [], []
+    ident = build_id()
     for bdir, lib, extra in targets:
         os.makedirs(bdir, exist_ok=True)
+        id_file = os.path.join(bdir, "build_id")  # su3_api.cu is compiled again when it changes
+        if not os.path.exists(id_file) or open(id_file).read() != ident:
+            with open(id_file, "w") as f:
+                f.write(ident)
         objs = []
         compiled = False
         for src in SOURCES:
             s = os.path.join(CSRC, src)
             o = os.path.join(bdir, src.replace(".cu", ".o"))
             objs.append(o)
-            if force or _stale(o, [s] + headers):
-                jobs.append([_nvcc(), *ARCH, *FLAGS, *extra, "-c", s, "-o", o])
+            api = src == "su3_api.cu"
+            if force or _stale(o, [s] + headers + ([id_file] if api else [])):
+                ident_flag = [f'-DSU3_BUILD_ID="{ident}"'] if api else []
+                jobs.append([_nvcc(), *ARCH, *FLAGS, *extra, *ident_flag, "-c", s, "-o", o])
                 compiled = True
         links.append((lib, objs, compiled))
 

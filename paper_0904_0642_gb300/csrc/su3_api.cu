@@ -96,8 +96,12 @@ extern "C" su3_status su3_inject_fault(const char *site, int count) {
     return fail(SU3_EINVAL, "unknown fault site '%s'", site);
   return SU3_OK;
 }
+#ifndef SU3_BUILD_ID  // given by build.py: a hash of what the library is compiled from
+#define SU3_BUILD_ID "unknown"
+#endif
 extern "C" const char *su3_version(void) {
-  return debug_bounds_build() ? "su3gb300 1.0 (sm_103a, debug bounds)" : "su3gb300 1.0 (sm_103a)";
+  return debug_bounds_build() ? "su3gb300 1.0 (sm_103a, debug bounds, build " SU3_BUILD_ID ")"
+                              : "su3gb300 1.0 (sm_103a, build " SU3_BUILD_ID ")";
 }
 
 // ------------------------------------------------------------------ debug bounds checks

@@ -6,8 +6,9 @@ shape again takes the stored shape instead of timing every candidate.  The
 key holds what the timings depend on: storage form, D and extents,
 boundary and glued directions, sublattice cut, whether two couplings are in
 use, the number of chains of a fused launch, and the library's version
-string (which names the GPU architecture it was built for).  Plain host
-code: it reads and writes the file and nothing else.
+string (which names the GPU architecture it was built for and the sources it
+was built from: other kernels, other timings).  Plain host code: it reads and
+writes the file and nothing else.
 """
 from __future__ import annotations
 
