@@ -63,3 +63,52 @@ def test_scaled_links(dims, ndiv, scale):
         got = first_phase(lat.get_links(), dims)
     assert np.abs(want - first_phase(start, dims)).max() > 0.1  # the update did move them
     assert np.max(np.abs(got - want)) <= 1e-11
+
+
+def bad_link_case(dims, seed):
+    """A bad link in each place of a first-phase update: the link itself
+    (direction 0, colour 0), a staple's parallel link (direction 0, colour 1)
+    and its side links (direction 1, either colour)."""
+    V = int(np.prod(dims))
+    x = np.indices(dims[::-1]).reshape(len(dims), -1)[::-1].T  # x[site] = coordinates, x^1 fastest
+    colour = x.sum(axis=1) % 2
+    site = lambda c: int(np.ravel_multi_index(tuple(int(k) % n for k, n in zip(c, dims))[::-1], dims[::-1]))
+    rng = np.random.default_rng(seed)
+    e = np.eye(len(dims), dtype=int)
+    for mu, col in ((0, 0), (0, 1), (1, 0), (1, 1)):
+        y = x[rng.choice(np.flatnonzero(colour == col))]
+        if mu == 0:  # U_0(y), and the links whose staples hold it: y +- nu
+            near = [y] if col == 0 else [y + s * e[nu] for nu in range(1, len(dims)) for s in (1, -1)]
+        else:        # U_1(y) stands beside U_0 at y, y + 1, y - 0 and y - 0 + 1
+            near = [y, y + e[1], y - e[0], y - e[0] + e[1]]
+        near = sorted({site(c) for c in near if sum(c) % 2 == 0})
+        yield site(y), mu, near, V
+
+
+@pytest.mark.parametrize("dims,ndiv", SHAPES, ids=str)
+@pytest.mark.parametrize("bad", [1.5, -1.2, 40.0])
+def test_sites_of_one_bad_link(dims, ndiv, bad):
+    """One element out of range: of the links of the first phase those that the
+    bad link enters are the double form's bits, all others are the bits they
+    have without it."""
+    kw = dict(beta=5.7, hits=2, seed=9)
+    with su3.Lattice(dims, start=su3.SU3_START_HOT, **kw) as lat:
+        lat.reunitarize()
+        good = lat.get_links()
+
+    def swept(links):
+        with su3.Lattice(dims, ndiv=ndiv, **kw) as lat:
+            lat.set_links(links)
+            lat.sweep(1)
+            return lat.get_links()[0, :, 0]
+
+    without = swept(good)
+    first = np.flatnonzero(np.indices(dims[::-1]).sum(axis=0).reshape(-1) % 2 == 0)
+    for y, mu, near, V in bad_link_case(dims, 4):
+        links = good.copy()
+        links[0, y, mu, 1, 2, 0] = bad
+        got, double = swept(links), double_form(dims, links, **kw)[0, :, 0]
+        assert np.array_equal(got[near], double[near]), (mu, y)
+        far = np.setdiff1d(first, near)
+        assert np.array_equal(got[far], without[far]), (mu, y)
+        assert not np.array_equal(double[far], without[far])  # the two forms do differ in their last bits
