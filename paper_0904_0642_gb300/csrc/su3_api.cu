@@ -883,7 +883,6 @@ struct Engine {
     if (ch.sub) fill_plain(ch, block);
     ch.state = ChainState{};
     ch.state.active = 0;
-    ch.state.prev_stage = -1;
     out = ch;
     return SU3_OK;
   }

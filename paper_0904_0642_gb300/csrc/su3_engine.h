@@ -164,9 +164,8 @@ struct ChainState {
   uint32_t target;         // the chain goes idle at the start of this sweep
   int32_t active;          // 1: advancing; 0: idle
   uint32_t n_meas;         // measurements recorded
-  int32_t prev_stage;      // stage run by the last tick (-1: none); read by the halo refresh
   int32_t anchor;          // 1: the next measurement restarts the action bookkeeping
-  int32_t pad;
+  int32_t pad[2];
 };
 
 // The device side of a one-chain engine's fixed schedule.  The sweep counter

@@ -85,7 +85,6 @@ struct StageParams {
 };
 
 __device__ __host__ inline void advance_stage(const StageParams &d, ChainState &s) {
-  s.prev_stage = s.stage;
   if (s.stage < 2 * d.D) {
     s.stage += 1;
     if (s.stage == 2 * d.D) {
@@ -109,10 +108,7 @@ __device__ __host__ inline void advance_stage(const ChainDesc &d, ChainState &s)
 
 // The state of a chain after this launch's tick.
 __device__ __forceinline__ ChainState next_state(const StageParams &p, ChainState s) {
-  if (!s.active) {
-    s.prev_stage = -1;  // nothing ran: no halo refresh
-    return s;
-  }
+  if (!s.active) return s;
   if (s.stage == kStageMeasure) {
     s.n_meas += 1;
     s.anchor = 0;  // the measurement restarts the bookkeeping if it was set
