@@ -211,41 +211,24 @@ def cpu_baseline():
     return out
 
 
-def graph_stage_times(su3, torch, stream, seed, step_ms):
-    """Per-stage device times of the 32^4 step, all from CUDA-graph-timed
-    runs (CUDA events on the lattice's stream), so that they add up to the
-    timed step: a lattice re-unitarised every 10 sweeps runs 80 update ticks
-    + 1 re-unitarisation per 10-sweep call (T10), one re-unitarised every 20
-    sweeps 160 + 1 per 20-sweep call (T20); neither measures.  Then
-    update tick = (T20 - T10) / 80, re-unitarisation = T10 - 80 x tick (it
-    carries the call's one-block arm kernel), measurement = step - T10.
-    T10 and T20 are each the fastest of three alternating timings: a single
-    pair moved the derived tick by ~1 us between runs."""
-    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-    lats = {}
-    for every in (10, 20):
-        lats[every] = su3.Lattice(DIMS, beta=BETA, seed=seed, hits=HITS, storage=su3.SU3_FP32_12,
-                                  start=su3.SU3_START_HOT, reunit_every=every, stream=stream)
-        lats[every].autotune()
-        lats[every].sweep(every)
-    per_call = {10: float("inf"), 20: float("inf")}
-    for _ in range(3):
-        for every, calls in ((10, 12), (20, 6)):
-            torch.cuda.synchronize()
-            e0.record(stream)
-            for _ in range(calls):
-                lats[every].sweep(every)
-            e1.record(stream)
-            torch.cuda.synchronize()
-            per_call[every] = min(per_call[every], e0.elapsed_time(e1) / calls)
-    for lat in lats.values():
-        lat.close()
-    ticks = 2 * len(DIMS) * SWEEPS_PER_STEP
-    tick_ms = (per_call[20] - per_call[10]) / ticks
-    reunit_ms = per_call[10] - ticks * tick_ms
-    return {"update_tick_us": 1e3 * tick_ms, "reunit_us": 1e3 * reunit_ms,
-            "measure_us": 1e3 * (step_ms - per_call[10]), "T10_ms": per_call[10], "T20_ms": per_call[20],
-            "sum_ms": ticks * tick_ms + reunit_ms + (step_ms - per_call[10]), "step_ms": step_ms}
+def stage_times(lat, step_ms, steps=5):
+    """Per-stage device times of the step.  A re-unitarisation and a
+    measurement run alone between two events each (mean over `steps` steps);
+    the update phase is the rest of the timed step over its phases, launch
+    overlap and graph boundaries included.  An event pair around every phase
+    would keep consecutive launches from overlapping: that time is reported
+    beside it."""
+    lat.set_profiling(True)
+    lat.profile(reset=True)
+    for _ in range(steps):
+        lat.sweep(SWEEPS_PER_STEP)
+    prof = lat.profile(reset=True)
+    lat.set_profiling(False)
+    update, reunit, measure = (1e3 * prof[k + "_ms"] / max(1, prof[k + "_launches"])
+                               for k in ("update", "reunit", "measure"))
+    phases = 2 * len(DIMS) * SWEEPS_PER_STEP
+    return {"update_tick_us": (1e3 * step_ms - reunit - measure) / phases, "reunit_us": reunit, "measure_us": measure,
+            "event_timed_update_us": update}
 
 
 # ---------------------------------------------------------------- other workloads
@@ -595,19 +578,11 @@ def main():
     line["clocks"] = clocks
 
     if not args.no_extras:
-        # Roofline of the dominant kernel, the update tick.  Its duration comes
-        # from graph-timed runs (CUDA events on the launching stream, the
-        # launch overlap of the timed step included), so that 80 ticks + the
-        # re-unitarisation + the measurement add up to ms_per_step; the
-        # per-tick event timing (each tick wrapped in its own events, which
-        # loses the overlap of consecutive launches) is reported beside it.
+        # Roofline of the dominant kernel, the update tick.  Its duration is
+        # the timed step's, less the re-unitarisation and the measurement
+        # (stage_times).
         peaks, peak_src = measured_peaks()
-        st = graph_stage_times(su3, torch, stream, reps.seed(SEED), ms_max / args.steps)
-        lat.set_profiling(True)
-        lat.profile(reset=True)
-        lat.sweep(SWEEPS_PER_STEP)
-        prof = lat.profile(reset=True)
-        lat.set_profiling(False)
+        st = stage_times(lat, ms_max / args.steps)
         upd_ms = st["update_tick_us"] * 1e-3
         V = links // len(DIMS)
         alg_bytes = (V // 2) * (2 * len(DIMS) + 1) * 48
@@ -616,14 +591,12 @@ def main():
                             "frac": achieved / peaks["hbm_gbs"], "traffic": recorded_traffic("k_update_fp32"),
                             "peak_source": f"hbm_gbs of {peak_src}", "kernel": "k_update<StoreF32x12>",
                             "alg_bytes_per_launch": alg_bytes, "avg_launch_us": upd_ms * 1e3,
-                            "tick_source": "graph-timed: (T(20 sweeps, re-unitarised every 20) - T(10 sweeps, "
-                                           "every 10)) / 80 update ticks",
+                            "tick_source": "the timed step less one event-timed re-unitarisation and measurement, "
+                                           f"over {2 * len(DIMS) * SWEEPS_PER_STEP} update phases",
                             "reunit_us": st["reunit_us"], "measure_us": st["measure_us"],
-                            "stages_sum_ms": st["sum_ms"], "step_ms": st["step_ms"],
-                            "event_timed_us": {
-                                "update": 1e3 * prof["update_ms"] / max(1, prof["update_launches"]),
-                                "reunit": 1e3 * prof["reunit_ms"] / max(1, prof["reunit_launches"]),
-                                "measure": 1e3 * prof["measure_ms"] / max(1, prof["measure_launches"])}}
+                            "step_ms": ms_max / args.steps,
+                            "event_timed_us": {"update": st["event_timed_update_us"], "reunit": st["reunit_us"],
+                                               "measure": st["measure_us"]}}
 
         # End to end through the C ABI: every step uploads that step's input
         # configuration from pinned host memory (su3_stage_links_ex on the
