@@ -1628,6 +1628,9 @@ constexpr bool kIsEarly = V == kEarlyVariant || V == kEarlyRolled;
 constexpr int kParked0 = 15, kParked1 = 16;
 template <int V>
 constexpr bool kIsParked = V == kParked0 || V == kParked1;
+// FP64, fused launches with two-coupling chains among others.
+constexpr int kMixedVariant = 17;
+template <> struct TickBounds<kMixedVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };
 template <> struct TickBounds<kParked0> { static constexpr int kThreads = 256, kMinBlocks = 2; static constexpr bool kRolled = false; };
 template <> struct TickBounds<kParked1> { static constexpr int kThreads = kParkedThreads1, kMinBlocks = 5; static constexpr bool kRolled = false; };
 template <> struct TickBounds<kEarlyVariant> { static constexpr int kThreads = 256, kMinBlocks = 1; static constexpr bool kRolled = false; };
@@ -1729,14 +1732,19 @@ __device__ __forceinline__ void update_tile(const ChainDesc &d, uint32_t sweep, 
   } else {
     const int jj = p.jw + (int)(threadIdx.x & 31);
     const bool valid = jj < d.Vn;
-    double sum;
-    // the one-coupling FP64 update runs in fixed point
-    if constexpr (std::is_same<S, StoreF64x18>::value && !WT) {
-      ActionChange dr = {0, 0.0};
-      if (valid) update_site_fixed<SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
-      __syncwarp();
-      sum = warp_sum(dr);
-    } else {
+    double sum = 0.0;
+    // the one-coupling FP64 update runs in fixed point, also beside chains of
+    // two couplings: a chain's links do not depend on the others of its launch
+    constexpr bool kMixed = V == kMixedVariant;
+    constexpr bool kFixed = std::is_same<S, StoreF64x18>::value && (!WT || kMixed);
+    if (kFixed && !(kMixed && d.weighted)) {
+      if constexpr (kFixed) {
+        ActionChange dr = {0, 0.0};
+        if (valid) update_site_fixed<SUB>(d, sweep, colour, mu, layer, jj, np, na, dr);
+        __syncwarp();
+        sum = warp_sum(dr);
+      }
+    } else if constexpr (!kFixed || kMixed) {
       typename S::R dr = 0;  // in the kernel's precision
       if (valid) {
         if constexpr (kIsEarly<V> && TickBounds<V>::kRolled)

@@ -319,8 +319,9 @@ __global__ void __launch_bounds__(TickBounds<V>::kThreads, TickBounds<V>::kMinBl
 // ------------------------------------------------------------------ launchers
 
 // Tick kernel forms: FP32 12-real has variants 0..4 (TickBounds), FP32
-// 18-real variant 0 only, FP64 one form (10) and, as the launcher's variant 1
-// (not a choice of the caller), eight lanes per link.
+// 18-real variant 0 only, FP64 one form (10; kMixedVariant with two-coupling
+// chains) and, as the launcher's variant 1 (not a choice of the caller), eight
+// lanes per link.
 int tick_variants(int storage) { return storage == 1 ? 5 : 1; }
 
 template <class S, int V, bool WT, bool TOR>
@@ -358,7 +359,7 @@ static cudaError_t tick_dispatch(int storage, int variant, bool torus, A... a) {
   const bool tor = torus && !WT;
   if (storage == 0) {
     if (variant == 1 && !WT) return OP<StoreF64x18, kCoopVariant, false, false>::run(a...);
-    return OP<StoreF64x18, 10, WT, false>::run(a...);
+    return OP<StoreF64x18, WT ? kMixedVariant : 10, WT, false>::run(a...);
   }
   if (storage == 2) return tor ? OP<StoreF32x18, 0, false, kT>::run(a...) : OP<StoreF32x18, 0, WT, false>::run(a...);
   switch (variant) {
