@@ -9,10 +9,16 @@
 // and a product sum is accumulated exactly in two 64-bit integers,
 //   hh = sum h_a h_b          (units 2^-56)
 //   x  = sum h_a l_b + l_a h_b (units 2^-88),
-// three wide multiply-adds per real product.  The l_a l_b terms (at most 2^-58
-// each, their size in x's units is below one half per term) are dropped.  The
-// result is read as hh 2^32 + x, rounded to units 2^-60.  Every rounding is
-// thus 2^-57 or less, against 2^-54 to 2^-52 in the double-precision form.
+// three wide multiply-adds per real product.  The l_a l_b terms are dropped: at
+// most 2^-58 each and of either sign, 2^-59.6 root mean square (those of a
+// square have one sign: norm_fx adds them).  The result is read as hh 2^32 + x,
+// rounded to units 2^-60.  A sum of twelve products is thus within 2^-57.8 root
+// mean square (2^-54.4 at most), where each of the double-precision form's
+// operations rounds by 2^-54 to 2^-52.
+// What goes in and out: elements are read as floor(x 2^60), so that those below
+// 2^-7 lose the digits of their doubles beyond 2^-60; links are stored as the
+// nearest double; an update's change of Re Tr(U A) is rounded to 2^-51, the last
+// place of a double of its size, and a plaquette to 2^-56.
 //
 // Measured, one update phase: 24^4 (165888 links) 900 us in double, 218 us
 // here; 4^4 (128 links) 97 us in double, 32 us here, 11.4 us with eight lanes
